@@ -46,7 +46,17 @@
  * scf_set_mask, scf_evolve).  The
  * caller owns all particle, coefficient and centre buffers; the handle owns
  * its workspace (block partials, block maps, a coefficient buffer, the status
- * word), allocated once in scf_init.  No call allocates after scf_init.
+ * word), allocated once in scf_init.  No call allocates after scf_init
+ * (scf_step_host's first call excepted, see there).
+ *
+ * Radial bins.  A handle with enough particles for its (nmax, lmax) runs the
+ * coefficient and field passes of every entry point over particles sorted by
+ * radius, with the radial polynomials of each radius bin replaced by
+ * interpolants exact to the precision's rounding (workspace of about 40 bytes
+ * a particle and the bins' tables; without the memory for it the handle keeps
+ * the direct kernels).  The block shapes below are those of the direct
+ * kernels; selecting a float-float variant, or the one-thread-per-output
+ * kernel 1 in SCF_MIXED, selects the direct kernel.
  *
  * Errors.  Every entry point returns 0 (SCF_OK) or a negative SCF_ERR_* code;
  * scf_strerror gives a static description.  Device-side problems (non-finite
@@ -188,10 +198,13 @@ int scf_step(scf_handle* h, void* pos, void* vel, void* acc, double* com, int ns
  * write the host arrays in place over the host link: the transfers happen
  * inside the kernels, overlapped with their arithmetic, and the device arrays
  * are not used (they may be NULL); in SCF_MIXED with the register-tiled
- * kernel 1 the drifted positions and half-kicked velocities between kernels
- * 1 and 3 are kept in a device copy owned by the handle (2 x 16 bytes per
- * particle, allocated by the first such call, freed by scf_free), so the
- * host link carries the state in once and out once.  Otherwise the state is staged through the
+ * kernel 1, and over radial bins in either precision, the drifted positions
+ * and half-kicked velocities between kernels 1 and 3 are kept in a device copy
+ * owned by the handle (2 records per particle, allocated by the first such
+ * call, freed by scf_free), so the host link carries the state in once and out
+ * once; over radial bins kernel 3 leaves its results there and they go back by
+ * copies on a second stream of the handle, which its own stream waits for (in
+ * four pieces in SCF_MIXED).  Otherwise the state is staged through the
  * device arrays: copied in on a second stream of the handle, kernels 1 and 2,
  * then the positions and the centres copied back while kernel 3 runs, which
  * is launched in `chunks` pieces of its block map so that each piece's

@@ -12,6 +12,7 @@
 #include "../../include/scf.h"
 #include "scf_device.cuh"
 #include "scf_internal.h"
+#include "scf_bins.h"
 #include "scf_escape.h"
 
 struct scf_handle {
@@ -104,12 +105,65 @@ struct scf_handle {
   cudaStream_t side_stream = nullptr;                 // created at the greatest stream priority
   int side_priority = 0;
   cudaEvent_t side_ev[2] = {nullptr, nullptr};
+  // radial bins (scf_bins.h): the coefficient and field passes over particles
+  // sorted by radius, for handles that choose_bins admits
+  bool binned = false;                   // tables for the current exponent are in place
+  bool bins_off = false;                 // the direct kernels for now (the autotuner times them)
+  ScfBinShape bin{};
+  int bin_kcap = 0;                      // bins the allocation holds
+  int bin_blocks = 0, bin_mblocks = 0, bin_fblocks = 0;  // sorting, moment and field blocks
+  void* d_bin_base = nullptr;
+  int *d_sb_prog = nullptr, *d_sb_off = nullptr, *d_mb_prog = nullptr, *d_mb_task = nullptr, *d_fb_prog = nullptr,
+      *d_bin_rows_off = nullptr;
+  int64_t *d_sb_begin = nullptr, *d_sb_end = nullptr, *d_fb_begin = nullptr, *d_fb_end = nullptr,
+          *d_mrow_off = nullptr;
+  int* d_fb_task = nullptr;
+  unsigned *d_bin_code = nullptr, *d_bin_hist = nullptr, *d_bin_total = nullptr, *d_bin_ticket = nullptr,
+           *d_bin_start = nullptr, *d_task_start = nullptr, *d_field_start = nullptr;
+  double* d_binv = nullptr;
+  std::vector<int64_t> h_sb_begin;       // host copy: particle ranges of the sorting blocks
+  void *d_spos = nullptr, *d_mrows = nullptr, *d_bin_frame = nullptr, *d_field_rows = nullptr;
+  int2* d_skey = nullptr;
+  double *d_bin_t = nullptr, *d_bin_aux = nullptr;  // tables; nodes, node-to-monomial matrix and gscale
+  float* d_bin_tf = nullptr;
+  float2* d_bin_t2 = nullptr;
 };
 
 namespace {
 
 std::mutex g_const_mutex;
 std::vector<bool> g_const_ready;
+
+// Legendre constants of the radial-bin kernels (scf_bins.h).  gam is rational,
+// ((l-1)^2 - m^2) / (4 (l-1)^2 - 1), and rounded once: an error in it would leak
+// the monopole into every degree, systematically over the particles.
+void scf_make_bin_const(const ScfConst& t, ScfBinConst* b) {
+  using LD = long double;
+  std::vector<LD> sig(SCF_NLM_CAP);
+  LD diag = 1.0L / std::sqrt(4.0L * 3.14159265358979323846264338327950288L);
+  for (int m = 0; m <= SCF_LMAX_CAP; ++m) {
+    if (m > 0) diag *= -std::sqrt((2.0L * m + 1.0L) / (2.0L * m));
+    sig[scf_lm(m, m)] = diag;
+    for (int l = m + 1; l <= SCF_LMAX_CAP; ++l) {
+      const int i = scf_lm(l, m);
+      const LD l2 = (LD)l * l, k2 = (LD)(l - 1) * (l - 1), m2 = (LD)m * m;
+      sig[i] = std::sqrt((4.0L * l2 - 1.0L) / (l2 - m2)) * sig[scf_lm(l - 1, m)];
+      b->gam[i] = (double)((k2 - m2) / (4.0L * k2 - 1.0L));
+    }
+  }
+  for (int l = 0; l <= SCF_LMAX_CAP; ++l)
+    for (int m = 0; m <= l; ++m) {
+      const int i = scf_lm(l, m);
+      b->sig[i] = (double)sig[i];
+      b->kap[i] = m < l ? (double)(std::sqrt((LD)(l - m) * (l + m + 1)) * sig[scf_lm(l, m + 1)] / sig[i]) : 0.0;
+      b->gamf[i] = (float)b->gam[i];
+      b->gamlo[i] = (float)(b->gam[i] - (double)b->gamf[i]);
+      b->kapf[i] = (float)b->kap[i];
+      b->la[i] = m == l - 1 ? t.lsub[l] : t.la[i];
+      b->lb[i] = t.lb[i];
+      b->ldiag[l] = t.ldiag[l];
+    }
+}
 
 int upload_tables_once(int device) {
   std::lock_guard<std::mutex> lock(g_const_mutex);
@@ -123,6 +177,11 @@ int upload_tables_once(int device) {
   cudaError_t e3 = scf_upload_const_adjoint(t);
   cudaError_t e4 = scf_upload_const_forces_ff(t);
   cudaError_t e5 = scf_upload_const_coeffs_ff(t);
+  ScfBinConst b{};
+  scf_make_bin_const(*t, &b);
+  if (e5 == cudaSuccess) e5 = scf_upload_const_bins(&b);
+  if (e5 == cudaSuccess) e5 = scf_upload_const_bin_moments(&b);
+  if (e5 == cudaSuccess) e5 = scf_upload_const_bin_field(&b);
   delete t;
   if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess || e4 != cudaSuccess || e5 != cudaSuccess)
     return SCF_ERR_CUDA;
@@ -285,9 +344,109 @@ K3Args k3_args(scf_handle* h, const void* pos, void* vel, void* acc, const doubl
   return a;
 }
 
+// The radial-bin passes replace the default kernels: register-tiled kernel 1 in
+// mixed precision, the native kernels in double precision.
+bool bins_k1(const scf_handle* h) {
+  return h->binned && !h->bins_off && (h->cfg.precision == SCF_MIXED ? h->k1.variant == 1 : h->k1.variant != 2);
+}
+bool bins_k3(const scf_handle* h) { return h->binned && !h->bins_off && h->k3.variant != 2; }
+
+// Sorts the particles by bin (step mode: after the half kick and drift, which
+// leave the velocities in vel_out and a copy of the positions in pos_copy when given).
+int run_sort(scf_handle* h, void* pos, void* vel, const void* acc, const uint8_t* mask, int mode, void* pos_copy,
+             void* vel_out, bool status) {
+  BinArgs a{};
+  a.pos = pos;
+  a.vel = vel;
+  a.acc = acc;
+  a.pos_copy = pos_copy;
+  a.vel_out = vel_out;
+  a.mask = mask;
+  a.mode = mode;
+  a.dt = h->cfg.dt;
+  a.f32 = h->cfg.precision == SCF_MIXED;
+  a.dtf = (float)h->cfg.dt;
+  a.half_dtf = (float)(0.5 * h->cfg.dt);
+  a.inv_alphaf = (float)(1.0 / h->cfg.alpha);
+  a.b_prog = h->d_b;
+  a.status = h->d_status;
+  a.blk_prog = h->d_sb_prog;
+  a.blk_begin = h->d_sb_begin;
+  a.blk_end = h->d_sb_end;
+  a.prog_blk_off = h->d_sb_off;
+  a.prog_off = h->d_off;
+  a.n_blocks = h->bin_blocks;
+  a.n_prog = h->n_prog;
+  a.K = h->bin.K;
+  a.chunk = h->bin.chunk;
+  a.task = h->bin.task;
+  a.code = h->d_bin_code;
+  a.hist = h->d_bin_hist;
+  a.total = h->d_bin_total;
+  a.ticket = h->d_bin_ticket;
+  a.bin_start = h->d_bin_start;
+  a.task_start = h->d_task_start;
+  a.field_start = h->d_field_start;
+  a.binv = h->d_binv;
+  a.spos = h->d_spos;
+  a.skey = h->d_skey;
+  a.count_status = status ? 1 : 0;
+  return cuda_fail(scf_bin_sort_launch(a, h->stream));
+}
+
+// Kernel 1 over radial bins: sort, moments, partial coefficient rows.
+int run_binned_k1(scf_handle* h, void* pos, void* vel, const void* acc, const uint8_t* mask, int mode, void* pos_copy,
+                  void* vel_out) {
+  const int f32 = h->cfg.precision == SCF_MIXED;
+  int rc = run_sort(h, pos, vel, acc, mask, mode, pos_copy, vel_out, true);
+  if (rc != SCF_OK) return rc;
+  MomentArgs m{};
+  m.spos = h->d_spos;
+  m.bin_start = h->d_bin_start;
+  m.task_start = h->d_task_start;
+  m.prog_off = h->d_off;
+  m.blk_prog = h->d_mb_prog;
+  m.blk_task = h->d_mb_task;
+  m.row_off = h->d_mrow_off;
+  m.frame = h->d_bin_frame;
+  m.rows = h->d_mrows;
+  m.binv = h->d_binv;
+  m.alpha = h->cfg.alpha;
+  m.inv_alpha = 1.0 / h->cfg.alpha;
+  m.alphaf = (float)m.alpha;
+  m.inv_alphaf = (float)m.inv_alpha;
+  m.K = h->bin.K;
+  if (scf_moments_launch(f32, h->bin, m, h->bin_mblocks, h->stream) != cudaSuccess) return SCF_ERR_CUDA;
+  TransformArgs t{};
+  t.rows = h->d_mrows;
+  t.row_off = h->d_mrow_off;
+  t.task_start = h->d_task_start;
+  t.t = h->d_bin_t;
+  t.t2 = h->d_bin_t2;
+  t.partials = h->d_partials;
+  t.K = h->bin.K;
+  t.T = h->bin.T;
+  t.colpad = scf_bin_colpad(h->bin.L);
+  t.groups = h->bin.groups;
+  t.nmax = h->cfg.nmax;
+  t.lmax = h->cfg.lmax;
+  t.nlm = h->nlm;
+  t.nc = h->nc;
+  t.n_prog = h->n_prog;
+  t.f32 = f32;
+  return cuda_fail(scf_transform_launch(t, h->stream));
+}
+
 int run_coeffs(scf_handle* h, void* pos, void* vel, const void* acc, const uint8_t* mask, double* A_out, double* com,
                int mode, void* pos_copy = nullptr, void* vel_out = nullptr) {
-  if (h->k1_blocks > 0) {
+  const bool binned = bins_k1(h);
+  if (binned) {
+    if (timed(h, 0, [&] {
+          return run_binned_k1(h, pos, vel, acc, mask, mode, pos_copy, vel_out) == SCF_OK ? cudaSuccess
+                                                                                          : cudaErrorUnknown;
+        }) != cudaSuccess)
+      return SCF_ERR_CUDA;
+  } else if (h->k1_blocks > 0) {
     K1Args a = k1_args(h, pos, vel, acc, mask, mode);
     a.pos_copy = pos_copy;
     a.vel_out = vel_out;
@@ -298,6 +457,10 @@ int run_coeffs(scf_handle* h, void* pos, void* vel, const void* acc, const uint8
       return SCF_ERR_CUDA;
   }
   K2Args b = k2_args(h, A_out, com, mode);
+  if (binned) {  // double rows, one per bin group
+    b.prog_blk_off = h->d_bin_rows_off;
+    b.sub = 0;
+  }
   return cuda_fail(timed(h, 1, [&] { return scf_k2_launch(b, h->stream); }));
 }
 
@@ -320,10 +483,75 @@ int run_prep(scf_handle* h, const double* A, const double* com) {
   return cuda_fail(timed(h, 1, [&] { return scf_prep_launch(p, h->stream); }));
 }
 
-// Kernel 3 on the handle's F / a_host(R) (from kernel 2 or run_prep).
+// Kernel 3 over radial bins: field rows from F, then the sorted particles.
+int run_binned_k3(scf_handle* h, void* vel, void* acc, const double* com, int mode, const void* vel_in, int seg0 = 0,
+                  int seg1 = 0) {
+  const int f32 = h->cfg.precision == SCF_MIXED;
+  FieldRowArgs r{};
+  r.F = h->d_F;
+  r.t = f32 ? static_cast<const void*>(h->d_bin_tf) : static_cast<const void*>(h->d_bin_t);
+  r.total = h->d_bin_total;
+  r.P = h->d_field_rows;
+  r.K = h->bin.K;
+  r.T = h->bin.T;
+  r.L = h->bin.L;
+  r.nmax = h->cfg.nmax;
+  r.lmax = h->cfg.lmax;
+  r.nlm = h->nlm;
+  r.nc = h->nc;
+  r.n_prog = h->n_prog;
+  r.f32 = f32;
+  // (the rows serve every segment)
+  if (seg0 == 0 && scf_field_rows_launch(r, h->stream) != cudaSuccess) return SCF_ERR_CUDA;
+  BinFieldArgs a{};
+  a.spos = h->d_spos;
+  a.skey = h->d_skey;
+  a.vel = vel;
+  a.vel_in = vel_in;
+  a.acc = acc;
+  a.P = h->d_field_rows;
+  a.frame = h->d_bin_frame;
+  a.com = com;
+  a.aR = h->d_aR;
+  a.tid = h->d_tidf;
+  a.blk_prog = h->d_fb_prog;
+  a.blk_task = h->d_fb_task;
+  a.blk_begin = h->d_fb_begin;
+  a.blk_end = h->d_fb_end;
+  a.bin_start = h->d_bin_start;
+  a.field_start = h->d_field_start;
+  a.prog_off = h->d_off;
+  a.binv = h->d_binv;
+  a.K = h->bin.K;
+  a.mode = mode;
+  a.n_prog = h->n_prog;
+  a.seg0 = seg0;
+  a.seg1 = seg1;
+  a.prog_blk_off = h->d_sb_off;
+  a.hist = h->d_bin_hist;
+  a.total = h->d_bin_total;
+  a.dt = h->cfg.dt;
+  a.alpha = h->cfg.alpha;
+  a.inv_alpha = 1.0 / h->cfg.alpha;
+  a.host = h->host;
+  a.status = h->d_status;
+  return cuda_fail(scf_bin_field_launch(f32, h->bin, a, h->bin_fblocks, h->stream));
+}
+
+// Kernel 3 on the handle's F / a_host(R) (from kernel 2 or run_prep).  sorted:
+// run_coeffs has just run on the same positions (its sort serves this pass too).
 int run_forces(scf_handle* h, const void* pos, void* vel, void* acc, const double* com, int mode,
-               const void* vel_in = nullptr) {
+               const void* vel_in = nullptr, bool sorted = false) {
   if (h->k3_blocks == 0) return SCF_OK;
+  if (bins_k3(h) && mode != SCF_MODE_ADJ_J) {
+    return cuda_fail(timed(h, 2, [&] {
+      int rc = sorted && bins_k1(h) ? SCF_OK
+                                    : run_sort(h, const_cast<void*>(pos), nullptr, nullptr, nullptr, SCF_MODE_COEFFS,
+                                               nullptr, nullptr, false);
+      if (rc == SCF_OK) rc = run_binned_k3(h, vel, acc, com, mode, vel_in);
+      return rc == SCF_OK ? cudaSuccess : cudaErrorUnknown;
+    }));
+  }
   K3Args a = k3_args(h, pos, vel, acc, com, mode);
   a.vel_in = vel_in;
   if (h->k3.variant == 2 && mode != SCF_MODE_ADJ_J)
@@ -505,6 +733,189 @@ int use_k3(scf_handle* h, int tb) {
   return SCF_OK;
 }
 
+// Radial bins of a configuration: K and T so that the interpolated polynomials
+// of every degree and order are exact to the precision's rounding.  The fastest
+// oscillation of the family goes like nmax + lambda_lmax radians per radian of
+// theta; K is proportional to it.
+ScfBinShape bin_shape(const scf_config& c, double alpha, bool large) {
+  ScfBinShape s{};
+  const double w = c.nmax + (2.0 * c.lmax + 1.0) * alpha + 0.5;
+  if (c.precision == SCF_MIXED) {
+    s.T = large ? 6 : 8;
+    s.K = (int)std::ceil((large ? 12.4 : 3.1) * w);
+  } else {
+    s.T = large ? 8 : 10;
+    s.K = (int)std::ceil((large ? 40.0 : 11.5) * w);
+  }
+  s.K = (s.K + 31) / 32 * 32;
+  s.L = c.lmax <= 4 ? 4 : c.lmax <= 5 ? 5 : c.lmax <= 6 ? 6 : c.lmax <= 8 ? 8 : c.lmax <= 10 ? 10 : 12;
+  return s;
+}
+
+// Whether a handle's passes run over radial bins, and with which (K, T).  The
+// direct kernels cost N W, W = (nmax + 1)(lmax + 1)^2; the bins replace the
+// nmax + 1 terms by T, for a fixed sequence of passes and, per progenitor, the
+// K-sized tables.  Steps measured on a GB300, bins against direct (us):
+//   mixed  (20,10) 50k 58.5/57.6, 100k 69/86, 1e6 238/542;  (20,8) 50k 53/49, 100k 62/74;
+//          (10,5) 200k 60/56, 300k 67/72;  ten progenitors (20,10) 200k 144/134, 500k 201/282,
+//          (10,5) 200k 71/54, 1e6 146/178
+//   double (20,8) 4k 204/260, 100k 770/1600;  (20,10) 1e6 7500/20110;  (10,5) 10k 133/127,
+//          20k 148/177;  ten progenitors (20,10) 100k 1615/2255, (10,5) 40k 350/259
+// so the lines below; few radial orders (T >= nmax + 1) or degrees leave nothing
+// to save ((2,0) double, 100k: 305/111).  More, narrower bins with fewer terms
+// pay from about 400k (mixed) and 50k (double) particles a progenitor
+// ((20,8) double: 30k 337/318 us, 100k 770/842).
+bool choose_bins(const scf_handle* h, bool* large) {
+  const scf_config& c = h->cfg;
+  const bool f32 = c.precision == SCF_MIXED;
+  const int64_t n = h->n_total, per = n / h->n_prog;
+  const double W = (c.nmax + 1.0) * (c.lmax + 1.0) * (c.lmax + 1.0);
+  *large = per >= (f32 ? 400000 : 50000);
+  if (n >= (int64_t)1 << 31 || c.lmax < 3 || c.nmax < (f32 ? 8 : 6)) return false;
+  return f32 ? n >= 23000.0 * h->n_prog + 1.0e8 / W : n >= 2000.0 + 6800.0 * (h->n_prog - 1) + 4.5e6 / W;
+}
+
+// Tables of the handle's exponent; false (direct kernels) when they do not fit
+// the allocation or a value is not finite.
+bool bin_tables(scf_handle* h) {
+  bool large = false;
+  h->binned = false;
+  if (!h->d_bin_base || !choose_bins(h, &large)) return false;
+  const scf_config& c = h->cfg;
+  ScfBinShape s = bin_shape(c, c.alpha, large);
+  if (s.K > h->bin_kcap) return false;
+  s.chunk = h->bin.chunk;
+  s.groups = h->bin.groups;
+  s.task = h->bin.task;
+  h->bin = s;
+  std::unique_ptr<ScfConst> t(new (std::nothrow) ScfConst);
+  if (!t) return false;
+  scf_make_const(t.get(), c.alpha);
+  const int nd = s.T - 1, nn = c.nmax + 1;
+  std::vector<double> aux(2 * (size_t)nd + 2 * (size_t)nd * nd + (size_t)(c.lmax + 1) * nn);
+  scf_bin_nodes(s.T, aux.data(), aux.data() + 2 * nd);
+  double* gs = aux.data() + 2 * nd + 2 * nd * nd;
+  for (int l = 0; l <= c.lmax; ++l)
+    for (int n = 0; n < nn; ++n) gs[l * nn + n] = t->gscale[l][n];
+  if (!put(h->d_bin_aux, aux.data(), sizeof(double) * aux.size())) return false;
+  BinTableArgs a{};
+  a.K = s.K;
+  a.T = s.T;
+  a.nmax = c.nmax;
+  a.lmax = c.lmax;
+  a.f32 = c.precision == SCF_MIXED;
+  a.alpha = c.alpha;
+  a.nodes = h->d_bin_aux;
+  a.vinv = h->d_bin_aux + 2 * nd;
+  a.gscale = h->d_bin_aux + 2 * nd + 2 * nd * nd;
+  a.frame = h->d_bin_frame;
+  a.t = h->d_bin_t;
+  a.tf = h->d_bin_tf;
+  a.t2 = h->d_bin_t2;
+  if (scf_bin_table_launch(a, h->stream) != cudaSuccess) return false;
+  h->binned = true;
+  drop_graph(h);
+  return true;
+}
+
+// Workspace and maps of the radial bins; without them (no memory) the handle
+// keeps the direct kernels.
+int bin_init(scf_handle* h) {
+  bool large = false;
+  if (h->n_total == 0 || !choose_bins(h, &large)) return SCF_OK;
+  const scf_config& c = h->cfg;
+  const int f32 = c.precision == SCF_MIXED;
+  const size_t es = f32 ? 4 : 8, n = (size_t)h->n_total, np = h->n_prog;
+  // room for the exponents that scf_retune_alpha may move to
+  ScfBinShape s = bin_shape(c, std::max(c.alpha, 2.0), large);
+  h->bin_kcap = s.K;
+  s.chunk = h->n_total < 400 * (int64_t)h->n_sm ? 512 : h->n_total < 1600 * (int64_t)h->n_sm ? 1024 : 2048;
+  s.task = h->n_total < 300000 ? (f32 ? 256 : 128) : (f32 ? 512 : 256);
+  s.groups = std::max(1, std::min(s.K, h->n_sm / h->n_prog));
+  const Map3 sm = make_map3(h->offsets, h->n_prog, s.chunk);
+  Map3 fm = make_map3(h->offsets, h->n_prog, kBinField64Threads);  // double precision
+  std::vector<int> fb_task;                                         // single precision
+  if (f32) fm = Map3{};
+  std::vector<int> sb_off(np + 1, 0), mb_prog, mb_task, rows_off(np + 1);
+  for (int p : sm.prog) ++sb_off[p + 1];
+  for (size_t p = 0; p < np; ++p) sb_off[p + 1] += sb_off[p];
+  std::vector<int64_t> mrow(np);
+  int64_t rows = 0;
+  for (size_t p = 0; p < np; ++p) {
+    const int64_t np_ = h->offsets[p + 1] - h->offsets[p];
+    const int64_t tasks = np_ / s.task + std::min<int64_t>(np_, s.K);
+    mrow[p] = rows;
+    rows += tasks;
+    for (int64_t t = 0; t < tasks; ++t) {
+      mb_prog.push_back((int)p);
+      mb_task.push_back((int)t);
+    }
+    if (f32)
+      for (int64_t t = 0; t < np_ / kBinFieldTask + std::min<int64_t>(np_, s.K); ++t) {
+        fm.prog.push_back((int)p);
+        fb_task.push_back((int)t);
+      }
+    rows_off[p + 1] = (int)((p + 1) * s.groups);
+  }
+  h->cap_rows = std::max(h->cap_rows, np * (size_t)s.groups);
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    const size_t o = off;
+    off += round_up(bytes);
+    return o;
+  };
+  const size_t K = s.K, nn = c.nmax + 1, nl = c.lmax + 1, nsb = sm.prog.size(), nfb = fm.prog.size();
+  const size_t o_sbp = take(4 * nsb), o_sbb = take(8 * nsb), o_sbe = take(8 * nsb), o_sbo = take(4 * (np + 1));
+  const size_t o_fbp = take(4 * nfb), o_fbb = take(8 * nfb), o_fbe = take(8 * nfb);
+  const size_t o_mbp = take(4 * mb_prog.size()), o_mbt = take(4 * mb_prog.size()), o_mro = take(8 * np);
+  const size_t o_fbt = take(4 * nfb), o_tk = take(4 * np), o_fs = take(4 * np * (K + 1)), o_bi = take(8 * np);
+  const size_t o_ro = take(4 * (np + 1)), o_id = take(4 * n), o_hist = take(4 * nsb * K), o_tot = take(4 * np * K);
+  const size_t o_bs = take(4 * np * (K + 1)), o_ts = take(4 * np * (K + 1));
+  const size_t o_sp = take(32 * n), o_key = f32 ? off : take(8 * n);
+  const size_t o_rows = take(es * (size_t)rows * s.T * scf_bin_colpad(s.L));
+  const size_t o_fr = take(2 * es * K), o_P = take(es * np * K * scf_bin_row(s.L, s.T));
+  const size_t o_t = f32 ? off : take(8 * K * nl * nn * s.T), o_tf = f32 ? take(4 * K * nl * nn * s.T) : off,
+               o_t2 = f32 ? take(8 * K * nl * nn * s.T) : off;
+  const size_t o_aux = take(8 * (2 * (size_t)s.T * (s.T + 1) + nl * nn));
+  if (cudaMalloc(&h->d_bin_base, off) != cudaSuccess) {
+    cudaGetLastError();
+    h->d_bin_base = nullptr;
+    return SCF_OK;
+  }
+  char* base = static_cast<char*>(h->d_bin_base);
+  auto at = [&](auto*& p, size_t o) { p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(base + o); };
+  at(h->d_sb_prog, o_sbp), at(h->d_sb_begin, o_sbb), at(h->d_sb_end, o_sbe), at(h->d_sb_off, o_sbo);
+  at(h->d_fb_prog, o_fbp), at(h->d_fb_begin, o_fbb), at(h->d_fb_end, o_fbe);
+  at(h->d_mb_prog, o_mbp), at(h->d_mb_task, o_mbt), at(h->d_mrow_off, o_mro), at(h->d_bin_rows_off, o_ro);
+  at(h->d_bin_code, o_id), at(h->d_bin_hist, o_hist), at(h->d_bin_total, o_tot);
+  at(h->d_bin_start, o_bs), at(h->d_task_start, o_ts), at(h->d_skey, o_key);
+  at(h->d_fb_task, o_fbt), at(h->d_bin_ticket, o_tk), at(h->d_field_start, o_fs), at(h->d_binv, o_bi);
+  h->d_spos = base + o_sp;
+  h->d_mrows = base + o_rows;
+  h->d_bin_frame = base + o_fr;
+  h->d_field_rows = base + o_P;
+  at(h->d_bin_t, o_t), at(h->d_bin_tf, o_tf), at(h->d_bin_t2, o_t2), at(h->d_bin_aux, o_aux);
+  h->bin = s;
+  h->bin_blocks = (int)nsb;
+  h->bin_mblocks = (int)mb_prog.size();
+  h->bin_fblocks = (int)nfb;
+  h->h_sb_begin = sm.begin;
+  const bool ok = put(h->d_sb_prog, sm.prog.data(), 4 * nsb) && put(h->d_sb_begin, sm.begin.data(), 8 * nsb) &&
+                  put(h->d_sb_end, sm.end.data(), 8 * nsb) && put(h->d_sb_off, sb_off.data(), 4 * (np + 1)) &&
+                  put(h->d_fb_prog, fm.prog.data(), 4 * nfb) && put(h->d_mb_prog, mb_prog.data(), 4 * mb_prog.size()) &&
+                  (f32 ? put(h->d_fb_task, fb_task.data(), 4 * nfb)
+                       : put(h->d_fb_begin, fm.begin.data(), 8 * nfb) && put(h->d_fb_end, fm.end.data(), 8 * nfb)) &&
+                  put(h->d_mb_task, mb_task.data(), 4 * mb_task.size()) && put(h->d_mrow_off, mrow.data(), 8 * np) &&
+                  put(h->d_bin_rows_off, rows_off.data(), 4 * (np + 1));
+  // a progenitor without particles has no sorting block to write its (empty) bins
+  return ok && cudaMemset(h->d_bin_start, 0, 4 * np * (K + 1)) == cudaSuccess &&
+                 cudaMemset(h->d_task_start, 0, 4 * np * (K + 1)) == cudaSuccess &&
+                 cudaMemset(h->d_field_start, 0, 4 * np * (K + 1)) == cudaSuccess &&
+                 cudaMemset(h->d_bin_ticket, 0, 4 * np) == cudaSuccess
+             ? SCF_OK
+             : SCF_ERR_CUDA;
+}
+
 }  // namespace
 
 extern "C" {
@@ -540,6 +951,7 @@ int scf_init(const scf_config* cfg, int n_prog, const int64_t* offsets, const do
   }
   auto fail = [&](int code) {
     if (h->d_base) cudaFree(h->d_base);
+    if (h->d_bin_base) cudaFree(h->d_bin_base);
     delete h;
     return code;
   };
@@ -574,7 +986,9 @@ int scf_init(const scf_config* cfg, int n_prog, const int64_t* offsets, const do
   h->cap_blk3 = make_map3(h->offsets, n_prog, 32).prog.size();  // smallest kernel 3 tile (64 threads, split)
   if (h->cap_blk1 == 0 && h->n_total > 0) return fail(SCF_ERR_UNSUPPORTED);
 
-  // one allocation for the whole workspace
+  // the radial bins' own allocation, then one for the rest of the workspace
+  rc = bin_init(h);
+  if (rc != SCF_OK) return fail(rc);
   const size_t nb1 = std::max<size_t>(1, h->cap_blk1), nb3 = std::max<size_t>(1, h->cap_blk3);
   const size_t nrows = std::max<size_t>(1, h->cap_rows);
   size_t off = 0;
@@ -693,6 +1107,7 @@ int scf_init(const scf_config* cfg, int n_prog, const int64_t* offsets, const do
   if (rc != SCF_OK) return fail(rc);
   rc = use_k3(h, 128);
   if (rc != SCF_OK) return fail(rc);
+  bin_tables(h);
   *out = h;
   return SCF_OK;
 }
@@ -714,13 +1129,29 @@ int scf_forces(scf_handle* h, const void* pos, const double* A, const double* co
 
 namespace {
 
+constexpr int kHostSegments = 4;  // pieces in which a host-memory state goes back
+
+// The handle's copy stream and its events, made by the first call that needs them.
+bool make_copy_stream(scf_handle* h) {
+  if (h->copy_stream) return true;
+  if (cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking) != cudaSuccess) {
+    h->copy_stream = nullptr;
+    return false;
+  }
+  h->stage_ev.assign(SCF_STAGE_MAX_CHUNKS + 4, nullptr);  // start, in, done, kernels 1-2, one per chunk
+  for (cudaEvent_t& e : h->stage_ev)
+    if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return false;
+  return true;
+}
+
 // One step.  split (scf_step_host on mapped host memory): kernel 1 also
 // writes the drifted positions to the device copy and the half-kicked
 // velocities only there, and kernel 3 reads both from it, so the host link
 // carries the state in once and out once.
 int launch_step(scf_handle* h, void* pos, void* vel, void* acc, double* com, bool split = false) {
   void* spos = split ? h->d_split : nullptr;
-  void* svel = split ? static_cast<char*>(h->d_split) + 16 * (size_t)h->n_total : nullptr;
+  void* svel = split ? static_cast<char*>(h->d_split) + (h->cfg.precision == SCF_MIXED ? 16 : 32) * (size_t)h->n_total
+                     : nullptr;
   int rc = run_coeffs(h, pos, vel, acc, h->step_mask, h->d_A, com, SCF_MODE_STEP, spos, svel);
   if (rc != SCF_OK) return rc;
   // the next step's centre kick-drift-kick, on a second stream beside kernel 3
@@ -753,7 +1184,39 @@ int launch_step(scf_handle* h, void* pos, void* vel, void* acc, double* com, boo
         cudaEventRecord(h->side_ev[1], h->side_stream) != cudaSuccess)
       return SCF_ERR_CUDA;
   }
-  rc = split ? run_forces(h, spos, vel, acc, com, SCF_MODE_STEP, svel) : run_forces(h, pos, vel, acc, com, SCF_MODE_STEP);
+  if (split && bins_k3(h)) {
+    // the sorted pass writes in radial order: onto the device copies (the
+    // positions' one is free again once they are sorted), which go back by the
+    // copy stream, segment by segment of the caller's order in single precision
+    const size_t rec = h->cfg.precision == SCF_MIXED ? 16 : 32;
+    const int segs = h->cfg.precision == SCF_MIXED && h->bin_blocks >= kHostSegments ? kHostSegments : 1;
+    if (!make_copy_stream(h)) return SCF_ERR_CUDA;
+    for (int c = 0; c < segs && rc == SCF_OK; ++c) {
+      const int b0 = (int)((int64_t)h->bin_blocks * c / segs), b1 = (int)((int64_t)h->bin_blocks * (c + 1) / segs);
+      rc = segs == 1 ? run_forces(h, spos, svel, spos, com, SCF_MODE_STEP, svel, true)
+                     : cuda_fail(timed(h, 2, [&] {
+                         return run_binned_k3(h, svel, spos, com, SCF_MODE_STEP, svel, b0, b1) == SCF_OK
+                                    ? cudaSuccess
+                                    : cudaErrorUnknown;
+                       }));
+      const size_t k0 = rec * (size_t)h->h_sb_begin[b0],
+                   k1 = rec * (size_t)(b1 < h->bin_blocks ? h->h_sb_begin[b1] : h->n_total);
+      auto ok = [](cudaError_t e) { return e == cudaSuccess; };
+      if (rc == SCF_OK &&
+          !(ok(cudaEventRecord(h->stage_ev[c], h->stream)) && ok(cudaStreamWaitEvent(h->copy_stream, h->stage_ev[c], 0)) &&
+            ok(cudaMemcpyAsync(static_cast<char*>(acc) + k0, static_cast<char*>(spos) + k0, k1 - k0, cudaMemcpyDefault,
+                               h->copy_stream)) &&
+            ok(cudaMemcpyAsync(static_cast<char*>(vel) + k0, static_cast<char*>(svel) + k0, k1 - k0, cudaMemcpyDefault,
+                               h->copy_stream))))
+        rc = SCF_ERR_CUDA;
+    }
+    if (rc == SCF_OK && (cudaEventRecord(h->stage_ev[kHostSegments], h->copy_stream) != cudaSuccess ||
+                         cudaStreamWaitEvent(h->stream, h->stage_ev[kHostSegments], 0) != cudaSuccess))
+      rc = SCF_ERR_CUDA;
+  } else {
+    rc = split ? run_forces(h, spos, vel, acc, com, SCF_MODE_STEP, svel)
+               : run_forces(h, pos, vel, acc, com, SCF_MODE_STEP, nullptr, true);
+  }
   if (ahead && cudaStreamWaitEvent(h->stream, h->side_ev[1], 0) != cudaSuccess) return SCF_ERR_CUDA;
   return rc;
 }
@@ -857,10 +1320,13 @@ int scf_step_host(scf_handle* h, void* pos, void* vel, void* acc, double* com, v
   if (mapped && aligned16(mp[0]) && aligned16(mp[1]) && aligned16(mp[2])) {
     // mixed precision with the register-tiled kernel 1 and the native kernel
     // 3: the intermediate state stays on the device (launch_step, split)
-    const bool split = h->cfg.precision == SCF_MIXED && h->k1.variant == 1 && h->k3.variant != 2 &&
+    // (both precisions over radial bins, whose passes read and write in radial order)
+    const bool split = ((h->cfg.precision == SCF_MIXED && h->k1.variant == 1 && h->k3.variant != 2) ||
+                        (bins_k1(h) && bins_k3(h))) &&
                        h->n_total > 0;
     if (split && !h->d_split) {
-      if (cudaMalloc(&h->d_split, 2 * 16 * (size_t)h->n_total) != cudaSuccess) {
+      const size_t rec = h->cfg.precision == SCF_MIXED ? 16 : 32;
+      if (cudaMalloc(&h->d_split, 2 * rec * (size_t)h->n_total) != cudaSuccess) {
         cudaGetLastError();
         h->d_split = nullptr;
         return SCF_ERR_OUT_OF_MEMORY;
@@ -877,15 +1343,7 @@ int scf_step_host(scf_handle* h, void* pos, void* vel, void* acc, double* com, v
   if ((!pos || !vel || !acc) && h->n_total > 0) return SCF_ERR_NULL_POINTER;
   if (with_com && !com) return SCF_ERR_NULL_POINTER;
   if (!aligned16(pos) || !aligned16(vel) || !aligned16(acc)) return SCF_ERR_MISALIGNED;
-  if (!h->copy_stream) {
-    if (cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking) != cudaSuccess) {
-      h->copy_stream = nullptr;
-      return SCF_ERR_CUDA;
-    }
-    h->stage_ev.assign(SCF_STAGE_MAX_CHUNKS + 4, nullptr);  // start, in, done, kernels 1-2, one per chunk
-    for (cudaEvent_t& e : h->stage_ev)
-      if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return SCF_ERR_CUDA;
-  }
+  if (!make_copy_stream(h)) return SCF_ERR_CUDA;
   cudaStream_t cs = h->copy_stream;
   cudaEvent_t ev_start = h->stage_ev[0], ev_in = h->stage_ev[1], ev_done = h->stage_ev[2];
   cudaEvent_t* ev_out = &h->stage_ev[3];
@@ -906,7 +1364,9 @@ int scf_step_host(scf_handle* h, void* pos, void* vel, void* acc, double* com, v
   if (!ok(cudaEventRecord(ev_out[0], h->stream)) || !ok(cudaStreamWaitEvent(cs, ev_out[0], 0))) return SCF_ERR_CUDA;
   if (bytes && !ok(cudaMemcpyAsync(hh[0], dp[0], bytes, cudaMemcpyDeviceToHost, cs))) return SCF_ERR_CUDA;
   if (with_com && !ok(cudaMemcpyAsync(host_com, com, com_bytes, cudaMemcpyDeviceToHost, cs))) return SCF_ERR_CUDA;
-  const int c3 = std::max(1, std::min(chunks, h->k3_blocks));
+  // (over radial bins in one piece: a chunk of sorted particles is no range of the arrays)
+  const bool binned = bins_k3(h);
+  const int c3 = binned ? 1 : std::max(1, std::min(chunks, h->k3_blocks));
   for (int c = 0; c < c3 && h->k3_blocks > 0; ++c) {
     int b0, b1;
     block_range(h->k3_blocks, c3, c, &b0, &b1);
@@ -915,11 +1375,15 @@ int scf_step_host(scf_handle* h, void* pos, void* vel, void* acc, double* com, v
     a.blk_prog += b0;
     a.blk_begin += b0;
     a.blk_end += b0;
-    const cudaError_t e = timed(h, 2, [&] {
-      return h->k3.variant == 2 ? scf_k3_ff_launch(a, b1 - b0, h->k3, h->stream)
-                                : scf_k3_launch(h->cfg.precision, a, b1 - b0, h->k3_native, h->stream);
-    });
-    if (e != cudaSuccess) return SCF_ERR_CUDA;
+    if (binned) {
+      rc = run_forces(h, pos, vel, acc, com, SCF_MODE_STEP, nullptr, true);
+      if (rc != SCF_OK) return rc;
+    } else if (timed(h, 2, [&] {
+                 return h->k3.variant == 2 ? scf_k3_ff_launch(a, b1 - b0, h->k3, h->stream)
+                                           : scf_k3_launch(h->cfg.precision, a, b1 - b0, h->k3_native, h->stream);
+               }) != cudaSuccess) {
+      return SCF_ERR_CUDA;
+    }
     if (!ok(cudaEventRecord(ev_out[1 + c], h->stream)) || !ok(cudaStreamWaitEvent(cs, ev_out[1 + c], 0)))
       return SCF_ERR_CUDA;
     const size_t k0 = (size_t)h->h_blk3_begin[b0], k1 = (size_t)h->h_blk3_end[b1 - 1];
@@ -996,8 +1460,13 @@ int scf_autotune(scf_handle* h, const void* pos, const double* com, void* acc, i
   if (h->n_total == 0) return SCF_OK;
   const bool prof = h->prof_on;
   h->prof_on = false;
+  h->bins_off = true;  // the shapes timed here are those of the direct kernels
   cudaEvent_t e0 = nullptr, e1 = nullptr;
-  if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return SCF_ERR_CUDA;
+  if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
+    h->bins_off = false;
+    h->prof_on = prof;
+    return SCF_ERR_CUDA;
+  }
   int rc = SCF_OK;
   auto time_it = [&](auto&& work, double* ms) -> int {
     for (int w = 0; w < 2; ++w)
@@ -1050,6 +1519,7 @@ int scf_autotune(scf_handle* h, const void* pos, const double* com, void* acc, i
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   h->prof_on = prof;
+  h->bins_off = false;
   return rc;
 }
 
@@ -1265,7 +1735,7 @@ int scf_evolve(scf_handle* h, void* pos, void* vel, void* acc, double* com, int 
     // the field of the new set at the current positions (the next opening kick uses it)
     rc = run_coeffs(h, pos, nullptr, nullptr, mask, h->d_A, nullptr, SCF_MODE_COEFFS);
     if (rc == SCF_OK) rc = run_prep(h, h->d_A, com);
-    if (rc == SCF_OK) rc = run_forces(h, pos, nullptr, acc, com, SCF_MODE_COEFFS);
+    if (rc == SCF_OK) rc = run_forces(h, pos, nullptr, acc, com, SCF_MODE_COEFFS, nullptr, true);
     if (rc != SCF_OK) return rc;
     // leapfrog steps up to the next integration timestep (the shortest over progenitors)
     int k = ep->max_steps;
@@ -1324,7 +1794,7 @@ int scf_recentre(scf_handle* h, void* pos, void* vel, void* acc, double* com, co
                                    h->stream)) != SCF_OK)
     return SCF_ERR_CUDA;
   rc = run_prep(h, h->d_Atmp, nullptr);
-  if (rc == SCF_OK) rc = run_forces(h, pos, nullptr, acc, nullptr, SCF_MODE_COEFFS);
+  if (rc == SCF_OK) rc = run_forces(h, pos, nullptr, acc, nullptr, SCF_MODE_COEFFS, nullptr, true);
   if (rc != SCF_OK) return rc;
   // 3. core radius and velocity, the frame moved to (x_c, V_core)
   if (cuda_fail(scf_core_launch(a, h->stream)) != SCF_OK) return SCF_ERR_CUDA;
@@ -1431,6 +1901,7 @@ int set_alpha(scf_handle* h, double alpha) {
   int rc = h->cfg.precision == SCF_MIXED ? use_k1(h, 0) : SCF_ERR_UNSUPPORTED;
   if (rc != SCF_OK) rc = use_k1(h, 128);
   if (rc == SCF_OK) rc = use_k3(h, 128);
+  if (rc == SCF_OK) bin_tables(h);
   drop_graph(h);
   return rc;
 }
@@ -1585,10 +2056,12 @@ int scf_status(scf_handle* h, int* status) {
 
 int scf_launches_per_call(const scf_handle* h, int which) {
   if (!h) return SCF_ERR_NULL_POINTER;
-  const int k1 = h->k1_blocks > 0 ? 1 : 0, k3 = h->k3_blocks > 0 ? 1 : 0;
+  // over radial bins: three sorting passes, moments, transform; field rows, field
+  const int k1 = bins_k1(h) ? 5 : h->k1_blocks > 0 ? 1 : 0, k3 = bins_k3(h) ? 2 : h->k3_blocks > 0 ? 1 : 0;
+  const int sort = bins_k3(h) ? 3 : 0;
   if (which == 0) return k1 + 1;
-  if (which == 1) return 1 + k3;
-  if (which == 2) return k1 + 1 + k3;
+  if (which == 1) return 1 + sort + k3;
+  if (which == 2) return k1 + 1 + (bins_k1(h) ? 0 : sort) + k3;
   return SCF_ERR_INVALID_ARG;
 }
 
@@ -1646,6 +2119,7 @@ int scf_free(scf_handle* h) {
     if (e) cudaEventDestroy(e);
   if (h->side_stream) cudaStreamDestroy(h->side_stream);
   if (h->d_base && cudaFree(h->d_base) != cudaSuccess) rc = SCF_ERR_CUDA;
+  if (h->d_bin_base && cudaFree(h->d_bin_base) != cudaSuccess) rc = SCF_ERR_CUDA;
   if (h->d_split && cudaFree(h->d_split) != cudaSuccess) rc = SCF_ERR_CUDA;
   delete h;
   return rc;

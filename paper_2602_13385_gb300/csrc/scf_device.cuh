@@ -73,6 +73,25 @@ struct ScfHostParams {
   double GM[SCF_HOST_CAP], a[SCF_HOST_CAP], b[SCF_HOST_CAP];
 };
 
+// The same in single precision, for the single-precision tidal difference: a
+// conversion from double runs on the FP64 pipe (2 lanes per clock and SM), so
+// a kernel converts once per block (scf_host_f32, thread i component i), not in
+// every thread.
+struct ScfHostParamsF {
+  int n;
+  int kind[SCF_HOST_CAP];
+  float GM[SCF_HOST_CAP], a[SCF_HOST_CAP], b[SCF_HOST_CAP];
+};
+__device__ __forceinline__ void scf_host_f32(const ScfHostParams& hp, int i, ScfHostParamsF* f) {
+  if (i == 0) f->n = hp.n;
+  if (i < hp.n) {
+    f->kind[i] = hp.kind[i];
+    f->GM[i] = (float)hp.GM[i];
+    f->a[i] = (float)hp.a[i];
+    f->b[i] = (float)hp.b[i];
+  }
+}
+
 // Forward-mode dual number (value, derivative) in double precision: the
 // adjoint kernels evaluate the same formulas on duals to get exact
 // directional derivatives (Hessian-vector products) of the expansion and of
@@ -317,7 +336,7 @@ __device__ __forceinline__ void scf_tidal_prep_f32(const ScfHostParams& hp, int 
   }
 }
 
-__device__ __forceinline__ void scf_tidal_f32(const ScfHostParams& hp, const float (*tr)[SCF_TIDAL_W], float Rx,
+__device__ __forceinline__ void scf_tidal_f32(const ScfHostParamsF& hp, const float (*tr)[SCF_TIDAL_W], float Rx,
                                               float Ry, float Rz, float x, float y, float z, float& ax, float& ay,
                                               float& az) {
   ax = 0.f;
@@ -330,7 +349,7 @@ __device__ __forceinline__ void scf_tidal_f32(const ScfHostParams& hp, const flo
   const float dr = (2.f * (Rx * x + Ry * y + Rz * z) + xx) * scf_rcpf(r1 + r0);
   float lastB = __int_as_float(0x7fffffff), zb1 = 0.f, izb1 = 0.f, dzb = 0.f;  // NaN: the first disk computes them
   for (int i = 0; i < hp.n; ++i) {
-    const float GM = (float)hp.GM[i], A = (float)hp.a[i];
+    const float GM = hp.GM[i], A = hp.a[i];
     const float* t = tr[i];
     if (hp.kind[i] == 1) {  // Hernquist
       const float p1 = r1 * (r1 + A) * (r1 + A);
@@ -355,7 +374,7 @@ __device__ __forceinline__ void scf_tidal_f32(const ScfHostParams& hp, const flo
       ay -= g1 * y + dg * Ry;
       az -= g1 * z + dg * Rz;
     } else if (hp.kind[i] == 3) {  // Miyamoto-Nagai
-      const float B = (float)hp.b[i];
+      const float B = hp.b[i];
       const float zb0 = t[0], zab0 = t[1], D2_0 = t[2], D0 = t[3];
       if (B != lastB) {
         zb1 = sqrtf(Pz * Pz + B * B);
@@ -376,7 +395,7 @@ __device__ __forceinline__ void scf_tidal_f32(const ScfHostParams& hp, const flo
       const float dv = -A * dzb * izb1 * t[6];
       az -= GM * (z * v1 * i1 + Rz * (dv * i1 + t[5] * di));
     } else if (hp.kind[i] == 4) {  // cut-off power-law bulge
-      const float s = 0.5f * (3.f - (float)hp.b[i]);
+      const float s = 0.5f * (3.f - hp.b[i]);
       const float X0 = t[0], P0 = t[1], ia2 = t[3];
       const float X1 = r1 * r1 * ia2;
       const float dX = dr * (r1 + r0) * ia2;

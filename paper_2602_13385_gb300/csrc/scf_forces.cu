@@ -114,9 +114,17 @@ __device__ __forceinline__ void k3_body(const K3Args& a) {
   // single precision: the values of the tidal differences that depend on R
   // alone, formed by kernel 2 (or the force-coefficient set-up) for this R
   __shared__ float s_tid[kF2 ? SCF_HOST_CAP : 1][SCF_TIDAL_W];
+  // and everything else that would be a conversion from double in every thread
+  // (the FP64 pipe runs 1/64 of the FP32 one): the host, R, 1/b and dt/2
+  __shared__ ScfHostParamsF s_host;
+  __shared__ float s_f[5];
   if constexpr (kF2) {
     if (has_host && tid < a.host.n * SCF_TIDAL_W)
       (&s_tid[0][0])[tid] = a.tid[(size_t)prog * SCF_HOST_CAP * SCF_TIDAL_W + tid];
+    if (tid < SCF_HOST_CAP) scf_host_f32(a.host, tid, &s_host);
+    if (tid < 3) s_f[tid] = has_host ? (float)a.com[6 * prog + tid] : 0.f;
+    if (tid == 3) s_f[3] = (float)(1.0 / b);
+    if (tid == 4) s_f[4] = (float)(0.5 * a.dt);
   }
   __syncthreads();
 
@@ -155,7 +163,9 @@ __device__ __forceinline__ void k3_body(const K3Args& a) {
   if (!finite && half == 0) atomicOr(a.status, 1u);
   const T x = finite ? p.x : (T)0, y = finite ? p.y : (T)0, z = finite ? p.z : (T)0;
 
-  const T binv = (T)(1.0 / b);
+  T binv;
+  if constexpr (kF2) binv = s_f[3];
+  else binv = (T)(1.0 / b);
   const T r = sqrt(x * x + y * y + z * z);
   const T rinv = r > (T)0 ? (T)1 / r : (T)0;
   const T u = x * rinv, v = y * rinv, c = z * rinv;
@@ -357,7 +367,7 @@ __device__ __forceinline__ void k3_body(const K3Args& a) {
     if (has_host) {
       // the same difference in single precision without cancellation
       float tx, ty, tz;
-      scf_tidal_f32(a.host, s_tid, (float)s_R[0], (float)s_R[1], (float)s_R[2], p.x, p.y, p.z, tx, ty, tz);
+      scf_tidal_f32(s_host, s_tid, s_f[0], s_f[1], s_f[2], p.x, p.y, p.z, tx, ty, tz);
       gx += tx;
       gy += ty;
       gz += tz;
@@ -393,7 +403,9 @@ __device__ __forceinline__ void k3_body(const K3Args& a) {
   if (a.mode == SCF_MODE_STEP) {
     V4* vel4 = reinterpret_cast<V4*>(a.vel);
     V4 vv = a.vel_in ? reinterpret_cast<const V4*>(a.vel_in)[k] : vel4[k];
-    const T h = (T)(0.5 * a.dt);
+    T h;
+    if constexpr (kF2) h = s_f[4];
+    else h = (T)(0.5 * a.dt);
     vv.x += h * out.x;
     vv.y += h * out.y;
     vv.z += h * out.z;
