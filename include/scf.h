@@ -359,7 +359,9 @@ int scf_energy(scf_handle* h, const void* pos, const void* vel, const void* acc,
  * (each coordinate and mass split into two floats, 48 bits; a term's
  * relative error is about 1e-14 + 2^-48 |x| / r_ij) and blocks of 64 of them
  * are added in double.  In mixed precision each pair term and blocks of 64
- * of them are float (1/r the hardware approximation), added in double.  In
+ * of them (128, in sums of four, for the second particle of a pair) are float
+ * (1/r the hardware approximation), added in double.  Each unordered pair is
+ * evaluated once for both of its particles.  In
  * both, pairs whose r^2 lies outside the normal float range
  * [1.18e-38, 3.40e38] add nothing.
  *   pos, vel   device [N][4] in the handle's element type (16-byte aligned)
@@ -369,8 +371,8 @@ int scf_energy(scf_handle* h, const void* pos, const void* vel, const void* acc,
  *   mask_out   device [N] bytes, 1 = r <= r_x, or NULL
  *   stats_out  device [n_prog][4] doubles: n_bound, bound mass, r_x, size of the set
  * All sums have a fixed order (bitwise reproducible).  Cost O(sum_p N_p^2).
- * The workspace for it (8 (S+1) N bytes, S <= 16 pair-sum segments) is
- * reserved by scf_init.
+ * The workspace for it (8 (S+1) N bytes, S = 64 partial sums a particle, fewer
+ * where they would take more than 2 GiB) is reserved by scf_init.
  * Errors: SCF_ERR_NULL_POINTER, SCF_ERR_MISALIGNED, SCF_ERR_INVALID_ARG, SCF_ERR_CUDA. */
 int scf_bound(scf_handle* h, const void* pos, const void* vel, double kin, double frac, double* E_out,
               uint8_t* bound_out, uint8_t* mask_out, double* stats_out);

@@ -78,12 +78,12 @@ struct scf_handle {
   double* d_en_part = nullptr;        // [k3 blocks][4] energy partials
   // escape physics: particle offsets, pair-sum segments, radius keys, tidal scales
   int64_t* d_off = nullptr;              // [n_prog+1]
-  double* d_bpart = nullptr;             // [bound_split][n_total]
+  double* d_bpart = nullptr;             // [bound_slots][n_total]
   unsigned long long* d_key = nullptr;   // [n_total]
   double* d_tid = nullptr;               // [n_prog][16]
   double* d_half = nullptr;              // [n_prog][4] selection at frac 1/2 (complete refresh)
-  int bound_split = 1;
-  int64_t bound_chunks = 0;              // pair-kernel i-blocks of the largest progenitor
+  int bound_slots = 1;
+  int64_t bound_chunks = 0, bound_chunks_all = 0;  // pair-kernel chunks of the largest progenitor, of all
   const uint8_t* step_mask = nullptr;    // coefficient set of scf_step (scf_set_mask)
   double* d_Atmp = nullptr;              // [n_prog][2*NC] scratch coefficients
   ScfLaunchInfo k1d{}, k3d{};
@@ -1022,10 +1022,11 @@ int scf_init(const scf_config* cfg, int n_prog, const int64_t* offsets, const do
       chunks += c;
       h->bound_chunks = std::max(h->bound_chunks, c);
     }
-    h->bound_split = scf_bound_split(chunks, h->n_sm);
+    h->bound_chunks_all = chunks;
+    h->bound_slots = scf_bound_slots(h->n_total);
   }
   const size_t o_off = take(sizeof(int64_t) * (n_prog + 1));
-  const size_t o_bpart = take(sizeof(double) * (size_t)h->bound_split * (size_t)h->n_total);
+  const size_t o_bpart = take(sizeof(double) * (size_t)h->bound_slots * (size_t)h->n_total);
   const size_t o_key = take(sizeof(unsigned long long) * (size_t)h->n_total);
   const size_t o_tid = take(sizeof(double) * 16 * (size_t)n_prog);
   const size_t o_half = take(sizeof(double) * 4 * (size_t)n_prog);
@@ -1630,7 +1631,8 @@ int scf_bound(scf_handle* h, const void* pos, const void* vel, double kin, doubl
   a.n_prog = h->n_prog;
   a.n_total = h->n_total;
   a.f32 = h->cfg.precision == SCF_MIXED;
-  a.split = h->bound_split;
+  a.slots = h->bound_slots;
+  a.total_chunks = h->bound_chunks_all;
   a.G = h->cfg.G;
   a.kin = kin;
   a.frac = frac;
@@ -1640,7 +1642,7 @@ int scf_bound(scf_handle* h, const void* pos, const void* vel, double kin, doubl
   a.bound = bound_out;
   a.mask = mask_out;
   a.stats = stats_out;
-  return cuda_fail(scf_bound_launch(a, h->bound_chunks, h->stream));
+  return cuda_fail(scf_bound_launch(a, h->bound_chunks, h->n_sm, h->stream));
 }
 
 namespace {

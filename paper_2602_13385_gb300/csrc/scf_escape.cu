@@ -11,16 +11,14 @@
 //   integration timestep dt_int = sqrt(eta) (|T|_F^2 / 6)^(-1/4).
 //
 // Kernels:
-//   k_bound_pairs  O(N^2) pair sums.  Grid (i-chunk, progenitor, j-segment):
-//                  each block stages its j-segment through shared memory in
-//                  tiles and keeps four (float) or two (double) i-particles
-//                  per thread in registers.  Single precision sums blocks of
-//                  64 pair terms in float and adds them in double; double
-//                  precision evaluates the pair terms in float-float
-//                  arithmetic (k_bound_pairs_ff) and adds blocks of 64 of
-//                  them in double.  Each block writes one double per
-//                  particle and segment.
-//   k_bound_finish one thread per particle: adds the segments in order, forms
+//   k_bound_pairs  O(N^2) pair sums, every unordered pair once: chunk A of a
+//                  progenitor's particles against chunk B = A + r (round r),
+//                  one 1/r for both particles.  The i-particles (A) sit in
+//                  registers; the j-particles (B) are dealt one pair a lane and
+//                  their sums travel around the warp with them.  Double precision
+//                  evaluates the pair terms in float-float arithmetic
+//                  (k_bound_pairs_ff).
+//   k_bound_finish one thread per particle: adds the slots in order, forms
 //                  E_i and the bound flag, and the radius key (bits of r^2).
 //   k_select       one block per progenitor: bound count and mass, radix
 //                  selection of the k-th smallest key (8 passes of 8 bits over
@@ -29,6 +27,7 @@
 // Every sum has a fixed order, so results are bitwise reproducible.
 #include <cmath>
 #include <cstdint>
+#include <cooperative_groups.h>
 #include <math_constants.h>
 
 #include "scf_device.cuh"
@@ -38,92 +37,176 @@
 namespace {
 
 constexpr int kPairThreads = 128;
-constexpr int kPairSub = 64;      // pair terms summed in the element type before the double add
+constexpr int kPairWarps = kPairThreads / 32;
 constexpr int kSelectThreads = 1024;
+constexpr int kSelectBlocks = 8;  // cluster of the selection
 
 template <typename V4>
 struct Elem;
 template <>
 struct Elem<float4> {
-  using T = float;
   static constexpr int I = 4;     // i-particles per thread
 };
 template <>
 struct Elem<ScfD4> {
-  using T = double;
   static constexpr int I = 2;
 };
-
-// 1/sqrt(r2) of a single-precision pair by the hardware approximation
-// (rsqrt.approx.ftz.f32, a few ulp); 0 for a pair that adds nothing: r2 zero,
-// below the smallest normal float (which the approximation flushes to zero)
-// or not finite.
-__device__ __forceinline__ float pair_inv_r(float r2) {
-  float y;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(r2));
-  return r2 >= 1.17549435e-38f ? y : 0.f;  // r2 = inf gives y = 0
-}
 template <typename V4>
-__global__ void __launch_bounds__(kPairThreads) k_bound_pairs(BoundArgs a) {
-  using T = typename Elem<V4>::T;
-  constexpr int kPairI = Elem<V4>::I;
-  __shared__ V4 s_j[kPairThreads];
-  const V4* pos = reinterpret_cast<const V4*>(a.pos);
-  for (int p = blockIdx.y; p < a.n_prog; p += gridDim.y) {
-    const int64_t o0 = a.prog_off[p], o1 = a.prog_off[p + 1];
-    const int64_t ib = o0 + (int64_t)blockIdx.x * (kPairThreads * kPairI);
-    if (ib >= o1) continue;  // the same for every thread of the block
-    const int64_t seg = (o1 - o0 + a.split - 1) / a.split;
-    const int64_t j0 = min(o1, o0 + (int64_t)blockIdx.z * seg), j1 = min(o1, j0 + seg);
-    T xi[kPairI], yi[kPairI], zi[kPairI];
-    double acc[kPairI];
+constexpr int kPairChunk = kPairThreads * Elem<V4>::I;  // particles of a chunk
+
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float2 dup(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 neg(float2 x) { return make_float2(-x.x, -x.y); }
+__device__ __forceinline__ float2 rotate(float2 x, int lane) {  // from the next lane
+  return make_float2(__shfl_sync(0xffffffffu, x.x, (lane + 1) & 31), __shfl_sync(0xffffffffu, x.y, (lane + 1) & 31));
+}
+__device__ __forceinline__ bool finite2(float2 x) { return isfinite(x.x) && isfinite(x.y); }
+
+// 1/sqrt(r2) of single-precision pairs by the hardware approximation
+// (rsqrt.approx.ftz.f32, a few ulp).  A pair that adds nothing (r2 zero, below
+// the smallest normal float, which the approximation flushes to zero, or NaN)
+// gives an infinity or NaN: SAFE replaces it by 0, the fast form leaves it to
+// show in the sums, which are then formed again by SAFE.  r2 = inf gives 0.
+template <bool SAFE>
+__device__ __forceinline__ float2 pair_inv_r(float2 r2) {
+  float2 y = make_float2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
+  if (SAFE) {
+    y.x = r2.x >= 1.17549435e-38f ? y.x : 0.f;
+    y.y = r2.y >= 1.17549435e-38f ? y.y : 0.f;
+  }
+  return y;
+}
+
+// Single precision.  A lane's i-particles, each coordinate in both halves of a
+// packed operand (negated: separations are sums).
+struct PairI {
+  float2 x[4], y[4], z[4], m[4];
+};
+
+// One rotation: the warp's 128 i-particles against 64 j-particles, two a lane at a
+// time (xy, zm: (x, x', y, y') and (z, z', m, m') of 32 pairs).  part[q] += m_j / r
+// over the lane's 32 steps, sj = the j sums sum m_i / r, back at their home lane.
+// Bound by the FP32 pipe: 12 additions, 12 products and 9 accumulations, packed,
+// for eight unordered pairs (the special-function unit a third busy).
+template <bool SAFE>
+__device__ __forceinline__ void rotation(const PairI& pi, const float4* xy, const float4* zm, int lane, float2* part,
+                                         float2& sj) {
+  sj = dup(0.f);
+#pragma unroll 4
+  for (int s = 0; s < 32; ++s) {
+    const int k = (lane + s) & 31;
+    const float4 a = xy[k], b = zm[k];
+    const float2 xj = make_float2(a.x, a.y), yj = make_float2(a.z, a.w), zj = make_float2(b.x, b.y),
+                 mj = make_float2(b.z, b.w);
+    float2 t = dup(0.f);
 #pragma unroll
-    for (int q = 0; q < kPairI; ++q) {
-      const int64_t i = ib + threadIdx.x + q * kPairThreads;
-      const V4 pi = i < o1 ? pos[i] : V4{};
-      xi[q] = pi.x;
-      yi[q] = pi.y;
-      zi[q] = pi.z;
+    for (int q = 0; q < 4; ++q) {
+      const float2 dx = __fadd2_rn(xj, pi.x[q]), dy = __fadd2_rn(yj, pi.y[q]), dz = __fadd2_rn(zj, pi.z[q]);
+      const float2 ri = pair_inv_r<SAFE>(__ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx))));
+      part[q] = __ffma2_rn(mj, ri, part[q]);
+      t = q == 0 ? __fmul2_rn(pi.m[q], ri) : __ffma2_rn(pi.m[q], ri, t);
+    }
+    sj = rotate(__fadd2_rn(sj, t), lane);
+  }
+}
+
+// Pair sums over the rounds [r0, r0 + gridDim.z R): block (A, progenitor, g) takes
+// the R rounds from r0 + g R.  Round r pairs chunk A with chunk B = A + r (mod P),
+// r = 1 .. P/2 (r = P/2 of an even P for A < P/2 only); round 0 is the chunk with
+// itself, every ordered pair, done by block g = 0 of the first launch.  A slot of
+// part has one writer per element and launch: slot g the i sums of group g, slot
+// gridDim.z + g R + k the j sums of its k-th round; launches follow one another,
+// so every sum has a fixed order.
+__global__ void __launch_bounds__(kPairThreads) k_bound_pairs(BoundArgs a) {
+  constexpr int C = kPairChunk<float4>, I = 4;
+  __shared__ float4 s_xy[C / 2], s_zm[C / 2];
+  __shared__ float s_sum[kPairWarps][C];
+  const float4* pos = reinterpret_cast<const float4*>(a.pos);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, A = blockIdx.x;
+  for (int p = blockIdx.y; p < a.n_prog; p += gridDim.y) {
+    const int64_t o0 = a.prog_off[p], n = a.prog_off[p + 1] - o0;
+    const int P = (int)((n + C - 1) / C);
+    if (A >= P) continue;  // the same for every thread of the block
+    PairI pi;
+    double acc[I];
+#pragma unroll
+    for (int q = 0; q < I; ++q) {
+      const int64_t i = (int64_t)A * C + warp * (32 * I) + q * 32 + lane;
+      // a particle past the end: far from everything, no mass
+      const float4 x = i < n ? pos[o0 + i] : make_float4(1e18f, 0.f, 0.f, 0.f);
+      pi.x[q] = dup(-x.x);
+      pi.y[q] = dup(-x.y);
+      pi.z[q] = dup(-x.z);
+      pi.m[q] = dup(x.w);
       acc[q] = 0.0;
     }
-    for (int64_t jb = j0; jb < j1; jb += kPairThreads) {
-      const int cnt = (int)min((int64_t)kPairThreads, j1 - jb);
+    const int rb = a.round0 + blockIdx.z * a.rounds;
+    for (int rr = rb == 1 && a.round0 == 1 ? -1 : 0; rr < a.rounds; ++rr) {
+      const bool self = rr < 0;  // the first launch's block g = 0 starts with round 0
+      const int r = self ? 0 : rb + rr;
+      if (r > P / 2 || (2 * r == P && A >= r)) break;
+      const int B = A + r < P ? A + r : A + r - P;
       __syncthreads();
-      if ((int)threadIdx.x < cnt) s_j[threadIdx.x] = pos[jb + threadIdx.x];
+      for (int k = tid; k < C / 2; k += kPairThreads) {
+        const int64_t j = (int64_t)B * C + 2 * k;
+        const float4 far = make_float4(-1e18f, 0.f, 0.f, 0.f);
+        const float4 u = j < n ? pos[o0 + j] : far, v = j + 1 < n ? pos[o0 + j + 1] : far;
+        s_xy[k] = make_float4(u.x, v.x, u.y, v.y);
+        s_zm[k] = make_float4(u.z, v.z, u.w, v.w);
+      }
       __syncthreads();
-      for (int s = 0; s < cnt; s += kPairSub) {
-        const int e = min(cnt, s + kPairSub);
-        T part[kPairI];
+      float2 part[I];
+      for (int c = 0; c < C / 64; ++c) {
+        // blocks of 64 terms (two rotations of 32, two lanes) before the double add
+        float2 was[I], sj;
 #pragma unroll
-        for (int q = 0; q < kPairI; ++q) part[q] = T(0);
-#pragma unroll 4
-        for (int jj = s; jj < e; ++jj) {
-          const V4 pj = s_j[jj];
-#pragma unroll
-          for (int q = 0; q < kPairI; ++q) {
-            const T dx = pj.x - xi[q], dy = pj.y - yi[q], dz = pj.z - zi[q];
-            const T r2 = dx * dx + dy * dy + dz * dz;
-            // the self pair (and any coincident pair, and non-finite r2) adds nothing
-            const T ri = pair_inv_r(r2);
-            part[q] += pj.w * ri;
-          }
+        for (int q = 0; q < I; ++q) {
+          if (c % 2 == 0) part[q] = dup(0.f);
+          was[q] = part[q];
         }
+        bool ok = !self;
+        if (!self) {
+          rotation<false>(pi, s_xy + 32 * c, s_zm + 32 * c, lane, part, sj);
+          ok = finite2(sj) && finite2(part[0]) && finite2(part[1]) && finite2(part[2]) && finite2(part[3]);
+        }
+        if (__any_sync(0xffffffffu, !ok)) {
 #pragma unroll
-        for (int q = 0; q < kPairI; ++q) acc[q] += (double)part[q];
+          for (int q = 0; q < I; ++q) part[q] = was[q];
+          rotation<true>(pi, s_xy + 32 * c, s_zm + 32 * c, lane, part, sj);
+        }
+        if (c % 2 == 1)
+#pragma unroll
+          for (int q = 0; q < I; ++q) acc[q] += (double)part[q].x + (double)part[q].y;
+        *reinterpret_cast<float2*>(&s_sum[warp][64 * c + 2 * lane]) = sj;
+      }
+      __syncthreads();
+      if (!self) {
+        double* out = a.part + (size_t)(gridDim.z + blockIdx.z * a.rounds + rr) * (size_t)a.n_total + o0 + (int64_t)B * C;
+        for (int k = tid; k < C && (int64_t)B * C + k < n; k += kPairThreads) {
+          double v = 0.0;
+#pragma unroll
+          for (int w = 0; w < kPairWarps; ++w) v += (double)s_sum[w][k];
+          out[k] += v;
+        }
       }
     }
 #pragma unroll
-    for (int q = 0; q < kPairI; ++q) {
-      const int64_t i = ib + threadIdx.x + q * kPairThreads;
-      if (i < o1) a.part[(size_t)blockIdx.z * (size_t)a.n_total + (size_t)i] = acc[q];
+    for (int q = 0; q < I; ++q) {
+      const int64_t i = (int64_t)A * C + warp * (32 * I) + q * 32 + lane;
+      if (i < n) a.part[(size_t)blockIdx.z * (size_t)a.n_total + (size_t)(o0 + i)] += acc[q];
     }
+    __syncthreads();
   }
 }
 
 // Double-precision pair sums in float-float arithmetic ("double-single"):
 // GB300 retires 64 single-precision FMAs for each double one, and a pair term
 // carried as unevaluated sums of two floats (Dekker 1971; Knuth's TwoSum and
-// the FMA-based exact product) costs about 80 single-precision operations
+// the FMA-based exact product) costs tens of single-precision operations
 // against 11 double ones, so it runs several times faster at a relative error
 // near 1e-13.  Positions and masses are split once into hi + lo floats when
 // they are staged (48 of a double's 53 bits: a pair term's relative error
@@ -132,112 +215,168 @@ __global__ void __launch_bounds__(kPairThreads) k_bound_pairs(BoundArgs a) {
 // parts plus the difference of the lo parts; r^2 keeps each square's
 // rounding error; 1/r is
 // the hardware estimate refined by one Newton step whose residual 1 - r^2 y^2
-// is formed in float-float; m / r is added to a float-float sum, folded into
-// a double every 64 pairs.
-struct FF {
-  float h, l;
+// is formed in float-float; m / r is added to float-float sums, folded into
+// doubles after every rotation.  Two j-particles at a time in packed operations
+// (the _rn intrinsics are never contracted, which would break the transformations).
+struct FF2 {
+  float2 h, l;
 };
-
-// The error-free transformations are written with the _rn intrinsics, which
-// the compiler never contracts into FMAs (a contraction would break them).
-__device__ __forceinline__ FF two_sum(float a, float b) {
-  const float s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+__device__ __forceinline__ FF2 two_sum2(float2 a, float2 b) {
+  const float2 s = __fadd2_rn(a, b);
+  const float2 bb = __fadd2_rn(s, neg(a));
+  return {s, __fadd2_rn(__fadd2_rn(a, neg(__fadd2_rn(s, neg(bb)))), __fadd2_rn(b, neg(bb)))};
+}
+// s += (h, l)
+__device__ __forceinline__ void add_ff(FF2& s, float2 h, float2 l) {
+  const FF2 t = two_sum2(s.h, h);
+  s.h = t.h;
+  s.l = __fadd2_rn(s.l, __fadd2_rn(t.l, l));
+}
+// m / r as a pair: m (hi, lo) times y (hi, lo)
+__device__ __forceinline__ FF2 mul_ff(float2 mh, float2 ml, float2 yh, float2 yl) {
+  const float2 p = __fmul2_rn(mh, yh);
+  return {p, __ffma2_rn(mh, yl, __ffma2_rn(ml, yh, __ffma2_rn(mh, yh, neg(p))))};
 }
 
-__device__ __forceinline__ FF split_double(double x) {
+struct SplitF {
+  float h, l;
+};
+__device__ __forceinline__ SplitF split_double(double x) {
   const float h = __double2float_rn(x);
   return {h, __double2float_rn(x - (double)h)};
 }
 
-__device__ __forceinline__ float rsqrt_approx(float x) {
-  float y;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
+// A lane's i-particles: hi and lo parts, coordinates negated.
+struct PairIFF {
+  float2 xh[2], xl[2], yh[2], yl[2], zh[2], zl[2], mh[2], ml[2];
+};
+
+// 64 i-particles of a warp (two a lane) against 64 j-particles, as rotation().
+template <bool SAFE>
+__device__ __forceinline__ void rotation_ff(const PairIFF& pi, const float4* hxy, const float4* hzm, const float4* lxy,
+                                            const float4* lzm, int lane, FF2* part, FF2& sj) {
+#pragma unroll
+  for (int q = 0; q < 2; ++q) part[q] = {dup(0.f), dup(0.f)};
+  sj = {dup(0.f), dup(0.f)};
+  const float2 half = dup(0.5f), one = dup(1.f);
+#pragma unroll 1
+  for (int s = 0; s < 32; ++s) {
+    const int k = (lane + s) & 31;
+    const float4 ha = hxy[k], hb = hzm[k], la = lxy[k], lb = lzm[k];
+    const float2 mjh = make_float2(hb.z, hb.w), mjl = make_float2(lb.z, lb.w);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      // separation: exact difference of the hi parts + difference of the lo parts
+      const FF2 dx = two_sum2(make_float2(ha.x, ha.y), pi.xh[q]), dy = two_sum2(make_float2(ha.z, ha.w), pi.yh[q]),
+                dz = two_sum2(make_float2(hb.x, hb.y), pi.zh[q]);
+      const float2 lx = __fadd2_rn(dx.l, __fadd2_rn(make_float2(la.x, la.y), pi.xl[q]));
+      const float2 ly = __fadd2_rn(dy.l, __fadd2_rn(make_float2(la.z, la.w), pi.yl[q]));
+      const float2 lz = __fadd2_rn(dz.l, __fadd2_rn(make_float2(lb.x, lb.y), pi.zl[q]));
+      // r^2 = sum (h + l)^2 = sum h^2 + (2h + l) l, with the exact rounding
+      // error of each h^2, renormalised (all of r^2 may sit in the l parts)
+      const float2 px = __fmul2_rn(dx.h, dx.h), py = __fmul2_rn(dy.h, dy.h), pz = __fmul2_rn(dz.h, dz.h);
+      const float2 cx = __ffma2_rn(__fadd2_rn(__fadd2_rn(dx.h, dx.h), lx), lx, __ffma2_rn(dx.h, dx.h, neg(px)));
+      const float2 cy = __ffma2_rn(__fadd2_rn(__fadd2_rn(dy.h, dy.h), ly), ly, __ffma2_rn(dy.h, dy.h, neg(py)));
+      const float2 cz = __ffma2_rn(__fadd2_rn(__fadd2_rn(dz.h, dz.h), lz), lz, __ffma2_rn(dz.h, dz.h, neg(pz)));
+      const FF2 s1 = two_sum2(px, py);
+      const FF2 s2 = two_sum2(s1.h, pz);
+      const FF2 r2 = two_sum2(s2.h, __fadd2_rn(__fadd2_rn(s1.l, s2.l), __fadd2_rn(__fadd2_rn(cx, cy), cz)));
+      // 1/r: one Newton step y0 (1 + d/2), d = 1 - r^2 y0^2 in float-float
+      const float2 y0 = make_float2(rsqrt_approx(r2.h.x), rsqrt_approx(r2.h.y));
+      const float2 t = __fmul2_rn(y0, y0), te = __ffma2_rn(y0, y0, neg(t));
+      const float2 u = __fmul2_rn(r2.h, t);
+      const float2 ue = __ffma2_rn(r2.l, t, __ffma2_rn(r2.h, te, __ffma2_rn(r2.h, t, neg(u))));
+      const float2 d = __fadd2_rn(__fadd2_rn(one, neg(u)), neg(ue));
+      const float2 corr = __fmul2_rn(__fmul2_rn(half, y0), d);
+      float2 yh = __fadd2_rn(y0, corr), yl = __fadd2_rn(corr, neg(__fadd2_rn(yh, neg(y0))));
+      if (SAFE) {  // pairs outside the normal range add nothing
+        const bool ok0 = r2.h.x >= 1.17549435e-38f && r2.h.x <= 3.40282347e38f;
+        const bool ok1 = r2.h.y >= 1.17549435e-38f && r2.h.y <= 3.40282347e38f;
+        yh = make_float2(ok0 ? yh.x : 0.f, ok1 ? yh.y : 0.f);
+        yl = make_float2(ok0 ? yl.x : 0.f, ok1 ? yl.y : 0.f);
+      }
+      const FF2 wi = mul_ff(mjh, mjl, yh, yl), wj = mul_ff(pi.mh[q], pi.ml[q], yh, yl);
+      add_ff(part[q], wi.h, wi.l);
+      add_ff(sj, wj.h, wj.l);
+    }
+    sj.h = rotate(sj.h, lane);
+    sj.l = rotate(sj.l, lane);
+  }
 }
 
 __global__ void __launch_bounds__(kPairThreads) k_bound_pairs_ff(BoundArgs a) {
-  constexpr int kPairI = Elem<ScfD4>::I;
-  __shared__ float4 s_hi[kPairThreads], s_lo[kPairThreads];
+  constexpr int C = kPairChunk<ScfD4>, I = 2;
+  __shared__ float4 s_hxy[C / 2], s_hzm[C / 2], s_lxy[C / 2], s_lzm[C / 2];
+  __shared__ double s_sum[kPairWarps][C];
   const ScfD4* pos = reinterpret_cast<const ScfD4*>(a.pos);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, A = blockIdx.x;
   for (int p = blockIdx.y; p < a.n_prog; p += gridDim.y) {
-    const int64_t o0 = a.prog_off[p], o1 = a.prog_off[p + 1];
-    const int64_t ib = o0 + (int64_t)blockIdx.x * (kPairThreads * kPairI);
-    if (ib >= o1) continue;  // the same for every thread of the block
-    const int64_t seg = (o1 - o0 + a.split - 1) / a.split;
-    const int64_t j0 = min(o1, o0 + (int64_t)blockIdx.z * seg), j1 = min(o1, j0 + seg);
-    FF xi[kPairI], yi[kPairI], zi[kPairI];
-    double acc[kPairI];
+    const int64_t o0 = a.prog_off[p], n = a.prog_off[p + 1] - o0;
+    const int P = (int)((n + C - 1) / C);
+    if (A >= P) continue;  // the same for every thread of the block
+    PairIFF pi;
+    double acc[I];
 #pragma unroll
-    for (int q = 0; q < kPairI; ++q) {
-      const int64_t i = ib + threadIdx.x + q * kPairThreads;
-      const ScfD4 pi = i < o1 ? pos[i] : ScfD4{};
-      xi[q] = split_double(pi.x);
-      yi[q] = split_double(pi.y);
-      zi[q] = split_double(pi.z);
+    for (int q = 0; q < I; ++q) {
+      const int64_t i = (int64_t)A * C + warp * (32 * I) + q * 32 + lane;
+      const ScfD4 v = i < n ? pos[o0 + i] : ScfD4{1e18, 0.0, 0.0, 0.0};
+      const SplitF x = split_double(-v.x), y = split_double(-v.y), z = split_double(-v.z), m = split_double(v.w);
+      pi.xh[q] = dup(x.h), pi.xl[q] = dup(x.l);
+      pi.yh[q] = dup(y.h), pi.yl[q] = dup(y.l);
+      pi.zh[q] = dup(z.h), pi.zl[q] = dup(z.l);
+      pi.mh[q] = dup(m.h), pi.ml[q] = dup(m.l);
       acc[q] = 0.0;
     }
-    for (int64_t jb = j0; jb < j1; jb += kPairThreads) {
-      const int cnt = (int)min((int64_t)kPairThreads, j1 - jb);
+    const int rb = a.round0 + blockIdx.z * a.rounds;
+    for (int rr = rb == 1 && a.round0 == 1 ? -1 : 0; rr < a.rounds; ++rr) {
+      const bool self = rr < 0;
+      const int r = self ? 0 : rb + rr;
+      if (r > P / 2 || (2 * r == P && A >= r)) break;
+      const int B = A + r < P ? A + r : A + r - P;
       __syncthreads();
-      if ((int)threadIdx.x < cnt) {
-        const ScfD4 pj = pos[jb + threadIdx.x];
-        const FF x = split_double(pj.x), y = split_double(pj.y), z = split_double(pj.z), m = split_double(pj.w);
-        s_hi[threadIdx.x] = make_float4(x.h, y.h, z.h, m.h);
-        s_lo[threadIdx.x] = make_float4(x.l, y.l, z.l, m.l);
+      for (int k = tid; k < C; k += kPairThreads) {
+        const int64_t j = (int64_t)B * C + k;
+        const ScfD4 v = j < n ? pos[o0 + j] : ScfD4{-1e18, 0.0, 0.0, 0.0};
+        const SplitF x = split_double(v.x), y = split_double(v.y), z = split_double(v.z), m = split_double(v.w);
+        float *hxy = reinterpret_cast<float*>(&s_hxy[k / 2]) + (k & 1), *hzm = reinterpret_cast<float*>(&s_hzm[k / 2]) + (k & 1),
+              *lxy = reinterpret_cast<float*>(&s_lxy[k / 2]) + (k & 1), *lzm = reinterpret_cast<float*>(&s_lzm[k / 2]) + (k & 1);
+        hxy[0] = x.h, hxy[2] = y.h, hzm[0] = z.h, hzm[2] = m.h;
+        lxy[0] = x.l, lxy[2] = y.l, lzm[0] = z.l, lzm[2] = m.l;
       }
       __syncthreads();
-      for (int s = 0; s < cnt; s += kPairSub) {
-        const int e = min(cnt, s + kPairSub);
-        FF sum[kPairI];
-#pragma unroll
-        for (int q = 0; q < kPairI; ++q) sum[q] = {0.f, 0.f};
-#pragma unroll 2
-        for (int jj = s; jj < e; ++jj) {
-          const float4 hj = s_hi[jj], lj = s_lo[jj];
-#pragma unroll
-          for (int q = 0; q < kPairI; ++q) {
-            // separation: exact difference of the hi parts + difference of the lo parts
-            const FF dx = two_sum(hj.x, -xi[q].h), dy = two_sum(hj.y, -yi[q].h), dz = two_sum(hj.z, -zi[q].h);
-            const float lx = __fadd_rn(dx.l, __fsub_rn(lj.x, xi[q].l));
-            const float ly = __fadd_rn(dy.l, __fsub_rn(lj.y, yi[q].l));
-            const float lz = __fadd_rn(dz.l, __fsub_rn(lj.z, zi[q].l));
-            // r^2 = sum (h + l)^2 = sum h^2 + (2h + l) l, with the exact rounding
-            // error of each h^2, renormalised (all of r^2 may sit in the l parts)
-            const float px = __fmul_rn(dx.h, dx.h), py = __fmul_rn(dy.h, dy.h), pz = __fmul_rn(dz.h, dz.h);
-            const float cx = fmaf(__fadd_rn(__fadd_rn(dx.h, dx.h), lx), lx, fmaf(dx.h, dx.h, -px));
-            const float cy = fmaf(__fadd_rn(__fadd_rn(dy.h, dy.h), ly), ly, fmaf(dy.h, dy.h, -py));
-            const float cz = fmaf(__fadd_rn(__fadd_rn(dz.h, dz.h), lz), lz, fmaf(dz.h, dz.h, -pz));
-            const FF s1 = two_sum(px, py);
-            const FF s2 = two_sum(s1.h, pz);
-            const FF r2 = two_sum(s2.h, __fadd_rn(__fadd_rn(s1.l, s2.l), __fadd_rn(__fadd_rn(cx, cy), cz)));
-            const float r2h = r2.h, r2l = r2.l;
-            // 1/r: one Newton step y0 (1 + d/2), d = 1 - r^2 y0^2 in float-float
-            const float y0 = rsqrt_approx(r2h);
-            const float t = __fmul_rn(y0, y0), te = fmaf(y0, y0, -t);
-            const float u = __fmul_rn(r2h, t);
-            const float ue = fmaf(r2l, t, fmaf(r2h, te, fmaf(r2h, t, -u)));
-            const float d = __fsub_rn(__fsub_rn(1.f, u), ue);
-            const float corr = __fmul_rn(__fmul_rn(0.5f, y0), d);
-            const float yh = __fadd_rn(y0, corr), yl = __fsub_rn(corr, __fsub_rn(yh, y0));
-            // m / r into the float-float sum; pairs outside the normal range add nothing
-            const bool ok = r2h >= 1.17549435e-38f && r2h <= 3.40282347e38f;
-            const float ph = ok ? __fmul_rn(hj.w, yh) : 0.f;
-            const float pe = ok ? fmaf(hj.w, yl, fmaf(lj.w, yh, fmaf(hj.w, yh, -ph))) : 0.f;
-            const FF ns = two_sum(sum[q].h, ph);
-            sum[q] = {ns.h, __fadd_rn(sum[q].l, __fadd_rn(ns.l, pe))};
-          }
+      for (int c = 0; c < C / 64; ++c) {
+        FF2 part[I], sj;
+        bool ok = !self;
+        if (!self) {
+          rotation_ff<false>(pi, s_hxy + 32 * c, s_hzm + 32 * c, s_lxy + 32 * c, s_lzm + 32 * c, lane, part, sj);
+          ok = finite2(sj.h) && finite2(sj.l) && finite2(part[0].h) && finite2(part[0].l) && finite2(part[1].h) &&
+               finite2(part[1].l);
         }
+        if (__any_sync(0xffffffffu, !ok))
+          rotation_ff<true>(pi, s_hxy + 32 * c, s_hzm + 32 * c, s_lxy + 32 * c, s_lzm + 32 * c, lane, part, sj);
 #pragma unroll
-        for (int q = 0; q < kPairI; ++q) acc[q] += (double)sum[q].h + (double)sum[q].l;
+        for (int q = 0; q < I; ++q)
+          acc[q] += ((double)part[q].h.x + (double)part[q].l.x) + ((double)part[q].h.y + (double)part[q].l.y);
+        *reinterpret_cast<double2*>(&s_sum[warp][64 * c + 2 * lane]) =
+            make_double2((double)sj.h.x + (double)sj.l.x, (double)sj.h.y + (double)sj.l.y);
+      }
+      __syncthreads();
+      if (!self) {
+        double* out = a.part + (size_t)(gridDim.z + blockIdx.z * a.rounds + rr) * (size_t)a.n_total + o0 + (int64_t)B * C;
+        for (int k = tid; k < C && (int64_t)B * C + k < n; k += kPairThreads) {
+          double v = 0.0;
+#pragma unroll
+          for (int w = 0; w < kPairWarps; ++w) v += s_sum[w][k];
+          out[k] += v;
+        }
       }
     }
 #pragma unroll
-    for (int q = 0; q < kPairI; ++q) {
-      const int64_t i = ib + threadIdx.x + q * kPairThreads;
-      if (i < o1) a.part[(size_t)blockIdx.z * (size_t)a.n_total + (size_t)i] = acc[q];
+    for (int q = 0; q < I; ++q) {
+      const int64_t i = (int64_t)A * C + warp * (32 * I) + q * 32 + lane;
+      if (i < n) a.part[(size_t)blockIdx.z * (size_t)a.n_total + (size_t)(o0 + i)] += acc[q];
     }
+    __syncthreads();
   }
 }
 
@@ -246,7 +385,7 @@ __global__ void k_bound_finish(BoundArgs a) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= a.n_total) return;
   double pot = 0.0;
-  for (int s = 0; s < a.split; ++s) pot += a.part[(size_t)s * (size_t)a.n_total + (size_t)i];
+  for (int s = 0; s < a.slots; ++s) pot += a.part[(size_t)s * (size_t)a.n_total + (size_t)i];
   const V4 v = reinterpret_cast<const V4*>(a.vel)[i];
   const V4 p = reinterpret_cast<const V4*>(a.pos)[i];
   const double vx = v.x, vy = v.y, vz = v.z;
@@ -260,24 +399,33 @@ __global__ void k_bound_finish(BoundArgs a) {
   a.key[i] = (unsigned long long)__double_as_longlong(r2);
 }
 
+// One cluster of kSelectBlocks blocks per progenitor: the blocks' histograms and
+// sums meet through distributed shared memory, so a radix pass is one sweep of
+// the cluster's threads over the particles (a single block's 1024 threads took
+// 297 us at N = 1e5).
 template <typename V4>
-__global__ void __launch_bounds__(kSelectThreads) k_select(BoundArgs a) {
+__global__ void __cluster_dims__(kSelectBlocks, 1, 1) __launch_bounds__(kSelectThreads) k_select(BoundArgs a) {
+  namespace cg = cooperative_groups;
   constexpr int NW = kSelectThreads / 32;
-  __shared__ unsigned s_hist[256];
-  __shared__ double s_m[NW];
-  __shared__ unsigned long long s_c[NW];
-  __shared__ unsigned long long s_prefix, s_krem, s_nb;
-  __shared__ double s_mb;
-  const int p = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __shared__ unsigned s_hist[2][256];   // alternating: a pass is read remotely while the next is cleared
+  __shared__ unsigned s_scan[256];
+  __shared__ double s_m[NW], s_mb;
+  __shared__ unsigned long long s_c[NW], s_n;
+  __shared__ unsigned s_digit, s_below;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank();
+  const int p = blockIdx.x / kSelectBlocks, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t o0 = a.prog_off[p], o1 = a.prog_off[p + 1];
+  const int64_t first = o0 + (int64_t)rank * kSelectThreads + tid;
+  constexpr int64_t kStride = (int64_t)kSelectThreads * kSelectBlocks;
   const V4* pos = reinterpret_cast<const V4*>(a.pos);
   const uint8_t* bound = a.bound;
   const unsigned long long* key = a.key;
 
-  // bound count and bound mass (fixed order: thread strides, shuffle tree, warps in order)
+  // bound count and bound mass (fixed order: thread strides, shuffle tree, warps and blocks in order)
   unsigned long long c = 0;
   double m = 0.0;
-  for (int64_t k = o0 + tid; k < o1; k += kSelectThreads)
+  for (int64_t k = first; k < o1; k += kStride)
     if (bound[k]) {
       ++c;
       m += (double)pos[k].w;
@@ -299,74 +447,90 @@ __global__ void __launch_bounds__(kSelectThreads) k_select(BoundArgs a) {
       nb += s_c[w];
       mb += s_m[w];
     }
-    unsigned long long k = 0;
-    if (nb > 0) {
-      const double kk = ceil(a.frac * (double)nb);
-      k = kk < 1.0 ? 1ull : (unsigned long long)kk;
-      if (k > nb) k = nb;
-    }
-    s_nb = nb;
+    s_n = nb;
     s_mb = mb;
-    s_krem = k;
-    s_prefix = 0ull;
   }
-  __syncthreads();
-  const unsigned long long nb = s_nb;
-
-  // radix selection of the k-th smallest key among the bound particles
+  cluster.sync();
+  unsigned long long nb = 0;
+  double mb = 0.0;
+  for (int b = 0; b < kSelectBlocks; ++b) {
+    nb += *cluster.map_shared_rank(&s_n, b);
+    mb += *cluster.map_shared_rank(&s_mb, b);
+  }
+  unsigned long long krem = 0, prefix = 0;
   if (nb > 0) {
+    const double kk = ceil(a.frac * (double)nb);
+    krem = kk < 1.0 ? 1ull : (unsigned long long)kk;
+    if (krem > nb) krem = nb;
+    // radix selection of the k-th smallest key among the bound particles
     for (int pass = 0; pass < 8; ++pass) {
       const int shift = 56 - 8 * pass;
       const unsigned long long hi = pass == 0 ? 0ull : (~0ull << (shift + 8));
-      for (int d = tid; d < 256; d += kSelectThreads) s_hist[d] = 0u;
+      unsigned* hist = s_hist[pass & 1];
+      if (tid < 256) hist[tid] = 0u;
       __syncthreads();
-      const unsigned long long prefix = s_prefix;
-      for (int64_t k = o0 + tid; k < o1; k += kSelectThreads) {
+      for (int64_t k = first; k < o1; k += kStride) {
         if (!bound[k]) continue;
-        const unsigned long long kk = key[k];
-        if ((kk & hi) == prefix) atomicAdd(&s_hist[(kk >> shift) & 255ull], 1u);
+        const unsigned long long kk2 = key[k];
+        if ((kk2 & hi) == prefix) atomicAdd(&hist[(kk2 >> shift) & 255ull], 1u);
+      }
+      cluster.sync();
+      // every block adds all the blocks' counts and finds the digit by a scan
+      unsigned v = 0, t = 0;
+      if (tid < 256) {
+        for (int b = 0; b < kSelectBlocks; ++b) v += *cluster.map_shared_rank(&hist[tid], b);
+        t = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const unsigned u = __shfl_up_sync(0xffffffffu, t, o);
+          if (lane >= o) t += u;
+        }
+        if (lane == 31) s_scan[warp] = t;
       }
       __syncthreads();
-      if (tid == 0) {
-        const unsigned long long krem = s_krem;
-        unsigned long long cum = 0;
-        for (int d = 0; d < 256; ++d) {
-          const unsigned long long hd = s_hist[d];
-          if (cum + hd >= krem) {
-            s_prefix = prefix | ((unsigned long long)d << shift);
-            s_krem = krem - cum;
-            break;
-          }
-          cum += hd;
+      if (tid < 256) {
+        for (int w = 0; w < warp; ++w) t += s_scan[w];
+        if (t >= krem && t - v < krem) {
+          s_digit = (unsigned)tid;
+          s_below = t - v;
         }
       }
       __syncthreads();
+      prefix |= (unsigned long long)s_digit << shift;
+      krem -= s_below;
     }
   }
   // key of r_x^2 (0 = the bits of +0.0 when nothing is bound)
-  const unsigned long long kx = nb > 0 ? s_prefix : 0ull;
+  const unsigned long long kx = nb > 0 ? prefix : 0ull;
 
   // the coefficient set r <= r_x, and its size
   unsigned long long cm = 0;
-  for (int64_t k = o0 + tid; k < o1; k += kSelectThreads) {
+  for (int64_t k = first; k < o1; k += kStride) {
     const bool in = key[k] <= kx;
     if (a.mask) a.mask[k] = in ? 1 : 0;
     cm += in ? 1ull : 0ull;
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) cm += __shfl_xor_sync(0xffffffffu, cm, o);
-  __syncthreads();
+  cluster.sync();  // s_n has been read by every block
   if (lane == 0) s_c[warp] = cm;
   __syncthreads();
   if (tid == 0) {
+    unsigned long long t = 0;
+    for (int w = 0; w < NW; ++w) t += s_c[w];
+    s_n = t;
+  }
+  cluster.sync();
+  if (rank == 0 && tid == 0) {
     unsigned long long n_in = 0;
-    for (int w = 0; w < NW; ++w) n_in += s_c[w];
+    for (int b = 0; b < kSelectBlocks; ++b) n_in += *cluster.map_shared_rank(&s_n, b);
     double* st = a.stats + 4 * (size_t)p;
     st[0] = (double)nb;
-    st[1] = s_mb;
+    st[1] = mb;
     st[2] = sqrt(__longlong_as_double((long long)kx));
     st[3] = (double)n_in;
   }
+  cluster.sync();  // no block leaves while its shared memory is read
 }
 
 // Eigenvalues l1 >= l2 >= l3 of a symmetric 3x3 matrix S (row-major) by the
@@ -438,31 +602,49 @@ __global__ void k_tidal(TidalArgs a) {
 
 }  // namespace
 
-int scf_bound_split(int64_t i_chunks, int n_sm) {
-  if (i_chunks <= 0) return 1;
-  const int64_t s = (4 * (int64_t)n_sm + i_chunks - 1) / i_chunks;
-  return (int)(s < 1 ? 1 : (s > kBoundMaxSplit ? kBoundMaxSplit : s));
+int64_t scf_bound_chunk(int f32) { return f32 ? kPairChunk<float4> : kPairChunk<ScfD4>; }
+
+// Slots of the pair sums: 64, fewer where they would take more than 2 GiB (at
+// least 4: two groups of one round).
+int scf_bound_slots(int64_t n_total) {
+  const int64_t fit = n_total > 0 ? ((int64_t)1 << 31) / (8 * n_total) : kBoundMaxSlots;
+  return (int)(fit > kBoundMaxSlots ? kBoundMaxSlots : fit < 4 ? 4 : fit);
 }
 
-int64_t scf_bound_chunk(int f32) { return kPairThreads * (f32 ? Elem<float4>::I : Elem<ScfD4>::I); }
+template <typename V4>
+static void select_launch(const BoundArgs& a, cudaStream_t s) {
+  k_select<V4><<<a.n_prog * kSelectBlocks, kSelectThreads, 0, s>>>(a);
+}
 
-cudaError_t scf_bound_launch(const BoundArgs& a, int64_t max_chunks, cudaStream_t s) {
+cudaError_t scf_bound_launch(const BoundArgs& a, int64_t max_chunks, int n_sm, cudaStream_t s) {
   if (a.n_total > 0 && max_chunks > 0) {
-    const dim3 grid((unsigned)max_chunks, (unsigned)(a.n_prog < 65535 ? a.n_prog : 65535), (unsigned)a.split);
-    if (a.f32) k_bound_pairs<float4><<<grid, kPairThreads, 0, s>>>(a);
-    else k_bound_pairs_ff<<<grid, kPairThreads, 0, s>>>(a);
+    cudaError_t e = cudaMemsetAsync(a.part, 0, sizeof(double) * (size_t)a.slots * (size_t)a.n_total, s);
+    if (e != cudaSuccess) return e;
+    // groups x (1 + rounds) slots a launch: as many rounds a block (its
+    // i-particles are loaded once, its sums stored once) as still leave about 32
+    // blocks an SM, a few waves of short blocks (with eight, King N = 1e5 in
+    // double precision ran 1.5 waves a launch)
+    const int64_t total = max_chunks / 2;  // rounds of the largest progenitor
+    int groups = (int)((32 * (int64_t)n_sm + a.total_chunks - 1) / a.total_chunks);
+    groups = groups < 1 ? 1 : groups > a.slots / 2 ? a.slots / 2 : groups;
+    if (groups > total) groups = total < 1 ? 1 : (int)total;
+    BoundArgs b = a;
+    b.rounds = a.slots / groups - 1;
+    for (b.round0 = 1; b.round0 == 1 || b.round0 <= total; b.round0 += groups * b.rounds) {
+      const dim3 grid((unsigned)max_chunks, (unsigned)(a.n_prog < 65535 ? a.n_prog : 65535), (unsigned)groups);
+      if (a.f32) k_bound_pairs<<<grid, kPairThreads, 0, s>>>(b);
+      else k_bound_pairs_ff<<<grid, kPairThreads, 0, s>>>(b);
+    }
     const unsigned fb = (unsigned)((a.n_total + 255) / 256);
     if (a.f32) k_bound_finish<float4><<<fb, 256, 0, s>>>(a);
     else k_bound_finish<ScfD4><<<fb, 256, 0, s>>>(a);
   }
-  if (a.f32) k_select<float4><<<a.n_prog, kSelectThreads, 0, s>>>(a);
-  else k_select<ScfD4><<<a.n_prog, kSelectThreads, 0, s>>>(a);
-  return cudaGetLastError();
+  return scf_select_launch(a, s);
 }
 
 cudaError_t scf_select_launch(const BoundArgs& a, cudaStream_t s) {
-  if (a.f32) k_select<float4><<<a.n_prog, kSelectThreads, 0, s>>>(a);
-  else k_select<ScfD4><<<a.n_prog, kSelectThreads, 0, s>>>(a);
+  if (a.f32) select_launch<float4>(a, s);
+  else select_launch<ScfD4>(a, s);
   return cudaGetLastError();
 }
 

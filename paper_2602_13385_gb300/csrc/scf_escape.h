@@ -9,9 +9,8 @@
 
 #include "scf_device.cuh"
 
-// Upper bound on the number of j-segments the pair kernel splits each
-// progenitor into (more blocks when the progenitors are small).
-constexpr int kBoundMaxSplit = 16;
+// Most pair-sum slots (doubles per particle) of the workspace.
+constexpr int kBoundMaxSlots = 64;
 
 struct BoundArgs {
   const void* pos;             // [N][4] float (mixed) or double
@@ -20,9 +19,11 @@ struct BoundArgs {
   int n_prog;
   int64_t n_total;
   int f32;                     // particle arrays are float4
-  int split;                   // j-segments per progenitor
+  int slots;                   // slots of part
+  int64_t total_chunks;        // chunks of all progenitors
+  int round0, rounds;          // of a pair launch (set by scf_bound_launch)
   double G, kin, frac;
-  double* part;                // [split][N] partial sums of m_j / r_ij
+  double* part;                // [slots][N] partial sums of m_j / r_ij
   unsigned long long* key;     // [N] bits of r^2
   double* E_out;               // [N] energies, or null
   uint8_t* bound;              // [N] 1 = bound
@@ -40,12 +41,12 @@ struct TidalArgs {
   double* out;                 // [n_prog][16]
 };
 
-// j-segments per progenitor for a block map of i_chunks blocks in total.
-int scf_bound_split(int64_t i_chunks, int n_sm);
-// i-particles per block of the pair kernel (f32: single-precision particles).
+// Particles of a chunk of the pair kernel (f32: single-precision particles).
 int64_t scf_bound_chunk(int f32);
-// max_chunks: i-blocks of the largest progenitor.
-cudaError_t scf_bound_launch(const BoundArgs& a, int64_t max_chunks, cudaStream_t s);
+// Slots of BoundArgs::part for n_total particles.
+int scf_bound_slots(int64_t n_total);
+// max_chunks: chunks of the largest progenitor.
+cudaError_t scf_bound_launch(const BoundArgs& a, int64_t max_chunks, int n_sm, cudaStream_t s);
 cudaError_t scf_tidal_launch(const TidalArgs& a, cudaStream_t s);
 // The selection alone (bound flags and radius keys from a previous
 // scf_bound_launch; mask may be null).
