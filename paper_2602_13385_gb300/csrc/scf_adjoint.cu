@@ -19,8 +19,7 @@
 // sum_i beta(x_i + eps d_i)), and kernel 2 and kernel 3 in their ordinary
 // double form (mode ADJ_J) apply it.  The tidal term contributes T(R + x_k) d_k
 // to xbar_k and, summed per block, the partials the centre-orbit adjoint needs.
-#include "scf_device.cuh"
-#include "scf_internal.h"
+#include "scf_adjoint.cuh"
 
 static __constant__ ScfConst c_tab;
 
@@ -30,6 +29,7 @@ namespace {
 
 constexpr int kK1DualTile = 64;
 constexpr int kK3DualThreads = 128;
+constexpr int kComAdjThreads = 256;  // the binned field pass leaves one row of partials a warp
 
 __device__ __forceinline__ Dual dual_pos(double x, double d) { return Dual(x, d); }
 
@@ -292,28 +292,7 @@ __global__ void __launch_bounds__(kK3DualThreads) k3_dual(K3Args a) {
                      gy, gz);
     if (has_host) {
       const double Px = s_R[0] + p.x, Py = s_R[1] + p.y, Pz = s_R[2] + p.z;
-      Dual hx, hy, hz;
-      scf_host_accel_t<Dual>(a.host, Dual(Px, dx), Dual(Py, dy), Dual(Pz, dz), hx, hy, hz);
-      gx += hx.d;
-      gy += hy.d;
-      gz += hz.d;
-      acc[0] += dx;
-      acc[1] += dy;
-      acc[2] += dz;
-      acc[3] += hx.d;
-      acc[4] += hy.d;
-      acc[5] += hz.d;
-#pragma unroll
-      for (int c = 0; c < SCF_HOST_CAP; ++c) {
-        if (c >= a.host.n) break;
-        double ux, uy, uz;  // a_c / GM_c
-        scf_host_comp_accel<double>(a.host.kind[c], 1.0, a.host.a[c], a.host.b[c], Px, Py, Pz, ux, uy, uz);
-        Dual sx, sy, sz;    // derivative in the scale length a_c
-        scf_host_comp_accel<Dual>(a.host.kind[c], Dual(a.host.GM[c]), Dual(a.host.a[c], 1.0), Dual(a.host.b[c]),
-                                  Dual(Px), Dual(Py), Dual(Pz), sx, sy, sz);
-        acc[6 + 2 * c] += dx * ux + dy * uy + dz * uz;
-        acc[7 + 2 * c] += dx * sx.d + dy * sy.d + dz * sz.d;
-      }
+      scf_adj_tide(a.host, Px, Py, Pz, dx, dy, dz, gx, gy, gz, acc);
     }
     if (!(isfinite(gx) && isfinite(gy) && isfinite(gz))) atomicOr(a.status, 2u);
     ScfD4 X = xb4[k];
@@ -341,7 +320,7 @@ __global__ void __launch_bounds__(kK3DualThreads) k3_dual(K3Args a) {
 }
 
 // ---------------------------------------------------------------------------
-// Centre-orbit adjoint at one level, one warp per progenitor.  With S the
+// Centre-orbit adjoint at one level, one block per progenitor.  With S the
 // progenitor's summed partials and u = w Vbar - sum d:
 //   Rbar += sum T(P_k) d_k + T(R) u
 //   GMbar_c += sum d_k . a_c(P_k)/GM_c + a_c(R)/GM_c . u
@@ -350,14 +329,15 @@ __global__ void __launch_bounds__(kK3DualThreads) k3_dual(K3Args a) {
 // level), then, unless this is the last level of the sweep, the drift is
 // undone: Vbar += dt Rbar.
 // ---------------------------------------------------------------------------
-__global__ void k_com_adj(ComAdjArgs a) {
+__global__ void __launch_bounds__(kComAdjThreads) k_com_adj(ComAdjArgs a) {
+  __shared__ double s_red[kComAdjThreads / 32][SCF_ADJ_Q];
   const int p = blockIdx.x;
-  const int lane = threadIdx.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nq = 6 + 2 * a.host.n;
   double S[SCF_ADJ_Q];
 #pragma unroll
   for (int i = 0; i < SCF_ADJ_Q; ++i) S[i] = 0.0;
-  for (int b = lane; b < a.n_blocks; b += 32) {
+  for (int b = threadIdx.x; b < a.n_blocks; b += kComAdjThreads) {
     if (a.blk3_prog[b] != p) continue;
     const double* src = a.part + (size_t)b * SCF_ADJ_Q;
 #pragma unroll
@@ -368,7 +348,15 @@ __global__ void k_com_adj(ComAdjArgs a) {
   for (int i = 0; i < SCF_ADJ_Q; ++i)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) S[i] += __shfl_xor_sync(0xffffffffu, S[i], o);
-  if (lane != 0) return;
+  if (lane == 0)
+#pragma unroll
+    for (int i = 0; i < SCF_ADJ_Q; ++i) s_red[warp][i] = S[i];
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+#pragma unroll
+  for (int w = 1; w < kComAdjThreads / 32; ++w)
+#pragma unroll
+    for (int i = 0; i < SCF_ADJ_Q; ++i) S[i] += s_red[w][i];
   const double* R = a.com + 6 * p;
   double* cb = a.combar + 6 * p;
   const double ux = a.weight * cb[3] - S[0], uy = a.weight * cb[4] - S[1], uz = a.weight * cb[5] - S[2];
@@ -472,6 +460,6 @@ cudaError_t scf_k3_dual_launch(const K3Args& a, int blocks, const ScfLaunchInfo&
 }
 
 cudaError_t scf_com_adj_launch(const ComAdjArgs& a, cudaStream_t s) {
-  k_com_adj<<<a.n_prog, 32, 0, s>>>(a);
+  k_com_adj<<<a.n_prog, kComAdjThreads, 0, s>>>(a);
   return cudaGetLastError();
 }

@@ -122,6 +122,7 @@ struct scf_handle {
            *d_bin_start = nullptr, *d_task_start = nullptr, *d_field_start = nullptr;
   double* d_binv = nullptr;
   std::vector<int64_t> h_sb_begin;       // host copy: particle ranges of the sorting blocks
+  double* d_bin_adj_part = nullptr;   // double precision: [bin_fblocks][SCF_ADJ_Q]
   void *d_spos = nullptr, *d_mrows = nullptr, *d_bin_frame = nullptr, *d_field_rows = nullptr;
   int2* d_skey = nullptr;
   double *d_bin_t = nullptr, *d_bin_aux = nullptr;  // tables; nodes, node-to-monomial matrix and gscale
@@ -182,6 +183,7 @@ int upload_tables_once(int device) {
   if (e5 == cudaSuccess) e5 = scf_upload_const_bins(&b);
   if (e5 == cudaSuccess) e5 = scf_upload_const_bin_moments(&b);
   if (e5 == cudaSuccess) e5 = scf_upload_const_bin_field(&b);
+  if (e5 == cudaSuccess) e5 = scf_upload_const_bin_adjoint(&b);
   delete t;
   if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess || e4 != cudaSuccess || e5 != cudaSuccess)
     return SCF_ERR_CUDA;
@@ -394,12 +396,7 @@ int run_sort(scf_handle* h, void* pos, void* vel, const void* acc, const uint8_t
   return cuda_fail(scf_bin_sort_launch(a, h->stream));
 }
 
-// Kernel 1 over radial bins: sort, moments, partial coefficient rows.
-int run_binned_k1(scf_handle* h, void* pos, void* vel, const void* acc, const uint8_t* mask, int mode, void* pos_copy,
-                  void* vel_out) {
-  const int f32 = h->cfg.precision == SCF_MIXED;
-  int rc = run_sort(h, pos, vel, acc, mask, mode, pos_copy, vel_out, true);
-  if (rc != SCF_OK) return rc;
+MomentArgs moment_args(const scf_handle* h) {
   MomentArgs m{};
   m.spos = h->d_spos;
   m.bin_start = h->d_bin_start;
@@ -416,7 +413,11 @@ int run_binned_k1(scf_handle* h, void* pos, void* vel, const void* acc, const ui
   m.alphaf = (float)m.alpha;
   m.inv_alphaf = (float)m.inv_alpha;
   m.K = h->bin.K;
-  if (scf_moments_launch(f32, h->bin, m, h->bin_mblocks, h->stream) != cudaSuccess) return SCF_ERR_CUDA;
+  return m;
+}
+
+// Moment rows -> partial coefficient rows, one per bin group.
+int run_transform(scf_handle* h) {
   TransformArgs t{};
   t.rows = h->d_mrows;
   t.row_off = h->d_mrow_off;
@@ -433,8 +434,18 @@ int run_binned_k1(scf_handle* h, void* pos, void* vel, const void* acc, const ui
   t.nlm = h->nlm;
   t.nc = h->nc;
   t.n_prog = h->n_prog;
-  t.f32 = f32;
+  t.f32 = h->cfg.precision == SCF_MIXED;
   return cuda_fail(scf_transform_launch(t, h->stream));
+}
+
+// Kernel 1 over radial bins: sort, moments, partial coefficient rows.
+int run_binned_k1(scf_handle* h, void* pos, void* vel, const void* acc, const uint8_t* mask, int mode, void* pos_copy,
+                  void* vel_out) {
+  int rc = run_sort(h, pos, vel, acc, mask, mode, pos_copy, vel_out, true);
+  if (rc != SCF_OK) return rc;
+  if (scf_moments_launch(h->cfg.precision == SCF_MIXED, h->bin, moment_args(h), h->bin_mblocks, h->stream) != cudaSuccess)
+    return SCF_ERR_CUDA;
+  return run_transform(h);
 }
 
 int run_coeffs(scf_handle* h, void* pos, void* vel, const void* acc, const uint8_t* mask, double* A_out, double* com,
@@ -483,9 +494,10 @@ int run_prep(scf_handle* h, const double* A, const double* com) {
   return cuda_fail(timed(h, 1, [&] { return scf_prep_launch(p, h->stream); }));
 }
 
-// Kernel 3 over radial bins: field rows from F, then the sorted particles.
+// Kernel 3 over radial bins: field rows from F, then the sorted particles (adj:
+// its adjoint modes).
 int run_binned_k3(scf_handle* h, void* vel, void* acc, const double* com, int mode, const void* vel_in, int seg0 = 0,
-                  int seg1 = 0) {
+                  int seg1 = 0, const AdjArgs* adj = nullptr) {
   const int f32 = h->cfg.precision == SCF_MIXED;
   FieldRowArgs r{};
   r.F = h->d_F;
@@ -535,6 +547,8 @@ int run_binned_k3(scf_handle* h, void* vel, void* acc, const double* com, int mo
   a.inv_alpha = 1.0 / h->cfg.alpha;
   a.host = h->host;
   a.status = h->d_status;
+  if (adj) a.adj = *adj;
+  if (mode == SCF_MODE_ADJ_DUAL) return cuda_fail(scf_bin_field_dual_launch(h->bin, a, h->bin_fblocks, h->stream));
   return cuda_fail(scf_bin_field_launch(f32, h->bin, a, h->bin_fblocks, h->stream));
 }
 
@@ -872,6 +886,7 @@ int bin_init(scf_handle* h) {
   const size_t o_ro = take(4 * (np + 1)), o_id = take(4 * n), o_hist = take(4 * nsb * K), o_tot = take(4 * np * K);
   const size_t o_bs = take(4 * np * (K + 1)), o_ts = take(4 * np * (K + 1));
   const size_t o_sp = take(32 * n), o_key = f32 ? off : take(8 * n);
+  const size_t o_adj = f32 ? off : take(sizeof(double) * SCF_ADJ_Q * nfb);
   const size_t o_rows = take(es * (size_t)rows * s.T * scf_bin_colpad(s.L));
   const size_t o_fr = take(2 * es * K), o_P = take(es * np * K * scf_bin_row(s.L, s.T));
   const size_t o_t = f32 ? off : take(8 * K * nl * nn * s.T), o_tf = f32 ? take(4 * K * nl * nn * s.T) : off,
@@ -892,6 +907,7 @@ int bin_init(scf_handle* h) {
   at(h->d_fb_task, o_fbt), at(h->d_bin_ticket, o_tk), at(h->d_field_start, o_fs), at(h->d_binv, o_bi);
   h->d_spos = base + o_sp;
   h->d_mrows = base + o_rows;
+  if (!f32) at(h->d_bin_adj_part, o_adj);
   h->d_bin_frame = base + o_fr;
   h->d_field_rows = base + o_P;
   at(h->d_bin_t, o_t), at(h->d_bin_tf, o_tf), at(h->d_bin_t2, o_t2), at(h->d_bin_aux, o_aux);
@@ -1536,6 +1552,8 @@ int scf_adjoint_level(scf_handle* h, const void* pos, const double* com, double 
   if (!aligned16(pos) || !aligned16(xbar) || !aligned16(vbar)) return SCF_ERR_MISALIGNED;
   if (!std::isfinite(weight)) return SCF_ERR_INVALID_ARG;
   if (h->n_total == 0) return SCF_OK;
+  // over radial bins as the passes themselves: one sort serves the whole level
+  const bool binned = bins_k1(h) && bins_k3(h);
   if (!h->adj_ready) {
     int bps = 0;
     if (scf_k1_dual_prepare(h->cfg.lmax, h->cfg.nmax, &h->k1d, &bps) != cudaSuccess || bps < 1 ||
@@ -1553,12 +1571,15 @@ int scf_adjoint_level(scf_handle* h, const void* pos, const double* com, double 
   adj.vbar = vbar;
   adj.weight = weight;
   adj.drift = drift ? 1 : 0;
-  adj.part = h->d_adj_part;
+  adj.part = binned ? h->d_bin_adj_part : h->d_adj_part;
   // 1. coefficients and force coefficients at x_t
   int rc = run_coeffs(h, p, nullptr, nullptr, nullptr, h->d_A, nullptr, SCF_MODE_COEFFS);
   if (rc != SCF_OK) return rc;
   // 2. own-position term and tidal partials (dual numbers)
-  if (h->k3_blocks > 0) {
+  if (binned) {
+    rc = run_binned_k3(h, nullptr, nullptr, host ? com : nullptr, SCF_MODE_ADJ_DUAL, nullptr, 0, 0, &adj);
+    if (rc != SCF_OK) return rc;
+  } else if (h->k3_blocks > 0) {
     K3Args a = k3_args(h, pos, nullptr, nullptr, host ? com : nullptr, SCF_MODE_ADJ_DUAL);
     a.adj = adj;
     if (scf_k3_dual_launch(a, h->k3_blocks, h->k3d, h->stream) != cudaSuccess) return SCF_ERR_CUDA;
@@ -1566,9 +1587,9 @@ int scf_adjoint_level(scf_handle* h, const void* pos, const double* com, double 
   // 3. centre orbit and host parameters
   if (host) {
     ComAdjArgs c{};
-    c.part = h->d_adj_part;
-    c.blk3_prog = h->d_blk3_prog;
-    c.n_blocks = h->k3_blocks;
+    c.part = adj.part;
+    c.blk3_prog = binned ? h->d_fb_prog : h->d_blk3_prog;
+    c.n_blocks = binned ? h->bin_fblocks : h->k3_blocks;
     c.com = com;
     c.combar = combar;
     c.thetabar = thetabar;
@@ -1580,14 +1601,25 @@ int scf_adjoint_level(scf_handle* h, const void* pos, const double* com, double 
     if (scf_com_adj_launch(c, h->stream) != cudaSuccess) return SCF_ERR_CUDA;
   }
   // 4. A^J = sum_i d_i . grad B(x_i) (dual numbers, unit weights), normalised by kernel 2
-  if (h->k1_blocks > 0) {
+  K2Args b = k2_args(h, h->d_A, nullptr, SCF_MODE_COEFFS);
+  if (binned) {
+    MomentDualArgs a{};
+    a.m = moment_args(h);
+    a.skey = h->d_skey;
+    a.adj = adj;
+    if (scf_moments_dual_launch(h->bin, a, h->bin_mblocks, h->stream) != cudaSuccess) return SCF_ERR_CUDA;
+    rc = run_transform(h);
+    if (rc != SCF_OK) return rc;
+    b.prog_blk_off = h->d_bin_rows_off;
+    b.sub = 0;
+  } else if (h->k1_blocks > 0) {
     K1Args a = k1_args(h, p, nullptr, nullptr, nullptr, SCF_MODE_ADJ_DUAL);
     a.adj = adj;
     if (scf_k1_dual_launch(a, h->k1_blocks, h->k1d, h->stream) != cudaSuccess) return SCF_ERR_CUDA;
   }
-  K2Args b = k2_args(h, h->d_A, nullptr, SCF_MODE_COEFFS);
   if (scf_k2_launch(b, h->stream) != cudaSuccess) return SCF_ERR_CUDA;
   // 5. xbar_k += m_k f(x_k; A^J), then the drift is undone
+  if (binned) return run_binned_k3(h, nullptr, nullptr, nullptr, SCF_MODE_ADJ_J, nullptr, 0, 0, &adj);
   if (h->k3_blocks > 0) {
     K3Args a = k3_args(h, pos, nullptr, nullptr, nullptr, SCF_MODE_ADJ_J);
     a.adj = adj;

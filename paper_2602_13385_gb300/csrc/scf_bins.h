@@ -121,6 +121,13 @@ struct MomentArgs {
   float alphaf, inv_alphaf;
   int K;
 };
+// Adjoint: the directional derivative of the moments of unit masses along weight * vbar.
+struct MomentDualArgs {
+  MomentArgs m;
+  const int2* skey;
+  AdjArgs adj;
+};
+cudaError_t scf_moments_dual_launch(const ScfBinShape& sh, const MomentDualArgs& a, int blocks, cudaStream_t s);
 cudaError_t scf_moments_launch(int f32, const ScfBinShape& sh, const MomentArgs& a, int blocks, cudaStream_t s);
 
 // Moment rows -> partial coefficient rows [prog][groups][2 NC] (doubles).
@@ -177,8 +184,11 @@ struct BinFieldArgs {
   const int* prog_blk_off;
   const unsigned* hist;
   const unsigned* total;
+  AdjArgs adj;             // modes ADJ_J and ADJ_DUAL (double precision)
 };
 constexpr int kBinField64Threads = 32;
+// xbar += derivative of the field along weight * vbar (and the tidal partials, one row a block).
+cudaError_t scf_bin_field_dual_launch(const ScfBinShape& sh, const BinFieldArgs& a, int blocks, cudaStream_t s);
 cudaError_t scf_bin_field_launch(int f32, const ScfBinShape& sh, const BinFieldArgs& a, int blocks, cudaStream_t s);
 
 // Interpolation polynomials of the family in `tab` (alpha): frame and t tables.
@@ -200,3 +210,4 @@ void scf_bin_nodes(int T, double* nodes, double* vinv);
 cudaError_t scf_upload_const_bins(const ScfBinConst* t);
 cudaError_t scf_upload_const_bin_moments(const ScfBinConst* t);
 cudaError_t scf_upload_const_bin_field(const ScfBinConst* t);
+cudaError_t scf_upload_const_bin_adjoint(const ScfBinConst* t);

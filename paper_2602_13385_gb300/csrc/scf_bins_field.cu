@@ -256,6 +256,25 @@ __device__ __forceinline__ void field_of(const BinFieldArgs& a, typename Vec<T>:
   }
   out.w = pot;
   if (!(isfinite(out.x) && isfinite(out.y) && isfinite(out.z))) atomicOr(a.status, 2u);
+  if constexpr (sizeof(T) == 8) {
+    if (a.mode == SCF_MODE_ADJ_J) {  // xbar_k += m_k f(x_k; A^J), then the drift is undone, as in the direct kernel
+      ScfD4* xb = reinterpret_cast<ScfD4*>(a.adj.xbar) + idx;
+      ScfD4 X = *xb;
+      X.x += p.w * out.x;
+      X.y += p.w * out.y;
+      X.z += p.w * out.z;
+      *xb = X;
+      if (a.adj.drift) {
+        ScfD4* vb = reinterpret_cast<ScfD4*>(a.adj.vbar) + idx;
+        ScfD4 V = *vb;
+        V.x += a.dt * X.x;
+        V.y += a.dt * X.y;
+        V.z += a.dt * X.z;
+        *vb = V;
+      }
+      return;
+    }
+  }
   reinterpret_cast<V4*>(a.acc)[idx] = out;
   if (a.mode == SCF_MODE_STEP) {
     const T h = (T)fh.half_dt;
