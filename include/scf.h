@@ -49,8 +49,8 @@
  * word), allocated once in scf_init.  No call allocates after scf_init
  * (scf_step_host's first call excepted, see there).
  *
- * Radial bins.  A handle with enough particles for its (nmax, lmax) runs the
- * coefficient and field passes of every entry point over particles sorted by
+ * Radial bins.  A handle with enough particles for its (nmax, lmax) runs its
+ * coefficient and field passes (alone, from a larger size) over particles sorted by
  * radius, with the radial polynomials of each radius bin replaced by
  * interpolants exact to the precision's rounding (workspace of about 40 bytes
  * a particle and the bins' tables; without the memory for it the handle keeps
@@ -203,8 +203,8 @@ int scf_step(scf_handle* h, void* pos, void* vel, void* acc, double* com, int ns
  * owned by the handle (2 records per particle, allocated by the first such
  * call, freed by scf_free), so the host link carries the state in once and out
  * once; over radial bins kernel 3 leaves its results there and they go back by
- * copies on a second stream of the handle, which its own stream waits for (in
- * four pieces in SCF_MIXED).  Otherwise the state is staged through the
+ * copies.  (In SCF_MIXED the host link bounds such a step and it runs the
+ * direct kernels unless SCF_OPT_RADIAL_BINS is 2.)  Otherwise the state is staged through the
  * device arrays: copied in on a second stream of the handle, kernels 1 and 2,
  * then the positions and the centres copied back while kernel 3 runs, which
  * is launched in `chunks` pieces of its block map so that each piece's
@@ -261,6 +261,10 @@ int scf_step_host(scf_handle* h, void* pos, void* vel, void* acc, double* com, v
  *                     one that was stepped ahead (same dt); 0 = kernel 2
  *                     always computes it.  Either way the results are
  *                     bitwise the same.
+ *   SCF_OPT_RADIAL_BINS 0 = the direct kernels in every pass; 1 (default) =
+ *                     radial bins in the passes that are faster over them (size
+ *                     rules per entry point); 2 = in every pass of a handle
+ *                     that has bins.
  * Setting a tile or block size synchronises the stream and rewrites the block
  * maps in the workspace (sized in scf_init for every allowed value).
  * Errors: SCF_ERR_NULL_POINTER, SCF_ERR_INVALID_ARG (unknown option or value),
@@ -271,6 +275,7 @@ int scf_step_host(scf_handle* h, void* pos, void* vel, void* acc, double* com, v
 #define SCF_OPT_K1_VARIANT 4
 #define SCF_OPT_K3_VARIANT 5
 #define SCF_OPT_CENTRE_AHEAD 6
+#define SCF_OPT_RADIAL_BINS 7
 int scf_set_option(scf_handle* h, int option, int value);
 int scf_get_option(const scf_handle* h, int option, int* value);
 

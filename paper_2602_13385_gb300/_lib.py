@@ -49,6 +49,7 @@ SCF_OPT_K3_BLOCK = 3
 SCF_OPT_K1_VARIANT = 4
 SCF_OPT_K3_VARIANT = 5
 SCF_OPT_CENTRE_AHEAD = 6
+SCF_OPT_RADIAL_BINS = 7
 
 
 class ScfError(RuntimeError):

@@ -108,7 +108,8 @@ struct scf_handle {
   // radial bins (scf_bins.h): the coefficient and field passes over particles
   // sorted by radius, for handles that choose_bins admits
   bool binned = false;                   // tables for the current exponent are in place
-  bool bins_off = false;                 // the direct kernels for now (the autotuner times them)
+  bool bins_off = false;                 // the direct kernels for now (autotuner, single-precision host steps)
+  int bins_mode = 1;                     // SCF_OPT_RADIAL_BINS
   ScfBinShape bin{};
   int bin_kcap = 0;                      // bins the allocation holds
   int bin_blocks = 0, bin_mblocks = 0, bin_fblocks = 0;  // sorting, moment and field blocks
@@ -121,7 +122,6 @@ struct scf_handle {
   unsigned *d_bin_code = nullptr, *d_bin_hist = nullptr, *d_bin_total = nullptr, *d_bin_ticket = nullptr,
            *d_bin_start = nullptr, *d_task_start = nullptr, *d_field_start = nullptr;
   double* d_binv = nullptr;
-  std::vector<int64_t> h_sb_begin;       // host copy: particle ranges of the sorting blocks
   double* d_bin_adj_part = nullptr;   // double precision: [bin_fblocks][SCF_ADJ_Q]
   void *d_spos = nullptr, *d_mrows = nullptr, *d_bin_frame = nullptr, *d_field_rows = nullptr;
   int2* d_skey = nullptr;
@@ -349,9 +349,37 @@ K3Args k3_args(scf_handle* h, const void* pos, void* vel, void* acc, const doubl
 // The radial-bin passes replace the default kernels: register-tiled kernel 1 in
 // mixed precision, the native kernels in double precision.
 bool bins_k1(const scf_handle* h) {
-  return h->binned && !h->bins_off && (h->cfg.precision == SCF_MIXED ? h->k1.variant == 1 : h->k1.variant != 2);
+  return h->binned && !h->bins_off && h->bins_mode != 0 && (h->cfg.precision == SCF_MIXED ? h->k1.variant == 1 : h->k1.variant != 2);
 }
-bool bins_k3(const scf_handle* h) { return h->binned && !h->bins_off && h->k3.variant != 2; }
+bool bins_k3(const scf_handle* h) {
+  return h->binned && !h->bins_off && h->bins_mode != 0 && h->k3.variant != 2;
+}
+
+// The coefficients or the field alone: a step shares one sort and one set of
+// per-progenitor passes between the two, so alone each pays from a larger size.
+// Measured on a GB300, bins against direct (us; P progenitors):
+//   coefficients, mixed   (10,5) 600k 73/73, P = 8 79/72;  (20,10) 200k 70/70, 600k 105/152, P = 8 132/153
+//   coefficients, double  (10,5) 60k 143/131, 200k 274/361;  (20,8) 16k 153/149, 60k 271/360, P = 8 413/355, 140k 610/686
+//   field, mixed          (10,5) 600k 75/58, P = 8 77/58;  (20,10) 200k 69/81, 600k 110/193, P = 8 136/193
+//   field, double         (10,5) 60k 171/240;  (20,8) 12k 134/208, 60k 314/686, P = 8 407/688
+// (what the bins save grows with W above a floor that the sort costs; the field in double precision
+// pays wherever the step does).
+bool bins_alone(const scf_handle* h, bool field) {
+  if (h->bins_mode == 2 || (field && h->cfg.precision == SCF_FP64)) return true;
+  const double n = (double)h->n_total, P = h->n_prog, W = (h->cfg.nmax + 1.0) * (h->cfg.lmax + 1.0) * (h->cfg.lmax + 1.0);
+  if (W <= 350.0) return false;
+  if (h->cfg.precision == SCF_FP64) return n >= 2000.0 + 14000.0 * (P - 1.0) + 2.0e7 / (W - 280.0);
+  return field ? n >= 30000.0 * P + 1.8e8 / (W - 350.0) : n >= 35000.0 * P + 4.0e8 / W;
+}
+bool bins_coeffs(const scf_handle* h) { return bins_k1(h) && bins_alone(h, false); }
+bool bins_forces(const scf_handle* h) { return bins_k3(h) && bins_alone(h, true); }
+
+// The state of a step in host memory crosses the link inside the direct
+// kernels; over radial bins the sorted passes wait for all of it.  In single
+// precision the link bounds the step and the direct kernels are faster (us, bins
+// against direct, mapped memory: (10,5) 400k 256/193, 700k 411/316; (20,10) 200k 214/151, 700k 454/428,
+// 1e6 607/599, eight progenitors 700k 554/430); in double precision the bins stay ((20,8) 60k 615/1085).
+bool host_step_direct(const scf_handle* h) { return h->cfg.precision == SCF_MIXED && h->bins_mode != 2; }
 
 // Sorts the particles by bin (step mode: after the half kick and drift, which
 // leave the velocities in vel_out and a copy of the positions in pos_copy when given).
@@ -449,8 +477,8 @@ int run_binned_k1(scf_handle* h, void* pos, void* vel, const void* acc, const ui
 }
 
 int run_coeffs(scf_handle* h, void* pos, void* vel, const void* acc, const uint8_t* mask, double* A_out, double* com,
-               int mode, void* pos_copy = nullptr, void* vel_out = nullptr) {
-  const bool binned = bins_k1(h);
+               int mode, void* pos_copy = nullptr, void* vel_out = nullptr, bool alone = false) {
+  const bool binned = alone ? bins_coeffs(h) : bins_k1(h);
   if (binned) {
     if (timed(h, 0, [&] {
           return run_binned_k1(h, pos, vel, acc, mask, mode, pos_copy, vel_out) == SCF_OK ? cudaSuccess
@@ -496,8 +524,8 @@ int run_prep(scf_handle* h, const double* A, const double* com) {
 
 // Kernel 3 over radial bins: field rows from F, then the sorted particles (adj:
 // its adjoint modes).
-int run_binned_k3(scf_handle* h, void* vel, void* acc, const double* com, int mode, const void* vel_in, int seg0 = 0,
-                  int seg1 = 0, const AdjArgs* adj = nullptr) {
+int run_binned_k3(scf_handle* h, void* vel, void* acc, const double* com, int mode, const void* vel_in,
+                  const AdjArgs* adj = nullptr) {
   const int f32 = h->cfg.precision == SCF_MIXED;
   FieldRowArgs r{};
   r.F = h->d_F;
@@ -513,8 +541,7 @@ int run_binned_k3(scf_handle* h, void* vel, void* acc, const double* com, int mo
   r.nc = h->nc;
   r.n_prog = h->n_prog;
   r.f32 = f32;
-  // (the rows serve every segment)
-  if (seg0 == 0 && scf_field_rows_launch(r, h->stream) != cudaSuccess) return SCF_ERR_CUDA;
+  if (scf_field_rows_launch(r, h->stream) != cudaSuccess) return SCF_ERR_CUDA;
   BinFieldArgs a{};
   a.spos = h->d_spos;
   a.skey = h->d_skey;
@@ -537,11 +564,6 @@ int run_binned_k3(scf_handle* h, void* vel, void* acc, const double* com, int mo
   a.K = h->bin.K;
   a.mode = mode;
   a.n_prog = h->n_prog;
-  a.seg0 = seg0;
-  a.seg1 = seg1;
-  a.prog_blk_off = h->d_sb_off;
-  a.hist = h->d_bin_hist;
-  a.total = h->d_bin_total;
   a.dt = h->cfg.dt;
   a.alpha = h->cfg.alpha;
   a.inv_alpha = 1.0 / h->cfg.alpha;
@@ -555,9 +577,9 @@ int run_binned_k3(scf_handle* h, void* vel, void* acc, const double* com, int mo
 // Kernel 3 on the handle's F / a_host(R) (from kernel 2 or run_prep).  sorted:
 // run_coeffs has just run on the same positions (its sort serves this pass too).
 int run_forces(scf_handle* h, const void* pos, void* vel, void* acc, const double* com, int mode,
-               const void* vel_in = nullptr, bool sorted = false) {
+               const void* vel_in = nullptr, bool sorted = false, bool alone = false) {
   if (h->k3_blocks == 0) return SCF_OK;
-  if (bins_k3(h) && mode != SCF_MODE_ADJ_J) {
+  if (alone ? bins_forces(h) : bins_k3(h)) {
     return cuda_fail(timed(h, 2, [&] {
       int rc = sorted && bins_k1(h) ? SCF_OK
                                     : run_sort(h, const_cast<void*>(pos), nullptr, nullptr, nullptr, SCF_MODE_COEFFS,
@@ -568,7 +590,7 @@ int run_forces(scf_handle* h, const void* pos, void* vel, void* acc, const doubl
   }
   K3Args a = k3_args(h, pos, vel, acc, com, mode);
   a.vel_in = vel_in;
-  if (h->k3.variant == 2 && mode != SCF_MODE_ADJ_J)
+  if (h->k3.variant == 2)
     return cuda_fail(timed(h, 2, [&] { return scf_k3_ff_launch(a, h->k3_blocks, h->k3, h->stream); }));
   return cuda_fail(
       timed(h, 2, [&] { return scf_k3_launch(h->cfg.precision, a, h->k3_blocks, h->k3_native, h->stream); }));
@@ -915,7 +937,6 @@ int bin_init(scf_handle* h) {
   h->bin_blocks = (int)nsb;
   h->bin_mblocks = (int)mb_prog.size();
   h->bin_fblocks = (int)nfb;
-  h->h_sb_begin = sm.begin;
   const bool ok = put(h->d_sb_prog, sm.prog.data(), 4 * nsb) && put(h->d_sb_begin, sm.begin.data(), 8 * nsb) &&
                   put(h->d_sb_end, sm.end.data(), 8 * nsb) && put(h->d_sb_off, sb_off.data(), 4 * (np + 1)) &&
                   put(h->d_fb_prog, fm.prog.data(), 4 * nfb) && put(h->d_mb_prog, mb_prog.data(), 4 * mb_prog.size()) &&
@@ -1132,7 +1153,8 @@ int scf_init(const scf_config* cfg, int n_prog, const int64_t* offsets, const do
 int scf_coeffs(scf_handle* h, const void* pos, const uint8_t* mask, double* A_out) {
   if (!h || !A_out || (!pos && h->n_total > 0)) return SCF_ERR_NULL_POINTER;
   if (!aligned16(pos)) return SCF_ERR_MISALIGNED;
-  return run_coeffs(h, const_cast<void*>(pos), nullptr, nullptr, mask, A_out, nullptr, SCF_MODE_COEFFS);
+  return run_coeffs(h, const_cast<void*>(pos), nullptr, nullptr, mask, A_out, nullptr, SCF_MODE_COEFFS, nullptr,
+                    nullptr, true);
 }
 
 int scf_forces(scf_handle* h, const void* pos, const double* A, const double* com, void* acc) {
@@ -1141,12 +1163,10 @@ int scf_forces(scf_handle* h, const void* pos, const double* A, const double* co
   if (!aligned16(pos) || !aligned16(acc)) return SCF_ERR_MISALIGNED;
   int rc = run_prep(h, A, com);
   if (rc != SCF_OK) return rc;
-  return run_forces(h, pos, nullptr, acc, com, SCF_MODE_COEFFS);
+  return run_forces(h, pos, nullptr, acc, com, SCF_MODE_COEFFS, nullptr, false, true);
 }
 
 namespace {
-
-constexpr int kHostSegments = 4;  // pieces in which a host-memory state goes back
 
 // The handle's copy stream and its events, made by the first call that needs them.
 bool make_copy_stream(scf_handle* h) {
@@ -1203,32 +1223,11 @@ int launch_step(scf_handle* h, void* pos, void* vel, void* acc, double* com, boo
   }
   if (split && bins_k3(h)) {
     // the sorted pass writes in radial order: onto the device copies (the
-    // positions' one is free again once they are sorted), which go back by the
-    // copy stream, segment by segment of the caller's order in single precision
-    const size_t rec = h->cfg.precision == SCF_MIXED ? 16 : 32;
-    const int segs = h->cfg.precision == SCF_MIXED && h->bin_blocks >= kHostSegments ? kHostSegments : 1;
-    if (!make_copy_stream(h)) return SCF_ERR_CUDA;
-    for (int c = 0; c < segs && rc == SCF_OK; ++c) {
-      const int b0 = (int)((int64_t)h->bin_blocks * c / segs), b1 = (int)((int64_t)h->bin_blocks * (c + 1) / segs);
-      rc = segs == 1 ? run_forces(h, spos, svel, spos, com, SCF_MODE_STEP, svel, true)
-                     : cuda_fail(timed(h, 2, [&] {
-                         return run_binned_k3(h, svel, spos, com, SCF_MODE_STEP, svel, b0, b1) == SCF_OK
-                                    ? cudaSuccess
-                                    : cudaErrorUnknown;
-                       }));
-      const size_t k0 = rec * (size_t)h->h_sb_begin[b0],
-                   k1 = rec * (size_t)(b1 < h->bin_blocks ? h->h_sb_begin[b1] : h->n_total);
-      auto ok = [](cudaError_t e) { return e == cudaSuccess; };
-      if (rc == SCF_OK &&
-          !(ok(cudaEventRecord(h->stage_ev[c], h->stream)) && ok(cudaStreamWaitEvent(h->copy_stream, h->stage_ev[c], 0)) &&
-            ok(cudaMemcpyAsync(static_cast<char*>(acc) + k0, static_cast<char*>(spos) + k0, k1 - k0, cudaMemcpyDefault,
-                               h->copy_stream)) &&
-            ok(cudaMemcpyAsync(static_cast<char*>(vel) + k0, static_cast<char*>(svel) + k0, k1 - k0, cudaMemcpyDefault,
-                               h->copy_stream))))
-        rc = SCF_ERR_CUDA;
-    }
-    if (rc == SCF_OK && (cudaEventRecord(h->stage_ev[kHostSegments], h->copy_stream) != cudaSuccess ||
-                         cudaStreamWaitEvent(h->stream, h->stage_ev[kHostSegments], 0) != cudaSuccess))
+    // positions' one is free again once they are sorted), which then go back whole
+    const size_t bytes = (h->cfg.precision == SCF_MIXED ? 16 : 32) * (size_t)h->n_total;
+    rc = run_forces(h, spos, svel, spos, com, SCF_MODE_STEP, svel, true);
+    if (rc == SCF_OK && (cudaMemcpyAsync(acc, spos, bytes, cudaMemcpyDefault, h->stream) != cudaSuccess ||
+                         cudaMemcpyAsync(vel, svel, bytes, cudaMemcpyDefault, h->stream) != cudaSuccess))
       rc = SCF_ERR_CUDA;
   } else {
     rc = split ? run_forces(h, spos, vel, acc, com, SCF_MODE_STEP, svel)
@@ -1315,6 +1314,12 @@ int scf_step_host(scf_handle* h, void* pos, void* vel, void* acc, double* com, v
   if ((!host_pos || !host_vel || !host_acc) && h->n_total > 0) return SCF_ERR_NULL_POINTER;
   const bool with_com = h->host.n > 0;
   if (with_com && !host_com) return SCF_ERR_NULL_POINTER;
+  struct Direct {  // for this call
+    scf_handle* h;
+    bool was;
+    explicit Direct(scf_handle* h) : h(h), was(h->bins_off) { h->bins_off = was || host_step_direct(h); }
+    ~Direct() { h->bins_off = was; }
+  } direct(h);
   // Mapped page-locked host memory: the step's kernels read and write the
   // host arrays in place over the host link, so the transfers run inside
   // the kernels, overlapped with their arithmetic (the usual case with
@@ -1427,6 +1432,13 @@ int scf_set_option(scf_handle* h, int option, int value) {
     drop_graph(h);
     return SCF_OK;
   }
+  if (option == SCF_OPT_RADIAL_BINS) {
+    if (value < 0 || value > 2) return SCF_ERR_INVALID_ARG;
+    if (cudaStreamSynchronize(h->stream) != cudaSuccess) return SCF_ERR_CUDA;
+    h->bins_mode = value;
+    drop_graph(h);
+    return SCF_OK;
+  }
   if (option == SCF_OPT_K1_TILE || option == SCF_OPT_K3_BLOCK) {
     if (value != 64 && value != 128 && value != 256 && !(option == SCF_OPT_K3_BLOCK && value == 320))
       return SCF_ERR_INVALID_ARG;
@@ -1464,6 +1476,7 @@ int scf_get_option(const scf_handle* h, int option, int* value) {
   else if (option == SCF_OPT_K3_BLOCK) *value = h->k3.threads;
   else if (option == SCF_OPT_K3_VARIANT) *value = h->k3_ff ? 1 : 0;
   else if (option == SCF_OPT_CENTRE_AHEAD) *value = h->centre_ahead ? 1 : 0;
+  else if (option == SCF_OPT_RADIAL_BINS) *value = h->bins_mode;
   else return SCF_ERR_INVALID_ARG;
   return SCF_OK;
 }
@@ -1577,7 +1590,7 @@ int scf_adjoint_level(scf_handle* h, const void* pos, const double* com, double 
   if (rc != SCF_OK) return rc;
   // 2. own-position term and tidal partials (dual numbers)
   if (binned) {
-    rc = run_binned_k3(h, nullptr, nullptr, host ? com : nullptr, SCF_MODE_ADJ_DUAL, nullptr, 0, 0, &adj);
+    rc = run_binned_k3(h, nullptr, nullptr, host ? com : nullptr, SCF_MODE_ADJ_DUAL, nullptr, &adj);
     if (rc != SCF_OK) return rc;
   } else if (h->k3_blocks > 0) {
     K3Args a = k3_args(h, pos, nullptr, nullptr, host ? com : nullptr, SCF_MODE_ADJ_DUAL);
@@ -1619,7 +1632,7 @@ int scf_adjoint_level(scf_handle* h, const void* pos, const double* com, double 
   }
   if (scf_k2_launch(b, h->stream) != cudaSuccess) return SCF_ERR_CUDA;
   // 5. xbar_k += m_k f(x_k; A^J), then the drift is undone
-  if (binned) return run_binned_k3(h, nullptr, nullptr, nullptr, SCF_MODE_ADJ_J, nullptr, 0, 0, &adj);
+  if (binned) return run_binned_k3(h, nullptr, nullptr, nullptr, SCF_MODE_ADJ_J, nullptr, &adj);
   if (h->k3_blocks > 0) {
     K3Args a = k3_args(h, pos, nullptr, nullptr, nullptr, SCF_MODE_ADJ_J);
     a.adj = adj;
@@ -2093,8 +2106,8 @@ int scf_launches_per_call(const scf_handle* h, int which) {
   // over radial bins: three sorting passes, moments, transform; field rows, field
   const int k1 = bins_k1(h) ? 5 : h->k1_blocks > 0 ? 1 : 0, k3 = bins_k3(h) ? 2 : h->k3_blocks > 0 ? 1 : 0;
   const int sort = bins_k3(h) ? 3 : 0;
-  if (which == 0) return k1 + 1;
-  if (which == 1) return 1 + sort + k3;
+  if (which == 0) return (bins_coeffs(h) ? 5 : h->k1_blocks > 0 ? 1 : 0) + 1;
+  if (which == 1) return 1 + (bins_forces(h) ? 5 : h->k3_blocks > 0 ? 1 : 0);
   if (which == 2) return k1 + 1 + (bins_k1(h) ? 0 : sort) + k3;
   return SCF_ERR_INVALID_ARG;
 }

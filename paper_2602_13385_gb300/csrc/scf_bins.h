@@ -178,12 +178,6 @@ struct BinFieldArgs {
   double dt, alpha, inv_alpha;
   ScfHostParams host;
   unsigned* status;
-  // single precision, a segment of the caller's order: only the particles of
-  // the sorting blocks [seg0, seg1) (seg1 = 0: all)
-  int seg0, seg1;
-  const int* prog_blk_off;
-  const unsigned* hist;
-  const unsigned* total;
   AdjArgs adj;             // modes ADJ_J and ADJ_DUAL (double precision)
 };
 constexpr int kBinField64Threads = 32;

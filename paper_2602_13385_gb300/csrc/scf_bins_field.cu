@@ -293,10 +293,7 @@ __device__ __forceinline__ V4 load_vel(const BinFieldArgs& a, int idx) {
   return v;
 }
 
-// Single precision.  With a segment (seg1 > 0), block (bin, progenitor, part)
-// takes every gridDim.z-th run of the bin's particles from that segment of the
-// caller's order (the step of a host-memory state, whose segments go back while
-// the next one runs); one instantiation, so both forms give the same bits.
+// Single precision.
 template <int L, int NT>
 __global__ void __launch_bounds__(kBinFieldThreads) k_field(BinFieldArgs a) {
   constexpr int ROW = scf_bin_row(L, NT);
@@ -304,32 +301,17 @@ __global__ void __launch_bounds__(kBinFieldThreads) k_field(BinFieldArgs a) {
   __shared__ FieldHost<float> s_h;
   __shared__ int s_bin;
   const int tid = threadIdx.x, K = a.K;
-  int prog, bin;
-  unsigned k0, k1, stride;  // sorted particles of this block, from the progenitor's first
-  if (a.seg1 > 0) {
-    prog = blockIdx.y;
-    bin = blockIdx.x;
-    const int b0 = max(a.seg0, a.prog_blk_off[prog]), bn = a.prog_blk_off[prog + 1], b1 = min(a.seg1, bn);
-    if (b0 >= b1) return;
-    const unsigned first = a.bin_start[(size_t)prog * (K + 1) + bin];
-    k0 = first + a.hist[(size_t)b0 * K + bin] + blockIdx.z * kBinFieldThreads;
-    k1 = first + (b1 == bn ? a.total[(size_t)prog * K + bin] : a.hist[(size_t)b1 * K + bin]);
-    stride = gridDim.z * kBinFieldThreads;
-    if (k0 >= k1) return;
-  } else {
-    prog = a.blk_prog[blockIdx.x];
-    const unsigned task = (unsigned)a.blk_task[blockIdx.x];
-    const unsigned* fs = a.field_start + (size_t)prog * (K + 1);
-    if (task >= fs[K]) return;
-    for (int i = tid; i < K; i += kBinFieldThreads)  // the bin with fs[bin] <= task < fs[bin + 1]
-      if (fs[i] <= task && task < fs[i + 1]) s_bin = i;
-    __syncthreads();
-    bin = s_bin;
-    const unsigned* bs = a.bin_start + (size_t)prog * (K + 1);
-    k0 = bs[bin] + (task - fs[bin]) * kBinFieldTask;
-    k1 = min(bs[bin + 1], k0 + kBinFieldTask);
-    stride = kBinFieldThreads;
-  }
+  const int prog = a.blk_prog[blockIdx.x];
+  const unsigned task = (unsigned)a.blk_task[blockIdx.x];
+  const unsigned* fs = a.field_start + (size_t)prog * (K + 1);
+  if (task >= fs[K]) return;
+  for (int i = tid; i < K; i += kBinFieldThreads)  // the bin with fs[bin] <= task < fs[bin + 1]
+    if (fs[i] <= task && task < fs[i + 1]) s_bin = i;
+  __syncthreads();
+  const int bin = s_bin;
+  const unsigned* bs = a.bin_start + (size_t)prog * (K + 1);
+  // sorted particles of this block, from the progenitor's first
+  const unsigned k0 = bs[bin] + (task - fs[bin]) * kBinFieldTask, k1 = min(bs[bin + 1], k0 + kBinFieldTask);
   const float4* row = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(a.P) + ((size_t)prog * K + bin) * ROW);
   for (int i = tid; i < ROW / 4; i += kBinFieldThreads) reinterpret_cast<float4*>(s_row)[i] = row[i];
   const bool has_host = a.host.n > 0 && a.com != nullptr;
@@ -358,7 +340,7 @@ __global__ void __launch_bounds__(kBinFieldThreads) k_field(BinFieldArgs a) {
   __syncthreads();
   while (k < k1) {
     field_of<float, L, NT>(a, pos, idx, frame, s_row, s_h.binv, has_host, s_h, vel);
-    k += stride;
+    k += kBinFieldThreads;
     if (k < k1) {
       pos = rec[k].p;
       idx = rec[k].key.x;
@@ -393,8 +375,6 @@ template <typename T, int L, int NT>
 cudaError_t launch(const BinFieldArgs& a, int blocks, cudaStream_t s) {
   if constexpr (sizeof(T) == 8) {
     k_field64<L, NT><<<blocks, kBinField64Threads, 0, s>>>(a);
-  } else if (a.seg1 > 0) {
-    k_field<L, NT><<<dim3(a.K, a.n_prog, 4), kBinFieldThreads, 0, s>>>(a);
   } else {
     k_field<L, NT><<<blocks, kBinFieldThreads, 0, s>>>(a);
   }

@@ -27,6 +27,13 @@ def scf():
     return m
 
 
+def every_pass(sim):
+    """Radial bins in every pass, also where the direct kernels are the faster ones."""
+    from paper_2602_13385_gb300 import _lib
+    _lib.scf_set_option(sim._h, _lib.SCF_OPT_RADIAL_BINS, 2)
+    return sim
+
+
 def sample(n, seed, dtype):
     """A wide sample: core, halo far beyond the basis scale, and the special places."""
     g = np.random.default_rng(seed)
@@ -92,7 +99,7 @@ def test_bins_against_direct_kernels(scf, prec, nmax, lmax, alpha, offsets):
                        dtype=torch.float64)
     pos = sample(n, 3, cfg.dtype)
     mask = (torch.arange(n, device="cuda") % 7 != 0).to(torch.uint8)
-    sim = scf.SCF(cfg, offsets=offsets, b_per_prog=b)
+    sim = every_pass(scf.SCF(cfg, offsets=offsets, b_per_prog=b))
     assert sim.launches_per_call("coeffs") > 2, "the sample should be over the size rule"
     A = sim.coeffs(pos, mask=mask)
     assert torch.equal(A, sim.coeffs(pos, mask=mask))                  # fixed order
@@ -127,7 +134,7 @@ def test_bins_nonfinite_particles_are_left_out_and_flagged(scf, prec, n):
     bad[17, 0], bad[n - 1, 2], bad[4000, 3] = float("nan"), float("inf"), float("nan")
     good = pos.clone()
     good[[17, n - 1, 4000], 3] = 0.0
-    sim = scf.SCF(cfg, n=n)
+    sim = every_pass(scf.SCF(cfg, n=n))
     A = sim.coeffs(good)
     assert sim.status() == (0, 0)
     B = sim.coeffs(bad)
@@ -150,7 +157,7 @@ def test_bins_step_is_the_same_through_graph_plain_and_host_memory(scf, prec, n)
     for form in ("graph", "plain", "mapped", "staged"):
         s = torch.cuda.Stream()
         with torch.cuda.stream(s):
-            sim = scf.SCF(cfg, n=n)
+            sim = every_pass(scf.SCF(cfg, n=n))
             p, v, c = pos0.clone(), vel0.clone(), com0.clone()
             a = sim.forces(p, sim.coeffs(p), com=c)
             if form in ("graph", "plain"):
@@ -170,3 +177,31 @@ def test_bins_step_is_the_same_through_graph_plain_and_host_memory(scf, prec, n)
     for other in got[1:]:
         for x, y in zip(got[0], other):
             assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("prec,nmax,lmax,offsets", [("mixed", 10, 5, [0, 300001]), ("mixed", 20, 10, [0, 300001]),
+                                                    ("fp64", 10, 5, [0, 20000]), ("fp64", 20, 8, [0, 30001])])
+def test_passes_alone_and_host_steps_by_their_own_size_rules(scf, prec, nmax, lmax, offsets):
+    """Default handles against bins in every pass and none: the same results whatever each pass runs over."""
+    from paper_2602_13385_gb300 import _lib
+    cfg = scf.Config(nmax=nmax, lmax=lmax, b=0.7, precision=prec)
+    n = offsets[-1]
+    pos0 = sample(n, 8, cfg.dtype)
+    pos0[n // 2 + 2, :3] = 1.0
+    vel0 = torch.zeros_like(pos0)
+    got = []
+    for mode in (1, 0, 2):
+        sim = scf.SCF(cfg, offsets=offsets)
+        _lib.scf_set_option(sim._h, _lib.SCF_OPT_RADIAL_BINS, mode)
+        assert _lib.scf_get_option(sim._h, _lib.SCF_OPT_RADIAL_BINS) == mode
+        A = sim.coeffs(pos0)
+        acc = sim.forces(pos0, A)
+        h = [t.cpu().pin_memory() for t in (pos0, vel0, acc)]
+        d = [t.clone() for t in (pos0, vel0, acc)]
+        sim.step_host(*d, *h)
+        torch.cuda.synchronize()
+        assert sim.status() == (0, 0)
+        got.append([bi_orthonormal(A, nmax, lmax, 1.0), acc[:, :3]] + [t[:, :3] for t in h])
+    for other in got[1:]:
+        for x, y in zip(got[0], other):
+            assert ((x - y).abs().max() / y.abs().max()).item() < 2 * TOL[prec]
