@@ -91,6 +91,19 @@ def per_particle_flops(nmax, lmax):
     return k1, k3
 
 
+def per_particle_flops_binned(nmax, lmax, precision, n_per_prog):
+    """The same over radial bins: T polynomial terms in place of the nmax + 1
+    radial orders (coefficients: T FMAs per angular column; field: value and
+    derivative of two polynomials per (l, m >= 1) and one per degree, four pairs
+    of sums)."""
+    T = (6 if n_per_prog >= 400000 else 8) if precision == "mixed" else (8 if n_per_prog >= 50000 else 10)
+    nl = lmax + 1
+    nlm = nl * (nl + 1) // 2
+    k1 = 2 * T * nl * nl + 16 * nlm + 40
+    k3 = (nlm - nl) * (4 * (2 * T - 3) + 24) + nl * (2 * (2 * T - 3) + 14) + 100
+    return k1, k3
+
+
 def per_particle_bytes(elem):
     """Algorithmic HBM bytes per particle per step (4-component records)."""
     rec = 4 * elem
@@ -347,13 +360,13 @@ def workload_config(wl, precision, name):
 
 
 # --------------------------------------------------------------------- our arm
-# Pair terms of the boundedness sum on the FP32 pipe.  Single precision:
-# dx, dy, dz (3 adds), r^2 (1 multiply + 2 FMAs) and m / r accumulated
-# (1 FMA) = 7 operations; 1/sqrt runs on the special-function unit.  Double
-# precision runs the same terms in float-float arithmetic: 86 single-precision
-# operations per pair (exact differences, squares with their rounding errors,
-# a Newton step for 1/r, a float-float accumulation).
-PAIR_OPS = {"mixed": 7, "fp64": 86}
+# Pair terms of the boundedness sum on the FP32 pipe, per ordered pair: every
+# unordered pair is evaluated once for both of its particles.  Single precision:
+# dx, dy, dz (3 adds), r^2 (1 multiply + 2 FMAs) and two m / r accumulated
+# (2 FMAs) = 8 operations; 1/sqrt runs on the special-function unit.  Double
+# precision runs the same terms in float-float arithmetic: 98 operations an
+# unordered pair (24 the separation, 37 r^2, 13 1/r, 24 the two m / r sums).
+PAIR_OPS = {"mixed": 4, "fp64": 49}
 
 
 def escape_timing(sim, p, v, offsets, precision, clocks, torch, reps=3):
@@ -555,7 +568,9 @@ def run_line(name, args, steps, torch, barrier, world, rank, local, peaks, oracl
                    "the kernels read it from host memory and write the new state back over the host link"}
 
     # roofline: ALU-bound (FP64 pipe in fp64 mode, FP32 pipe in mixed mode)
-    k1f, k3f = per_particle_flops(wl.nmax, wl.lmax)
+    binned = sim.launches_per_call("step") > 3
+    k1f, k3f = (per_particle_flops_binned(wl.nmax, wl.lmax, precision, wl.n // (len(offsets) - 1)) if binned
+                else per_particle_flops(wl.nmax, wl.lmax))
     elem = 8 if precision == "fp64" else 4
     k1b, k3b = per_particle_bytes(elem)
     per_k = [kms[i] / max(1, kcount[i]) for i in range(3)]
@@ -568,7 +583,10 @@ def run_line(name, args, steps, torch, barrier, world, rank, local, peaks, oracl
     fma = FP64_FMA_PER_SM_CLK if is64 else FP32_FMA_PER_SM_CLK
     peak = N_SM * fma * 2 * clock * 1e6 / 1e12
     meas = peaks.get("fp64_tflops" if is64 else "fp32_tflops") if peaks else None
-    kname = "k3_forces" if dom == 2 else "k1_partials"
+    if binned:  # each pass's events span its sort and table kernels too
+        kname = "k_field (radial bins)" if dom == 2 else "k_bin_sort + k_moments + k_transform (radial bins)"
+    else:
+        kname = "k3_forces" if dom == 2 else "k1_partials"
     step_flops = wl.n * (k1f + k3f)
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                 "traffic": traffic_for(kname, name),
@@ -598,9 +616,9 @@ def run_line(name, args, steps, torch, barrier, world, rank, local, peaks, oracl
         "data": "synthetic (seeded sample, see config.workload)",
         "config": workload_config(wl, precision, name),
         "roofline": roofline, "e2e": e2e,
-        # the step kernels of the timed pass (3 per step), plus the centre step
-        # computed ahead on the side stream when there is a host
-        "gpu_launches": int(sum(kcount)) * (4 if use_com is not None else 3) // 3, "clocks": clocks,
+        # the step kernels of the timed pass, plus the centre step computed ahead
+        # on the side stream when there is a host
+        "gpu_launches": steps * (sim.launches_per_call("step") + (use_com is not None)), "clocks": clocks,
         "kernel_shapes": dict(sim.tiles(), autotuned=tuning is not None,
                               candidates_ms=None if tuning is None else tuning["ms"]),
         "src_hash": src_hash(),

@@ -52,7 +52,7 @@
  * Radial bins.  A handle with enough particles for its (nmax, lmax) runs its
  * coefficient and field passes (alone, from a larger size) over particles sorted by
  * radius, with the radial polynomials of each radius bin replaced by
- * interpolants exact to the precision's rounding (workspace of about 40 bytes
+ * interpolants exact to the precision's rounding (workspace of about 40 to 50 bytes
  * a particle and the bins' tables; without the memory for it the handle keeps
  * the direct kernels).  The block shapes below are those of the direct
  * kernels; selecting a float-float variant, or the one-thread-per-output

@@ -866,7 +866,10 @@ int bin_init(scf_handle* h) {
   ScfBinShape s = bin_shape(c, std::max(c.alpha, 2.0), large);
   h->bin_kcap = s.K;
   s.chunk = h->n_total < 400 * (int64_t)h->n_sm ? 512 : h->n_total < 1600 * (int64_t)h->n_sm ? 1024 : 2048;
-  s.task = h->n_total < 300000 ? (f32 ? 256 : 128) : (f32 ? 512 : 256);
+  // a moment task is one block: with few particles an SM that draws two long tasks sets the time ((20,8) double,
+  // 20k particles: moments 96, 70, 92 us with tasks of 128, 64, 32 and 12k 90, 54, 48; an adjoint run of 20k 9.65, 8.37,
+  // 8.56 ms); larger samples have blocks enough, and fewer rows to transform
+  s.task = h->n_total < 50000 ? (f32 ? 256 : 64) : h->n_total < 300000 ? (f32 ? 256 : 128) : (f32 ? 512 : 256);
   s.groups = std::max(1, std::min(s.K, h->n_sm / h->n_prog));
   const Map3 sm = make_map3(h->offsets, h->n_prog, s.chunk);
   Map3 fm = make_map3(h->offsets, h->n_prog, kBinField64Threads);  // double precision
