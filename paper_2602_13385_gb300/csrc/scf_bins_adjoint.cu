@@ -8,6 +8,9 @@
 // coordinate tau, which needs no dual arithmetic: with z0, z1 and z2 the
 // polynomial, its derivative and half its second derivative, the dual numbers of
 // the sum and of its derivative are (z0, z1 tau.d) and (z1, 2 z2 tau.d).
+// King N = 20000 (20,8), GB300: field 265 us, moments 201 us (62% and 47% of the
+// FP64 pipe: four or five warps an SM); a run of four steps forward and backward
+// 15.3 ms with the direct dual passes, 8.3 ms with these.
 #include <type_traits>
 
 #include "scf_adjoint.cuh"
