@@ -18,11 +18,28 @@ template <typename T> struct V4of;
 template <> struct V4of<double> { using type = ScfD4; };
 template <> struct V4of<float> { using type = float4; };
 
-// Bin of a particle: theta = acos(xi) = 2 atan(1 / sqrt(t)), t = s^(1/alpha).
-// Always in single precision (it only selects the polynomial piece; rounding at
-// an edge moves |tau| past 1 by less than 1e-3).
-__device__ __forceinline__ int bin_of(float x, float y, float z, float binv, float inv_alpha, int K) {
-  const float s = sqrtf(x * x + y * y + z * z) * binv;
+// Bin of a particle: theta = acos(xi) = 2 atan(1 / sqrt(t)), t = s^(1/alpha), s = r / b.
+// In single precision (it only selects the polynomial piece; where rounding moves a
+// particle across an edge, |tau| ends a little above 1), but a double-precision handle's
+// units are the caller's: the position is divided by b in double, and the square is
+// formed from components scaled by a power of two where it would leave the float range
+// (at large alpha s = 1e25 is still bins away from the outermost one).
+__device__ __forceinline__ float radius_of(float x, float y, float z, float binv) {
+  return sqrtf(x * x + y * y + z * z) * binv;  // as the moments and the field form it
+}
+__device__ __forceinline__ float radius_of(double x, double y, double z, double binv) {
+  float u = (float)(x * binv), v = (float)(y * binv), w = (float)(z * binv);
+  const float top = fmaxf(fabsf(u), fmaxf(fabsf(v), fabsf(w)));
+  const float up = top > 1e18f ? 0x1p-64f : top < 1e-18f ? 0x1p64f : 1.f;
+  const float down = top > 1e18f ? 0x1p64f : top < 1e-18f ? 0x1p-64f : 1.f;
+  u *= up;
+  v *= up;
+  w *= up;
+  return sqrtf(u * u + v * v + w * w) * down;
+}
+template <typename T>
+__device__ __forceinline__ int bin_of(T x, T y, T z, T binv, float inv_alpha, int K) {
+  const float s = radius_of(x, y, z, binv);
   const float t = inv_alpha == 1.f ? s : powf(s, inv_alpha);
   const float th = 2.f * atan2f(1.f, sqrtf(t));
   return min(max((int)(th * ((float)K * 0.318309886f)), 0), K - 1);
@@ -41,8 +58,8 @@ __global__ void __launch_bounds__(kBinSortThreads) k_bin_count(BinArgs a) {
   unsigned short* cnt = reinterpret_cast<unsigned short*>(smem_u);  // [warps][K]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, blk = blockIdx.x, K = a.K;
   for (int i = tid; i < kBinWarps * K / 2; i += kBinSortThreads) smem_u[i] = 0;
-  __shared__ float s_b;
-  if (tid == 0) s_b = 1.f / (float)a.b_prog[a.blk_prog[blk]];
+  __shared__ T s_b;
+  if (tid == 0) s_b = (T)(1.0 / a.b_prog[a.blk_prog[blk]]);
   const float ia = a.inv_alphaf;
   const int64_t k0 = a.blk_begin[blk] + warp * (32 * J) + lane, k1 = a.blk_end[blk];
   V4* pos = reinterpret_cast<V4*>(a.pos);
@@ -75,7 +92,7 @@ __global__ void __launch_bounds__(kBinSortThreads) k_bin_count(BinArgs a) {
       }
   }
   __syncthreads();
-  const float binv = s_b;
+  const T binv = s_b;
   unsigned short* c = cnt + warp * K;
   int bin[J], place[J];
 #pragma unroll
@@ -84,7 +101,7 @@ __global__ void __launch_bounds__(kBinSortThreads) k_bin_count(BinArgs a) {
     bin[j] = K;
     if (on) {
       const bool fin = scf_finite3(p[j].x, p[j].y, p[j].z);
-      bin[j] = fin ? bin_of((float)p[j].x, (float)p[j].y, (float)p[j].z, binv, ia, K) : 0;
+      bin[j] = fin ? bin_of<T>(p[j].x, p[j].y, p[j].z, binv, ia, K) : 0;
       if (a.count_status && !(fin && isfinite(p[j].w))) atomicOr(a.status, 1u);
     }
   }
