@@ -20,6 +20,7 @@ struct scf_handle {
   int n_prog = 0;
   int device = 0;
   cudaStream_t stream = nullptr;
+  cudaStream_t setup = nullptr;          // where put, clear and the tables go: stream (see scf_init)
   int nlm = 0, nc = 0;
   int64_t n_total = 0;
   int n_sm = 0;
@@ -187,6 +188,7 @@ int upload_tables_once(int device) {
   delete t;
   if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess || e4 != cudaSuccess || e5 != cudaSuccess)
     return SCF_ERR_CUDA;
+  if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) return SCF_ERR_CUDA;  // landed before any stream reads them
   g_const_ready[device] = true;
   return SCF_OK;
 }
@@ -661,8 +663,15 @@ Map3 make_map3(const std::vector<int64_t>& off, int n_prog, int64_t tb) {
   return m;
 }
 
-bool put(void* dst, const void* src, size_t bytes) {
-  return bytes == 0 || cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
+// Uploads and clears in the order of the kernels that read them (h->setup): a copy
+// from pageable memory or a memset on the legacy stream may still be under way when
+// the call returns, and a non-blocking stream does not wait for it.  (src is staged
+// before the call returns.)
+bool put(const scf_handle* h, void* dst, const void* src, size_t bytes) {
+  return bytes == 0 || cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, h->setup) == cudaSuccess;
+}
+bool clear(const scf_handle* h, void* dst, int value, size_t bytes) {
+  return bytes == 0 || cudaMemsetAsync(dst, value, bytes, h->setup) == cudaSuccess;
 }
 
 // Kernel 3's single-precision radial steps of the family in t, one float4
@@ -674,7 +683,7 @@ bool put_steps(scf_handle* h, const ScfConst& t) {
   for (int l = 0; l <= h->cfg.lmax; ++l)
     for (int n = 0; n < nn; ++n)
       cs[(size_t)l * nn + n] = make_float4(t.gbetaf[l][n], t.hbetaf[l][n], t.hratiof[l][n], 0.f);
-  return put(h->d_cs, cs.data(), sizeof(float4) * cs.size());
+  return put(h, h->d_cs, cs.data(), sizeof(float4) * cs.size());
 }
 
 // Kernel 1 launch shape: the simple kernel with a particle tile of 64, 128
@@ -724,10 +733,10 @@ int use_k1(scf_handle* h, int tp) {
   Map1 m = make_map1(h->offsets, h->n_prog, info.tile, (int64_t)h->n_sm * bps);
   if (info.variant == 1) info.win = scf_k1_windows(longest_block(m), info);
   if (m.prog.size() > h->cap_blk1 || k1_rows(info, m.prog.size()) > h->cap_rows) return SCF_ERR_UNSUPPORTED;
-  bool ok = put(h->d_blk1_prog, m.prog.data(), sizeof(int) * m.prog.size()) &&
-            put(h->d_blk1_begin, m.begin.data(), sizeof(int64_t) * m.begin.size()) &&
-            put(h->d_blk1_end, m.end.data(), sizeof(int64_t) * m.end.size()) &&
-            put(h->d_prog_blk_off, m.prog_off.data(), sizeof(int) * m.prog_off.size());
+  bool ok = put(h, h->d_blk1_prog, m.prog.data(), sizeof(int) * m.prog.size()) &&
+            put(h, h->d_blk1_begin, m.begin.data(), sizeof(int64_t) * m.begin.size()) &&
+            put(h, h->d_blk1_end, m.end.data(), sizeof(int64_t) * m.end.size()) &&
+            put(h, h->d_prog_blk_off, m.prog_off.data(), sizeof(int) * m.prog_off.size());
   if (!ok) return SCF_ERR_CUDA;
   h->k1 = info;
   h->k1_blocks = (int)m.prog.size();
@@ -756,9 +765,9 @@ int use_k3(scf_handle* h, int tb) {
   }
   Map3 m = make_map3(h->offsets, h->n_prog, info.tile);
   if (m.prog.size() > h->cap_blk3) return SCF_ERR_UNSUPPORTED;
-  bool ok = put(h->d_blk3_prog, m.prog.data(), sizeof(int) * m.prog.size()) &&
-            put(h->d_blk3_begin, m.begin.data(), sizeof(int64_t) * m.begin.size()) &&
-            put(h->d_blk3_end, m.end.data(), sizeof(int64_t) * m.end.size());
+  bool ok = put(h, h->d_blk3_prog, m.prog.data(), sizeof(int) * m.prog.size()) &&
+            put(h, h->d_blk3_begin, m.begin.data(), sizeof(int64_t) * m.begin.size()) &&
+            put(h, h->d_blk3_end, m.end.data(), sizeof(int64_t) * m.end.size());
   if (!ok) return SCF_ERR_CUDA;
   h->k3 = info;
   h->k3_native = native;
@@ -833,7 +842,7 @@ bool bin_tables(scf_handle* h) {
   double* gs = aux.data() + 2 * nd + 2 * nd * nd;
   for (int l = 0; l <= c.lmax; ++l)
     for (int n = 0; n < nn; ++n) gs[l * nn + n] = t->gscale[l][n];
-  if (!put(h->d_bin_aux, aux.data(), sizeof(double) * aux.size())) return false;
+  if (!put(h, h->d_bin_aux, aux.data(), sizeof(double) * aux.size())) return false;
   BinTableArgs a{};
   a.K = s.K;
   a.T = s.T;
@@ -848,7 +857,7 @@ bool bin_tables(scf_handle* h) {
   a.t = h->d_bin_t;
   a.tf = h->d_bin_tf;
   a.t2 = h->d_bin_t2;
-  if (scf_bin_table_launch(a, h->stream) != cudaSuccess) return false;
+  if (scf_bin_table_launch(a, h->setup) != cudaSuccess) return false;
   h->binned = true;
   drop_graph(h);
   return true;
@@ -940,18 +949,18 @@ int bin_init(scf_handle* h) {
   h->bin_blocks = (int)nsb;
   h->bin_mblocks = (int)mb_prog.size();
   h->bin_fblocks = (int)nfb;
-  const bool ok = put(h->d_sb_prog, sm.prog.data(), 4 * nsb) && put(h->d_sb_begin, sm.begin.data(), 8 * nsb) &&
-                  put(h->d_sb_end, sm.end.data(), 8 * nsb) && put(h->d_sb_off, sb_off.data(), 4 * (np + 1)) &&
-                  put(h->d_fb_prog, fm.prog.data(), 4 * nfb) && put(h->d_mb_prog, mb_prog.data(), 4 * mb_prog.size()) &&
-                  (f32 ? put(h->d_fb_task, fb_task.data(), 4 * nfb)
-                       : put(h->d_fb_begin, fm.begin.data(), 8 * nfb) && put(h->d_fb_end, fm.end.data(), 8 * nfb)) &&
-                  put(h->d_mb_task, mb_task.data(), 4 * mb_task.size()) && put(h->d_mrow_off, mrow.data(), 8 * np) &&
-                  put(h->d_bin_rows_off, rows_off.data(), 4 * (np + 1));
+  const bool ok = put(h, h->d_sb_prog, sm.prog.data(), 4 * nsb) && put(h, h->d_sb_begin, sm.begin.data(), 8 * nsb) &&
+                  put(h, h->d_sb_end, sm.end.data(), 8 * nsb) && put(h, h->d_sb_off, sb_off.data(), 4 * (np + 1)) &&
+                  put(h, h->d_fb_prog, fm.prog.data(), 4 * nfb) && put(h, h->d_mb_prog, mb_prog.data(), 4 * mb_prog.size()) &&
+                  (f32 ? put(h, h->d_fb_task, fb_task.data(), 4 * nfb)
+                       : put(h, h->d_fb_begin, fm.begin.data(), 8 * nfb) && put(h, h->d_fb_end, fm.end.data(), 8 * nfb)) &&
+                  put(h, h->d_mb_task, mb_task.data(), 4 * mb_task.size()) && put(h, h->d_mrow_off, mrow.data(), 8 * np) &&
+                  put(h, h->d_bin_rows_off, rows_off.data(), 4 * (np + 1));
   // a progenitor without particles has no sorting block to write its (empty) bins
-  return ok && cudaMemset(h->d_bin_start, 0, 4 * np * (K + 1)) == cudaSuccess &&
-                 cudaMemset(h->d_task_start, 0, 4 * np * (K + 1)) == cudaSuccess &&
-                 cudaMemset(h->d_field_start, 0, 4 * np * (K + 1)) == cudaSuccess &&
-                 cudaMemset(h->d_bin_ticket, 0, 4 * np) == cudaSuccess
+  return ok && clear(h, h->d_bin_start, 0, 4 * np * (K + 1)) &&
+                 clear(h, h->d_task_start, 0, 4 * np * (K + 1)) &&
+                 clear(h, h->d_field_start, 0, 4 * np * (K + 1)) &&
+                 clear(h, h->d_bin_ticket, 0, 4 * np)
              ? SCF_OK
              : SCF_ERR_CUDA;
 }
@@ -978,7 +987,11 @@ int scf_init(const scf_config* cfg, int n_prog, const int64_t* offsets, const do
   if (!h) return SCF_ERR_OUT_OF_MEMORY;
   h->cfg = *cfg;
   h->n_prog = n_prog;
-  h->stream = reinterpret_cast<cudaStream_t>(stream);
+  h->stream = h->setup = reinterpret_cast<cudaStream_t>(stream);
+  // a stream under capture would take the uploads into its graph: they go by the legacy stream, waited for below
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess) cudaGetLastError();
+  else if (cap != cudaStreamCaptureStatusNone) h->setup = cudaStreamLegacy;
   h->nlm = (cfg->lmax + 1) * (cfg->lmax + 2) / 2;
   h->nc = (cfg->nmax + 1) * h->nlm;
   h->n_total = offsets[n_prog];
@@ -1122,7 +1135,7 @@ int scf_init(const scf_config* cfg, int n_prog, const int64_t* offsets, const do
     scf_make_const(t.get(), cfg->alpha);
     if (h->gen && !tables_finite(*t, cfg->lmax, cfg->nmax, cfg->precision == SCF_MIXED))
       return fail(SCF_ERR_UNSUPPORTED);
-    if (h->gen && !put(h->d_tab, t.get(), sizeof(ScfConst))) return fail(SCF_ERR_CUDA);
+    if (h->gen && !put(h, h->d_tab, t.get(), sizeof(ScfConst))) return fail(SCF_ERR_CUDA);
     if (!put_steps(h, *t)) return fail(SCF_ERR_CUDA);
   }
   std::vector<double> norm(2 * (size_t)h->nc), ksc(2 * (size_t)h->nc);
@@ -1131,14 +1144,14 @@ int scf_init(const scf_config* cfg, int n_prog, const int64_t* offsets, const do
   for (double x : norm)
     if (!std::isfinite(x)) return fail(SCF_ERR_UNSUPPORTED);
   std::vector<float> ksc_f(ksc.begin(), ksc.end());
-  const bool ksc_ok = cfg->precision == SCF_MIXED ? put(h->d_kscale, ksc_f.data(), sizeof(float) * ksc_f.size())
-                                                  : put(h->d_kscale, ksc.data(), sizeof(double) * ksc.size());
-  bool ok = ksc_ok && put(h->d_norm, norm.data(), sizeof(double) * norm.size()) &&
-            put(h->d_b, bs.data(), sizeof(double) * n_prog) &&
-            put(h->d_off, h->offsets.data(), sizeof(int64_t) * (n_prog + 1)) &&
-            cudaMemset(h->d_status, 0, sizeof(unsigned) * 4) == cudaSuccess &&
-            cudaMemset(h->d_cnext, 0xff, sizeof(double) * kCentreW * (size_t)n_prog) == cudaSuccess &&  // NaN keys
-            cudaMemset(h->d_A, 0, sizeof(double) * 2 * (size_t)h->nc * n_prog) == cudaSuccess;
+  const bool ksc_ok = cfg->precision == SCF_MIXED ? put(h, h->d_kscale, ksc_f.data(), sizeof(float) * ksc_f.size())
+                                                  : put(h, h->d_kscale, ksc.data(), sizeof(double) * ksc.size());
+  bool ok = ksc_ok && put(h, h->d_norm, norm.data(), sizeof(double) * norm.size()) &&
+            put(h, h->d_b, bs.data(), sizeof(double) * n_prog) &&
+            put(h, h->d_off, h->offsets.data(), sizeof(int64_t) * (n_prog + 1)) &&
+            clear(h, h->d_status, 0, sizeof(unsigned) * 4) &&
+            clear(h, h->d_cnext, 0xff, sizeof(double) * kCentreW * (size_t)n_prog) &&  // NaN keys
+            clear(h, h->d_A, 0, sizeof(double) * 2 * (size_t)h->nc * n_prog);
   if (!ok) return fail(SCF_ERR_CUDA);
   // default shapes: the register-tiled kernel 1 in mixed precision (128-particle
   // tiles of the simple kernel in double precision) and 128-thread kernel 3
@@ -1149,6 +1162,8 @@ int scf_init(const scf_config* cfg, int n_prog, const int64_t* offsets, const do
   rc = use_k3(h, 128);
   if (rc != SCF_OK) return fail(rc);
   bin_tables(h);
+  if (h->setup != h->stream && cudaStreamSynchronize(h->setup) != cudaSuccess) return fail(SCF_ERR_CUDA);
+  h->setup = h->stream;
   *out = h;
   return SCF_OK;
 }
@@ -1932,7 +1947,7 @@ int set_alpha(scf_handle* h, double alpha) {
     scf_make_const(t.get(), alpha);
     if (gen && !tables_finite(*t, h->cfg.lmax, h->cfg.nmax, h->cfg.precision == SCF_MIXED))
       return SCF_ERR_UNSUPPORTED;
-    if (gen && !put(h->d_tab, t.get(), sizeof(ScfConst))) return SCF_ERR_CUDA;
+    if (gen && !put(h, h->d_tab, t.get(), sizeof(ScfConst))) return SCF_ERR_CUDA;
     if (!put_steps(h, *t)) return SCF_ERR_CUDA;
   }
   std::vector<double> norm(2 * (size_t)h->nc), ksc(2 * (size_t)h->nc);
@@ -1941,9 +1956,9 @@ int set_alpha(scf_handle* h, double alpha) {
   for (double x : norm)
     if (!std::isfinite(x)) return SCF_ERR_UNSUPPORTED;
   std::vector<float> ksc_f(ksc.begin(), ksc.end());
-  const bool ok = (h->cfg.precision == SCF_MIXED ? put(h->d_kscale, ksc_f.data(), sizeof(float) * ksc_f.size())
-                                                 : put(h->d_kscale, ksc.data(), sizeof(double) * ksc.size())) &&
-                  put(h->d_norm, norm.data(), sizeof(double) * norm.size());
+  const bool ok = (h->cfg.precision == SCF_MIXED ? put(h, h->d_kscale, ksc_f.data(), sizeof(float) * ksc_f.size())
+                                                 : put(h, h->d_kscale, ksc.data(), sizeof(double) * ksc.size())) &&
+                  put(h, h->d_norm, norm.data(), sizeof(double) * norm.size());
   if (!ok) return SCF_ERR_CUDA;
   h->cfg.alpha = alpha;
   h->gen = gen;
@@ -1989,7 +2004,7 @@ int scf_retune_alpha(scf_handle* h, const void* pos, const uint8_t* mask, double
   // b search and one pass of sums; `live` counts progenitors with a set
   int live = 0;
   auto eval = [&](double al, double* H, double* dH, std::vector<double>* bs) -> int {
-    if (!put(d_bt, b0.data(), sizeof(double) * P)) return SCF_ERR_CUDA;
+    if (!put(h, d_bt, b0.data(), sizeof(double) * P)) return SCF_ERR_CUDA;
     a.b_prog = d_bt;
     a.alpha = al;
     a.inv_alpha = 1.0 / al;
@@ -2070,7 +2085,7 @@ int scf_retune_alpha(scf_handle* h, const void* pos, const uint8_t* mask, double
   }
   for (int p = 0; p < P; ++p)
     if (!(bs[p] > 0.0) || !std::isfinite(bs[p])) bs[p] = b0[p];
-  if (!put(h->d_b, bs.data(), sizeof(double) * P)) return SCF_ERR_CUDA;
+  if (!put(h, h->d_b, bs.data(), sizeof(double) * P)) return SCF_ERR_CUDA;
   if (alpha_out) *alpha_out = alpha;
   return SCF_OK;
 }

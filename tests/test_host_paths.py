@@ -1,0 +1,92 @@
+"""The library's host code without a GPU: what it allocates, uploads, launches
+and captures, on the fake runtime of fake_cuda.py."""
+import ctypes
+
+import pytest
+
+import fake_cuda
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    return fake_cuda.load(tmp_path_factory.mktemp("fake"))
+
+
+STREAM = 0x1234
+
+
+class Handle:
+    def __init__(self, fake, n, nmax=20, lmax=10, precision="fp64", alpha=1.0, stream=STREAM, limit=0, offsets=None):
+        from paper_2602_13385_gb300 import _lib
+        c = _lib.scf_config()
+        c.nmax, c.lmax, c.alpha, c.b, c.G, c.dt = nmax, lmax, alpha, 0.7, 1.0, 0.01
+        c.precision = {"fp64": _lib.SCF_FP64, "mixed": _lib.SCF_MIXED}[precision]
+        offsets = [0, n] if offsets is None else offsets
+        self.lib, self.h = fake.lib, ctypes.c_void_p()
+        fake.reset(limit)
+        self.rc = fake.lib.scf_init(ctypes.byref(c), len(offsets) - 1, (ctypes.c_int64 * len(offsets))(*offsets), None,
+                                    ctypes.c_void_p(stream), ctypes.byref(self.h))
+
+    def binned(self):
+        return self.lib.scf_launches_per_call(self.h, 2) > 4
+
+    def call(self, name, *args):
+        return getattr(self.lib, name)(self.h, *args)
+
+    def __enter__(self):
+        return self
+
+    def __exit__(self, *a):
+        if self.h:
+            self.lib.scf_free(self.h)
+
+
+def test_the_fake_runtime_sees_a_step(fake):
+    with Handle(fake, 20000) as h:
+        assert h.rc == 0 and h.binned()
+        fake.reset()
+        assert h.call("scf_step", 0x1000, 0x2000, 0x3000, None, 2) == 0
+        log = fake.log()
+        assert log.count(f"graph_launch {hex(STREAM)}") == 2
+        assert sum("k_moments" in x for x in fake.launches()) == 1
+    assert fake.used() == 0
+
+
+def unordered_uploads(log, stream):
+    """Uploads and clears that a launch on ``stream`` may overtake."""
+    pending, bad = 0, []
+    for x in log:
+        w = x.split()
+        if w[0] in ("copy", "copy_symbol", "memset") or w[0] in ("copy_async", "memset_async") and w[2] != hex(stream):
+            pending += 1
+        elif w[0] == "synchronize" and w[1] == "0x1":  # the legacy stream
+            pending = 0
+        elif w[0] == "launch" and pending:
+            bad.append(x)
+    return bad, pending
+
+
+@pytest.mark.parametrize("precision,n,alpha", [("fp64", 20000, 1.0), ("fp64", 20000, 0.5), ("mixed", 100000, 1.0),
+                                               ("fp64", 500, 1.0)])
+def test_setup_is_ordered_before_the_kernels_that_read_it(fake, precision, n, alpha):
+    """Also what the handle leaves behind: a call on its stream comes after all of it."""
+    with Handle(fake, n, precision=precision, alpha=alpha) as h:
+        assert h.rc == 0
+        assert unordered_uploads(fake.log(), STREAM) == ([], 0)
+        fake.reset()
+        assert h.call("scf_set_option", 3, 64 if alpha == 1.0 else 128) == 0  # a new block map
+        assert unordered_uploads(fake.log(), STREAM) == ([], 0)
+
+
+def test_setup_stays_out_of_a_capture(fake):
+    with Handle(fake, 20000, stream=STREAM):  # the constants are up
+        pass
+    fake.capturing()
+    try:
+        with Handle(fake, 20000, stream=STREAM) as h:
+            assert h.rc == 0 and h.binned()
+            log = fake.log()
+            assert not [x for x in log if hex(STREAM) in x]
+            assert log[-1] == "synchronize 0x1"
+    finally:
+        fake.capturing(False)
