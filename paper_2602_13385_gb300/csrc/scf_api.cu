@@ -84,6 +84,7 @@ struct scf_handle {
   double* d_tid = nullptr;               // [n_prog][16]
   double* d_half = nullptr;              // [n_prog][4] selection at frac 1/2 (complete refresh)
   int bound_slots = 1;
+  int64_t max_n = 0;                     // particles of the largest progenitor
   int64_t bound_chunks = 0, bound_chunks_all = 0;  // pair-kernel chunks of the largest progenitor, of all
   const uint8_t* step_mask = nullptr;    // coefficient set of scf_step (scf_set_mask)
   double* d_Atmp = nullptr;              // [n_prog][2*NC] scratch coefficients
@@ -1015,6 +1016,7 @@ int scf_init(const scf_config* cfg, int n_prog, const int64_t* offsets, const do
   if (cudaDeviceGetAttribute(&h->n_sm, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess)
     return fail(SCF_ERR_CUDA);
   h->offsets.assign(offsets, offsets + n_prog + 1);
+  for (int p = 0; p < n_prog; ++p) h->max_n = std::max(h->max_n, offsets[p + 1] - offsets[p]);
 
   // Capacity of the block maps and partial rows: the largest any candidate shape can need.
   // Both radial families count (alpha = 1 and the general kernels), since
@@ -1693,6 +1695,8 @@ int scf_bound(scf_handle* h, const void* pos, const void* vel, double kin, doubl
   a.prog_off = h->d_off;
   a.n_prog = h->n_prog;
   a.n_total = h->n_total;
+  a.max_n = h->max_n;
+  a.n_sm = h->n_sm;
   a.f32 = h->cfg.precision == SCF_MIXED;
   a.slots = h->bound_slots;
   a.total_chunks = h->bound_chunks_all;
@@ -1705,7 +1709,7 @@ int scf_bound(scf_handle* h, const void* pos, const void* vel, double kin, doubl
   a.bound = bound_out;
   a.mask = mask_out;
   a.stats = stats_out;
-  return cuda_fail(scf_bound_launch(a, h->bound_chunks, h->n_sm, h->stream));
+  return cuda_fail(scf_bound_launch(a, h->bound_chunks, h->stream));
 }
 
 namespace {
@@ -1786,6 +1790,8 @@ int scf_evolve(scf_handle* h, void* pos, void* vel, void* acc, double* com, int 
         a.prog_off = h->d_off;
         a.n_prog = h->n_prog;
         a.n_total = h->n_total;
+        a.max_n = h->max_n;
+        a.n_sm = h->n_sm;
         a.f32 = h->cfg.precision == SCF_MIXED;
         a.frac = 0.5;
         a.key = h->d_key;

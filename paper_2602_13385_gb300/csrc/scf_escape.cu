@@ -20,9 +20,10 @@
 //                  (k_bound_pairs_ff).
 //   k_bound_finish one thread per particle: adds the slots in order, forms
 //                  E_i and the bound flag, and the radius key (bits of r^2).
-//   k_select       one block per progenitor: bound count and mass, radix
-//                  selection of the k-th smallest key (8 passes of 8 bits over
-//                  shared-memory histograms of integer counts), the mask.
+//   k_select       one block, or a cluster of eight, per progenitor: bound count
+//                  and mass, radix selection of the k-th smallest key (8 passes
+//                  of 8 bits over shared-memory histograms of integer counts),
+//                  the mask.
 //   k_tidal        one thread per progenitor.
 // Every sum has a fixed order, so results are bitwise reproducible.
 #include <cmath>
@@ -36,10 +37,10 @@
 
 namespace {
 
+namespace cg = cooperative_groups;
+
 constexpr int kPairThreads = 128;
 constexpr int kPairWarps = kPairThreads / 32;
-constexpr int kSelectThreads = 1024;
-constexpr int kSelectBlocks = 8;  // cluster of the selection
 
 template <typename V4>
 struct Elem;
@@ -399,25 +400,32 @@ __global__ void k_bound_finish(BoundArgs a) {
   a.key[i] = (unsigned long long)__double_as_longlong(r2);
 }
 
-// One cluster of kSelectBlocks blocks per progenitor: the blocks' histograms and
-// sums meet through distributed shared memory, so a radix pass is one sweep of
-// the cluster's threads over the particles (a single block's 1024 threads took
-// 297 us at N = 1e5).
-template <typename V4>
-__global__ void __cluster_dims__(kSelectBlocks, 1, 1) __launch_bounds__(kSelectThreads) k_select(BoundArgs a) {
-  namespace cg = cooperative_groups;
-  constexpr int NW = kSelectThreads / 32;
+// NB blocks of NT threads per progenitor (select_launch says which): the blocks'
+// histograms and sums meet through distributed shared memory, so a radix pass is
+// one sweep of the cluster's threads over the particles.
+template <int NB>
+__device__ __forceinline__ void select_sync() {
+  if constexpr (NB == 1) __syncthreads();
+  else cg::this_cluster().sync();
+}
+template <int NB, typename T>
+__device__ __forceinline__ T* of_block(T* p, int b) {  // p of the cluster's block b
+  if constexpr (NB == 1) return p;
+  else return cg::this_cluster().map_shared_rank(p, b);
+}
+template <typename V4, int NT, int NB>
+__global__ void __cluster_dims__(NB, 1, 1) __launch_bounds__(NT) k_select(BoundArgs a) {
+  constexpr int NW = NT / 32;
   __shared__ unsigned s_hist[2][256];   // alternating: a pass is read remotely while the next is cleared
   __shared__ unsigned s_scan[256];
   __shared__ double s_m[NW], s_mb;
   __shared__ unsigned long long s_c[NW], s_n;
   __shared__ unsigned s_digit, s_below;
-  cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank();
-  const int p = blockIdx.x / kSelectBlocks, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int rank = (int)blockIdx.x % NB;
+  const int p = blockIdx.x / NB, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t o0 = a.prog_off[p], o1 = a.prog_off[p + 1];
-  const int64_t first = o0 + (int64_t)rank * kSelectThreads + tid;
-  constexpr int64_t kStride = (int64_t)kSelectThreads * kSelectBlocks;
+  const int64_t first = o0 + (int64_t)rank * NT + tid;
+  constexpr int64_t kStride = (int64_t)NT * NB;
   const V4* pos = reinterpret_cast<const V4*>(a.pos);
   const uint8_t* bound = a.bound;
   const unsigned long long* key = a.key;
@@ -450,12 +458,12 @@ __global__ void __cluster_dims__(kSelectBlocks, 1, 1) __launch_bounds__(kSelectT
     s_n = nb;
     s_mb = mb;
   }
-  cluster.sync();
+  select_sync<NB>();
   unsigned long long nb = 0;
   double mb = 0.0;
-  for (int b = 0; b < kSelectBlocks; ++b) {
-    nb += *cluster.map_shared_rank(&s_n, b);
-    mb += *cluster.map_shared_rank(&s_mb, b);
+  for (int b = 0; b < NB; ++b) {
+    nb += *of_block<NB>(&s_n, b);
+    mb += *of_block<NB>(&s_mb, b);
   }
   unsigned long long krem = 0, prefix = 0;
   if (nb > 0) {
@@ -474,11 +482,11 @@ __global__ void __cluster_dims__(kSelectBlocks, 1, 1) __launch_bounds__(kSelectT
         const unsigned long long kk2 = key[k];
         if ((kk2 & hi) == prefix) atomicAdd(&hist[(kk2 >> shift) & 255ull], 1u);
       }
-      cluster.sync();
+      select_sync<NB>();
       // every block adds all the blocks' counts and finds the digit by a scan
       unsigned v = 0, t = 0;
       if (tid < 256) {
-        for (int b = 0; b < kSelectBlocks; ++b) v += *cluster.map_shared_rank(&hist[tid], b);
+        for (int b = 0; b < NB; ++b) v += *of_block<NB>(&hist[tid], b);
         t = v;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -512,7 +520,7 @@ __global__ void __cluster_dims__(kSelectBlocks, 1, 1) __launch_bounds__(kSelectT
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) cm += __shfl_xor_sync(0xffffffffu, cm, o);
-  cluster.sync();  // s_n has been read by every block
+  select_sync<NB>();  // s_n has been read by every block
   if (lane == 0) s_c[warp] = cm;
   __syncthreads();
   if (tid == 0) {
@@ -520,17 +528,17 @@ __global__ void __cluster_dims__(kSelectBlocks, 1, 1) __launch_bounds__(kSelectT
     for (int w = 0; w < NW; ++w) t += s_c[w];
     s_n = t;
   }
-  cluster.sync();
+  select_sync<NB>();
   if (rank == 0 && tid == 0) {
     unsigned long long n_in = 0;
-    for (int b = 0; b < kSelectBlocks; ++b) n_in += *cluster.map_shared_rank(&s_n, b);
+    for (int b = 0; b < NB; ++b) n_in += *of_block<NB>(&s_n, b);
     double* st = a.stats + 4 * (size_t)p;
     st[0] = (double)nb;
     st[1] = mb;
     st[2] = sqrt(__longlong_as_double((long long)kx));
     st[3] = (double)n_in;
   }
-  cluster.sync();  // no block leaves while its shared memory is read
+  select_sync<NB>();  // no block leaves while its shared memory is read
 }
 
 // Eigenvalues l1 >= l2 >= l3 of a symmetric 3x3 matrix S (row-major) by the
@@ -611,12 +619,23 @@ int scf_bound_slots(int64_t n_total) {
   return (int)(fit > kBoundMaxSlots ? kBoundMaxSlots : fit < 4 ? 4 : fit);
 }
 
+// A progenitor's selection is ten sweeps over its particles with block barriers between
+// them.  A cluster of eight blocks has an eighth of the sweep and dearer barriers, and
+// takes eight blocks' room (two blocks of 1024 threads an SM): it pays for a large
+// progenitor while the clusters run in a few waves.  Whole calls, one block / cluster
+// (us): mixed 1 x 4096 43/52, 12000 107/107, 16384 163/156, 65536 1930/1812, 4 x 8000
+// 146/148, 16 x 12000 995/1005, 24000 3289/3276, 64 x 8000 1513/1561, 2048 x 64 136/1678.
+// Up to 1024 particles a block of 256 threads leaves nobody idle and eight fit an SM:
+// 304 x 64 27 against 35, 2048 x 300 171 against 239, 1 x 2000 36 against 33.
 template <typename V4>
 static void select_launch(const BoundArgs& a, cudaStream_t s) {
-  k_select<V4><<<a.n_prog * kSelectBlocks, kSelectThreads, 0, s>>>(a);
+  const int64_t waves = (8 * (int64_t)a.n_prog + 2 * a.n_sm - 1) / (2 * a.n_sm);
+  if (waves < 8 && a.max_n * (8 - waves) >= 156000 * waves - 58500) k_select<V4, 1024, 8><<<8 * a.n_prog, 1024, 0, s>>>(a);
+  else if (a.max_n > 1024) k_select<V4, 1024, 1><<<a.n_prog, 1024, 0, s>>>(a);
+  else k_select<V4, 256, 1><<<a.n_prog, 256, 0, s>>>(a);
 }
 
-cudaError_t scf_bound_launch(const BoundArgs& a, int64_t max_chunks, int n_sm, cudaStream_t s) {
+cudaError_t scf_bound_launch(const BoundArgs& a, int64_t max_chunks, cudaStream_t s) {
   if (a.n_total > 0 && max_chunks > 0) {
     cudaError_t e = cudaMemsetAsync(a.part, 0, sizeof(double) * (size_t)a.slots * (size_t)a.n_total, s);
     if (e != cudaSuccess) return e;
@@ -625,7 +644,7 @@ cudaError_t scf_bound_launch(const BoundArgs& a, int64_t max_chunks, int n_sm, c
     // blocks an SM, a few waves of short blocks (with eight, King N = 1e5 in
     // double precision ran 1.5 waves a launch)
     const int64_t total = max_chunks / 2;  // rounds of the largest progenitor
-    int groups = (int)((32 * (int64_t)n_sm + a.total_chunks - 1) / a.total_chunks);
+    int groups = (int)((32 * (int64_t)a.n_sm + a.total_chunks - 1) / a.total_chunks);
     groups = groups < 1 ? 1 : groups > a.slots / 2 ? a.slots / 2 : groups;
     if (groups > total) groups = total < 1 ? 1 : (int)total;
     BoundArgs b = a;

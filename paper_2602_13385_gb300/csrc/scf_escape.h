@@ -17,7 +17,8 @@ struct BoundArgs {
   const void* vel;             // [N][4]
   const int64_t* prog_off;     // [n_prog + 1] particle offsets
   int n_prog;
-  int64_t n_total;
+  int64_t n_total, max_n;      // particles of all progenitors, of the largest
+  int n_sm;
   int f32;                     // particle arrays are float4
   int slots;                   // slots of part
   int64_t total_chunks;        // chunks of all progenitors
@@ -46,7 +47,7 @@ int64_t scf_bound_chunk(int f32);
 // Slots of BoundArgs::part for n_total particles.
 int scf_bound_slots(int64_t n_total);
 // max_chunks: chunks of the largest progenitor.
-cudaError_t scf_bound_launch(const BoundArgs& a, int64_t max_chunks, int n_sm, cudaStream_t s);
+cudaError_t scf_bound_launch(const BoundArgs& a, int64_t max_chunks, cudaStream_t s);
 cudaError_t scf_tidal_launch(const TidalArgs& a, cudaStream_t s);
 // The selection alone (bound flags and radius keys from a previous
 // scf_bound_launch; mask may be null).

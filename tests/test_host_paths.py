@@ -90,3 +90,23 @@ def test_setup_stays_out_of_a_capture(fake):
             assert log[-1] == "synchronize 0x1"
     finally:
         fake.capturing(False)
+
+
+def grid_of(fake, kernel):
+    return [tuple(int(v) for v in x.split()[2:6]) for x in fake.log() if x.startswith("launch") and kernel in x]
+
+
+@pytest.mark.parametrize("sizes,blocks,threads", [([64] * 2048, 1, 256), ([1024], 1, 256), ([1025], 1, 1024),
+                                                  ([3000] * 304, 1, 1024), ([10000] * 64, 1, 1024), ([30000] * 16, 8, 1024),
+                                                  ([13000], 1, 1024), ([14000, 0, 5], 8, 1024), ([200000] * 300, 1, 1024)])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_blocks_of_the_selection(fake, precision, sizes, blocks, threads):
+    """A cluster of blocks a progenitor only where it pays (rule in scf_escape.cu)."""
+    off = [0]
+    for s in sizes:
+        off.append(off[-1] + s)
+    with Handle(fake, 0, nmax=4, lmax=2, precision=precision, offsets=off) as h:
+        assert h.rc == 0
+        fake.reset()
+        assert h.call("scf_bound", 0x1000, 0x2000, ctypes.c_double(0.5), ctypes.c_double(0.9), None, 0x3000, None, 0x4000) == 0
+        assert grid_of(fake, "k_select") == [(blocks * len(sizes), 1, 1, threads)]
