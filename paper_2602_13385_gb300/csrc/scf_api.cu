@@ -79,13 +79,12 @@ struct scf_handle {
   double* d_en_part = nullptr;        // [k3 blocks][4] energy partials
   // escape physics: particle offsets, pair-sum segments, radius keys, tidal scales
   int64_t* d_off = nullptr;              // [n_prog+1]
-  double* d_bpart = nullptr;             // [bound_slots][n_total]
+  double* d_bpart = nullptr;             // [bound.slots][n_total]
   unsigned long long* d_key = nullptr;   // [n_total]
   double* d_tid = nullptr;               // [n_prog][16]
   double* d_half = nullptr;              // [n_prog][4] selection at frac 1/2 (complete refresh)
-  int bound_slots = 1;
+  BoundPlan bound;
   int64_t max_n = 0;                     // particles of the largest progenitor
-  int64_t bound_chunks = 0, bound_chunks_all = 0;  // pair-kernel chunks of the largest progenitor, of all
   const uint8_t* step_mask = nullptr;    // coefficient set of scf_step (scf_set_mask)
   double* d_Atmp = nullptr;              // [n_prog][2*NC] scratch coefficients
   ScfLaunchInfo k1d{}, k3d{};
@@ -1069,19 +1068,9 @@ int scf_init(const scf_config* cfg, int n_prog, const int64_t* offsets, const do
   const size_t o_st = take(sizeof(unsigned) * 4);
   const size_t o_en = take(sizeof(double) * 4 * nb3);
   const size_t o_adj = cfg->precision == SCF_FP64 ? take(sizeof(double) * SCF_ADJ_Q * nb3) : off;
-  {
-    const int64_t chunk = scf_bound_chunk(cfg->precision == SCF_MIXED);
-    int64_t chunks = 0;
-    for (int p = 0; p < n_prog; ++p) {
-      const int64_t c = (h->offsets[p + 1] - h->offsets[p] + chunk - 1) / chunk;
-      chunks += c;
-      h->bound_chunks = std::max(h->bound_chunks, c);
-    }
-    h->bound_chunks_all = chunks;
-    h->bound_slots = scf_bound_slots(h->n_total);
-  }
+  h->bound = scf_bound_plan(offsets, n_prog, cfg->precision == SCF_MIXED, h->n_sm);
   const size_t o_off = take(sizeof(int64_t) * (n_prog + 1));
-  const size_t o_bpart = take(sizeof(double) * (size_t)h->bound_slots * (size_t)h->n_total);
+  const size_t o_bpart = take(sizeof(double) * (size_t)h->bound.slots * (size_t)h->n_total);
   const size_t o_key = take(sizeof(unsigned long long) * (size_t)h->n_total);
   const size_t o_tid = take(sizeof(double) * 16 * (size_t)n_prog);
   const size_t o_half = take(sizeof(double) * 4 * (size_t)n_prog);
@@ -1698,8 +1687,7 @@ int scf_bound(scf_handle* h, const void* pos, const void* vel, double kin, doubl
   a.max_n = h->max_n;
   a.n_sm = h->n_sm;
   a.f32 = h->cfg.precision == SCF_MIXED;
-  a.slots = h->bound_slots;
-  a.total_chunks = h->bound_chunks_all;
+  a.slots = h->bound.slots;
   a.G = h->cfg.G;
   a.kin = kin;
   a.frac = frac;
@@ -1709,7 +1697,7 @@ int scf_bound(scf_handle* h, const void* pos, const void* vel, double kin, doubl
   a.bound = bound_out;
   a.mask = mask_out;
   a.stats = stats_out;
-  return cuda_fail(scf_bound_launch(a, h->bound_chunks, h->stream));
+  return cuda_fail(scf_bound_launch(a, h->bound, h->stream));
 }
 
 namespace {

@@ -18,6 +18,7 @@
 //                  their sums travel around the warp with them.  Double precision
 //                  evaluates the pair terms in float-float arithmetic
 //                  (k_bound_pairs_ff).
+//   k_bound_ordered, _ff  every ordered pair, for small samples.
 //   k_bound_finish one thread per particle: adds the slots in order, forms
 //                  E_i and the bound flag, and the radius key (bits of r^2).
 //   k_select       one block, or a cluster of eight, per progenitor: bound count
@@ -26,6 +27,7 @@
 //                  the mask.
 //   k_tidal        one thread per progenitor.
 // Every sum has a fixed order, so results are bitwise reproducible.
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cooperative_groups.h>
@@ -381,6 +383,163 @@ __global__ void __launch_bounds__(kPairThreads) k_bound_pairs_ff(BoundArgs a) {
   }
 }
 
+// Ordered pairs, for samples too small to fill the chip with rounds of chunks (scf_bound_plan):
+// block (i-chunk, progenitor, segment) stages its segment of the j-particles through shared
+// memory and evaluates every pair of it for the i-particle alone, so a chunk's work is as many
+// independent blocks as there are slots, each with a short chain; slot s holds segment s.
+// King N = 4096 (us a call): mixed 43, rounds of chunks 80; float-float 102 and 134.
+constexpr int kPairSub = 64;  // pair terms summed in single precision (or float-float) before the double add
+
+__device__ __forceinline__ float pair_inv_r1(float r2) {
+  const float y = rsqrt_approx(r2);
+  return r2 >= 1.17549435e-38f ? y : 0.f;  // as pair_inv_r<true>
+}
+
+__global__ void __launch_bounds__(kPairThreads) k_bound_ordered(BoundArgs a) {
+  constexpr int kPairI = Elem<float4>::I;
+  __shared__ float4 s_j[kPairThreads];
+  const float4* pos = reinterpret_cast<const float4*>(a.pos);
+  for (int p = blockIdx.y; p < a.n_prog; p += gridDim.y) {
+    const int64_t o0 = a.prog_off[p], o1 = a.prog_off[p + 1];
+    const int64_t ib = o0 + (int64_t)blockIdx.x * (kPairThreads * kPairI);
+    if (ib >= o1) continue;  // the same for every thread of the block
+    const int64_t seg = (o1 - o0 + a.slots - 1) / a.slots;
+    const int64_t j0 = min(o1, o0 + (int64_t)blockIdx.z * seg), j1 = min(o1, j0 + seg);
+    float xi[kPairI], yi[kPairI], zi[kPairI];
+    double acc[kPairI];
+#pragma unroll
+    for (int q = 0; q < kPairI; ++q) {
+      const int64_t i = ib + threadIdx.x + q * kPairThreads;
+      const float4 pi = i < o1 ? pos[i] : float4{};
+      xi[q] = pi.x;
+      yi[q] = pi.y;
+      zi[q] = pi.z;
+      acc[q] = 0.0;
+    }
+    for (int64_t jb = j0; jb < j1; jb += kPairThreads) {
+      const int cnt = (int)min((int64_t)kPairThreads, j1 - jb);
+      __syncthreads();
+      if ((int)threadIdx.x < cnt) s_j[threadIdx.x] = pos[jb + threadIdx.x];
+      __syncthreads();
+      for (int s = 0; s < cnt; s += kPairSub) {
+        const int e = min(cnt, s + kPairSub);
+        float part[kPairI];
+#pragma unroll
+        for (int q = 0; q < kPairI; ++q) part[q] = 0.f;
+#pragma unroll 4
+        for (int jj = s; jj < e; ++jj) {
+          const float4 pj = s_j[jj];
+#pragma unroll
+          for (int q = 0; q < kPairI; ++q) {
+            const float dx = pj.x - xi[q], dy = pj.y - yi[q], dz = pj.z - zi[q];
+            const float r2 = dx * dx + dy * dy + dz * dz;
+            // the self pair (and any coincident pair, and non-finite r2) adds nothing
+            const float ri = pair_inv_r1(r2);
+            part[q] += pj.w * ri;
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < kPairI; ++q) acc[q] += (double)part[q];
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kPairI; ++q) {
+      const int64_t i = ib + threadIdx.x + q * kPairThreads;
+      if (i < o1) a.part[(size_t)blockIdx.z * (size_t)a.n_total + (size_t)i] = acc[q];
+    }
+  }
+}
+
+__device__ __forceinline__ SplitF two_sum1(float a, float b) {
+  const float s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+
+__global__ void __launch_bounds__(kPairThreads) k_bound_ordered_ff(BoundArgs a) {
+  constexpr int kPairI = Elem<ScfD4>::I;
+  __shared__ float4 s_hi[kPairThreads], s_lo[kPairThreads];
+  const ScfD4* pos = reinterpret_cast<const ScfD4*>(a.pos);
+  for (int p = blockIdx.y; p < a.n_prog; p += gridDim.y) {
+    const int64_t o0 = a.prog_off[p], o1 = a.prog_off[p + 1];
+    const int64_t ib = o0 + (int64_t)blockIdx.x * (kPairThreads * kPairI);
+    if (ib >= o1) continue;  // the same for every thread of the block
+    const int64_t seg = (o1 - o0 + a.slots - 1) / a.slots;
+    const int64_t j0 = min(o1, o0 + (int64_t)blockIdx.z * seg), j1 = min(o1, j0 + seg);
+    SplitF xi[kPairI], yi[kPairI], zi[kPairI];
+    double acc[kPairI];
+#pragma unroll
+    for (int q = 0; q < kPairI; ++q) {
+      const int64_t i = ib + threadIdx.x + q * kPairThreads;
+      const ScfD4 pi = i < o1 ? pos[i] : ScfD4{};
+      xi[q] = split_double(pi.x);
+      yi[q] = split_double(pi.y);
+      zi[q] = split_double(pi.z);
+      acc[q] = 0.0;
+    }
+    for (int64_t jb = j0; jb < j1; jb += kPairThreads) {
+      const int cnt = (int)min((int64_t)kPairThreads, j1 - jb);
+      __syncthreads();
+      if ((int)threadIdx.x < cnt) {
+        const ScfD4 pj = pos[jb + threadIdx.x];
+        const SplitF x = split_double(pj.x), y = split_double(pj.y), z = split_double(pj.z), m = split_double(pj.w);
+        s_hi[threadIdx.x] = make_float4(x.h, y.h, z.h, m.h);
+        s_lo[threadIdx.x] = make_float4(x.l, y.l, z.l, m.l);
+      }
+      __syncthreads();
+      for (int s = 0; s < cnt; s += kPairSub) {
+        const int e = min(cnt, s + kPairSub);
+        SplitF sum[kPairI];
+#pragma unroll
+        for (int q = 0; q < kPairI; ++q) sum[q] = {0.f, 0.f};
+#pragma unroll 2
+        for (int jj = s; jj < e; ++jj) {
+          const float4 hj = s_hi[jj], lj = s_lo[jj];
+#pragma unroll
+          for (int q = 0; q < kPairI; ++q) {
+            // separation: exact difference of the hi parts + difference of the lo parts
+            const SplitF dx = two_sum1(hj.x, -xi[q].h), dy = two_sum1(hj.y, -yi[q].h), dz = two_sum1(hj.z, -zi[q].h);
+            const float lx = __fadd_rn(dx.l, __fsub_rn(lj.x, xi[q].l));
+            const float ly = __fadd_rn(dy.l, __fsub_rn(lj.y, yi[q].l));
+            const float lz = __fadd_rn(dz.l, __fsub_rn(lj.z, zi[q].l));
+            // r^2 = sum (h + l)^2 = sum h^2 + (2h + l) l, with the exact rounding
+            // error of each h^2, renormalised (all of r^2 may sit in the l parts)
+            const float px = __fmul_rn(dx.h, dx.h), py = __fmul_rn(dy.h, dy.h), pz = __fmul_rn(dz.h, dz.h);
+            const float cx = fmaf(__fadd_rn(__fadd_rn(dx.h, dx.h), lx), lx, fmaf(dx.h, dx.h, -px));
+            const float cy = fmaf(__fadd_rn(__fadd_rn(dy.h, dy.h), ly), ly, fmaf(dy.h, dy.h, -py));
+            const float cz = fmaf(__fadd_rn(__fadd_rn(dz.h, dz.h), lz), lz, fmaf(dz.h, dz.h, -pz));
+            const SplitF s1 = two_sum1(px, py);
+            const SplitF s2 = two_sum1(s1.h, pz);
+            const SplitF r2 = two_sum1(s2.h, __fadd_rn(__fadd_rn(s1.l, s2.l), __fadd_rn(__fadd_rn(cx, cy), cz)));
+            const float r2h = r2.h, r2l = r2.l;
+            // 1/r: one Newton step y0 (1 + d/2), d = 1 - r^2 y0^2 in float-float
+            const float y0 = rsqrt_approx(r2h);
+            const float t = __fmul_rn(y0, y0), te = fmaf(y0, y0, -t);
+            const float u = __fmul_rn(r2h, t);
+            const float ue = fmaf(r2l, t, fmaf(r2h, te, fmaf(r2h, t, -u)));
+            const float d = __fsub_rn(__fsub_rn(1.f, u), ue);
+            const float corr = __fmul_rn(__fmul_rn(0.5f, y0), d);
+            const float yh = __fadd_rn(y0, corr), yl = __fsub_rn(corr, __fsub_rn(yh, y0));
+            // m / r into the float-float sum; pairs outside the normal range add nothing
+            const bool ok = r2h >= 1.17549435e-38f && r2h <= 3.40282347e38f;
+            const float ph = ok ? __fmul_rn(hj.w, yh) : 0.f;
+            const float pe = ok ? fmaf(hj.w, yl, fmaf(lj.w, yh, fmaf(hj.w, yh, -ph))) : 0.f;
+            const SplitF ns = two_sum1(sum[q].h, ph);
+            sum[q] = {ns.h, __fadd_rn(sum[q].l, __fadd_rn(ns.l, pe))};
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < kPairI; ++q) acc[q] += (double)sum[q].h + (double)sum[q].l;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kPairI; ++q) {
+      const int64_t i = ib + threadIdx.x + q * kPairThreads;
+      if (i < o1) a.part[(size_t)blockIdx.z * (size_t)a.n_total + (size_t)i] = acc[q];
+    }
+  }
+}
+
 template <typename V4>
 __global__ void k_bound_finish(BoundArgs a) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -610,13 +769,43 @@ __global__ void k_tidal(TidalArgs a) {
 
 }  // namespace
 
-int64_t scf_bound_chunk(int f32) { return f32 ? kPairChunk<float4> : kPairChunk<ScfD4>; }
+static int64_t scf_bound_chunk(int f32) { return f32 ? kPairChunk<float4> : kPairChunk<ScfD4>; }
 
 // Slots of the pair sums: 64, fewer where they would take more than 2 GiB (at
 // least 4: two groups of one round).
-int scf_bound_slots(int64_t n_total) {
+static int scf_bound_slots(int64_t n_total) {
   const int64_t fit = n_total > 0 ? ((int64_t)1 << 31) / (8 * n_total) : kBoundMaxSlots;
   return (int)(fit > kBoundMaxSlots ? kBoundMaxSlots : fit < 4 ? 4 : fit);
+}
+
+// Rounds of chunks or ordered pairs.  Both evaluate about 3e12 pairs a second in single
+// precision and 3.6e11 in float-float when the chip is full, of C^2 (P + P (P - 1) / 2) for the
+// P chunks of a progenitor and of C P n, and a call over rounds takes the time of kLag pairs more:
+// its shortest chain is a chunk against itself and one other.  Calls, ordered / rounds (us):
+//   mixed  1 x 8000 72/87, 12000 107/99, 16384 163/124; 4 x 3000 46/79, 8000 146/109; 16 x 3000 90/88;
+//          64 x 1000 54/76, 2000 138/127; 304 x 1000 150/154; 2048 x 64 136/290, 700 637/697, 1000 869/733
+//   double 1 x 4096 102/134, 6000 170/151; 4 x 1000 46/128, 3000 169/147; 64 x 300 65/128, 1000 259/248;
+//          2048 x 300 997/1403, 700 3192/2494
+BoundPlan scf_bound_plan(const int64_t* offsets, int n_prog, int f32, int n_sm) {
+  BoundPlan pl;
+  const int64_t C = scf_bound_chunk(f32);
+  const double kLag = f32 ? 6e7 : 1.2e7;
+  double ordered = 0.0, rounds = kLag;
+  for (int p = 0; p < n_prog; ++p) {
+    const int64_t n = offsets[p + 1] - offsets[p], P = (n + C - 1) / C;
+    pl.chunks += P;
+    pl.max_chunks = std::max(pl.max_chunks, P);
+    ordered += (double)C * P * n;
+    rounds += (double)C * C * (P + 0.5 * P * (P - 1.0));
+  }
+  pl.ordered = ordered <= rounds;
+  if (pl.ordered) {  // about four blocks an SM
+    const int64_t s = pl.chunks > 0 ? (4 * (int64_t)n_sm + pl.chunks - 1) / pl.chunks : 1;
+    pl.slots = (int)std::min<int64_t>(s, kBoundMaxSegments);
+  } else {
+    pl.slots = scf_bound_slots(offsets[n_prog]);
+  }
+  return pl;
 }
 
 // A progenitor's selection is ten sweeps over its particles with block barriers between
@@ -635,24 +824,31 @@ static void select_launch(const BoundArgs& a, cudaStream_t s) {
   else k_select<V4, 256, 1><<<a.n_prog, 256, 0, s>>>(a);
 }
 
-cudaError_t scf_bound_launch(const BoundArgs& a, int64_t max_chunks, cudaStream_t s) {
-  if (a.n_total > 0 && max_chunks > 0) {
-    cudaError_t e = cudaMemsetAsync(a.part, 0, sizeof(double) * (size_t)a.slots * (size_t)a.n_total, s);
-    if (e != cudaSuccess) return e;
-    // groups x (1 + rounds) slots a launch: as many rounds a block (its
-    // i-particles are loaded once, its sums stored once) as still leave about 32
-    // blocks an SM, a few waves of short blocks (with eight, King N = 1e5 in
-    // double precision ran 1.5 waves a launch)
-    const int64_t total = max_chunks / 2;  // rounds of the largest progenitor
-    int groups = (int)((32 * (int64_t)a.n_sm + a.total_chunks - 1) / a.total_chunks);
-    groups = groups < 1 ? 1 : groups > a.slots / 2 ? a.slots / 2 : groups;
-    if (groups > total) groups = total < 1 ? 1 : (int)total;
-    BoundArgs b = a;
-    b.rounds = a.slots / groups - 1;
-    for (b.round0 = 1; b.round0 == 1 || b.round0 <= total; b.round0 += groups * b.rounds) {
-      const dim3 grid((unsigned)max_chunks, (unsigned)(a.n_prog < 65535 ? a.n_prog : 65535), (unsigned)groups);
-      if (a.f32) k_bound_pairs<<<grid, kPairThreads, 0, s>>>(b);
-      else k_bound_pairs_ff<<<grid, kPairThreads, 0, s>>>(b);
+cudaError_t scf_bound_launch(const BoundArgs& a, const BoundPlan& pl, cudaStream_t s) {
+  if (a.n_total > 0) {
+    const unsigned gy = (unsigned)(a.n_prog < 65535 ? a.n_prog : 65535);
+    if (pl.ordered) {
+      const dim3 grid((unsigned)pl.max_chunks, gy, (unsigned)pl.slots);
+      if (a.f32) k_bound_ordered<<<grid, kPairThreads, 0, s>>>(a);
+      else k_bound_ordered_ff<<<grid, kPairThreads, 0, s>>>(a);
+    } else {
+      cudaError_t e = cudaMemsetAsync(a.part, 0, sizeof(double) * (size_t)a.slots * (size_t)a.n_total, s);
+      if (e != cudaSuccess) return e;
+      // groups x (1 + rounds) slots a launch: as many rounds a block (its
+      // i-particles are loaded once, its sums stored once) as still leave about 32
+      // blocks an SM, a few waves of short blocks (with eight, King N = 1e5 in
+      // double precision ran 1.5 waves a launch)
+      const int64_t total = pl.max_chunks / 2;  // rounds of the largest progenitor
+      int groups = (int)((32 * (int64_t)a.n_sm + pl.chunks - 1) / pl.chunks);
+      groups = groups < 1 ? 1 : groups > a.slots / 2 ? a.slots / 2 : groups;
+      if (groups > total) groups = total < 1 ? 1 : (int)total;
+      BoundArgs b = a;
+      b.rounds = a.slots / groups - 1;
+      for (b.round0 = 1; b.round0 == 1 || b.round0 <= total; b.round0 += groups * b.rounds) {
+        const dim3 grid((unsigned)pl.max_chunks, gy, (unsigned)groups);
+        if (a.f32) k_bound_pairs<<<grid, kPairThreads, 0, s>>>(b);
+        else k_bound_pairs_ff<<<grid, kPairThreads, 0, s>>>(b);
+      }
     }
     const unsigned fb = (unsigned)((a.n_total + 255) / 256);
     if (a.f32) k_bound_finish<float4><<<fb, 256, 0, s>>>(a);

@@ -9,8 +9,16 @@
 
 #include "scf_device.cuh"
 
-// Most pair-sum slots (doubles per particle) of the workspace.
+// Most pair-sum slots (doubles per particle) of the workspace, and of ordered pairs.
 constexpr int kBoundMaxSlots = 64;
+constexpr int kBoundMaxSegments = 16;
+
+// How a handle's pair sums run.
+struct BoundPlan {
+  bool ordered = true;         // every ordered pair; else rounds of chunks
+  int slots = 1;               // of BoundArgs::part
+  int64_t chunks = 0, max_chunks = 0;  // of all progenitors, of the largest
+};
 
 struct BoundArgs {
   const void* pos;             // [N][4] float (mixed) or double
@@ -21,7 +29,6 @@ struct BoundArgs {
   int n_sm;
   int f32;                     // particle arrays are float4
   int slots;                   // slots of part
-  int64_t total_chunks;        // chunks of all progenitors
   int round0, rounds;          // of a pair launch (set by scf_bound_launch)
   double G, kin, frac;
   double* part;                // [slots][N] partial sums of m_j / r_ij
@@ -42,12 +49,8 @@ struct TidalArgs {
   double* out;                 // [n_prog][16]
 };
 
-// Particles of a chunk of the pair kernel (f32: single-precision particles).
-int64_t scf_bound_chunk(int f32);
-// Slots of BoundArgs::part for n_total particles.
-int scf_bound_slots(int64_t n_total);
-// max_chunks: chunks of the largest progenitor.
-cudaError_t scf_bound_launch(const BoundArgs& a, int64_t max_chunks, cudaStream_t s);
+BoundPlan scf_bound_plan(const int64_t* offsets, int n_prog, int f32, int n_sm);
+cudaError_t scf_bound_launch(const BoundArgs& a, const BoundPlan& pl, cudaStream_t s);
 cudaError_t scf_tidal_launch(const TidalArgs& a, cudaStream_t s);
 // The selection alone (bound flags and radius keys from a previous
 // scf_bound_launch; mask may be null).

@@ -17,7 +17,9 @@ def scf():
 
 
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
-@pytest.mark.parametrize("sizes", [[1024], [1025], [13927], [13930], [14001, 0, 7, 300], [64] * 400, [1100] * 40])
+@pytest.mark.parametrize("sizes", [[1024], [1025], [13927], [13930], [14001, 0, 7, 300], [64] * 400, [1100] * 40,
+                                   [4600], [4900], [11100], [11400],      # ordered pairs below, rounds of chunks above
+                                   [14001, 0, 1, 255, 256, 257, 511, 512, 513, 768, 1025, 2049]])
 def test_sums_and_selection(scf, prec, sizes):
     off = [0]
     for s in sizes:

@@ -110,3 +110,19 @@ def test_blocks_of_the_selection(fake, precision, sizes, blocks, threads):
         fake.reset()
         assert h.call("scf_bound", 0x1000, 0x2000, ctypes.c_double(0.5), ctypes.c_double(0.9), None, 0x3000, None, 0x4000) == 0
         assert grid_of(fake, "k_select") == [(blocks * len(sizes), 1, 1, threads)]
+
+
+@pytest.mark.parametrize("precision,sizes,ordered", [
+    ("mixed", [300], True), ("mixed", [8000], True), ("mixed", [16384], False), ("mixed", [64] * 2048, True),
+    ("mixed", [700] * 2048, True), ("mixed", [1000] * 2048, False), ("mixed", [100000], False),
+    ("fp64", [1000], True), ("fp64", [4096], True), ("fp64", [6000], False), ("fp64", [300] * 2048, True),
+    ("fp64", [700] * 2048, False), ("fp64", [1000] * 16, True)])
+def test_small_samples_take_ordered_pairs(fake, precision, sizes, ordered):
+    off = [0]
+    for s in sizes:
+        off.append(off[-1] + s)
+    with Handle(fake, 0, nmax=4, lmax=2, precision=precision, offsets=off) as h:
+        fake.reset()
+        assert h.call("scf_bound", 0x1000, 0x2000, ctypes.c_double(0.5), ctypes.c_double(0.9), None, 0x3000, None, 0x4000) == 0
+        assert bool(grid_of(fake, "k_bound_ordered")) == ordered
+        assert bool(grid_of(fake, "k_bound_pairs")) != ordered
