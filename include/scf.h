@@ -376,8 +376,9 @@ int scf_energy(scf_handle* h, const void* pos, const void* vel, const void* acc,
  *   mask_out   device [N] bytes, 1 = r <= r_x, or NULL
  *   stats_out  device [n_prog][4] doubles: n_bound, bound mass, r_x, size of the set
  * All sums have a fixed order (bitwise reproducible).  Cost O(sum_p N_p^2).
- * The workspace for it (8 (S+1) N bytes, S = 64 partial sums a particle, fewer
- * where they would take more than 2 GiB) is reserved by scf_init.
+ * The workspace for it (8 (S+1) N bytes, S <= 64 partial sums a particle: at
+ * most 150 MB of them up to N = 2e6, S = 2 to 4 beyond; S = 1, which costs time,
+ * where there is no memory for more) is reserved by scf_init.
  * Errors: SCF_ERR_NULL_POINTER, SCF_ERR_MISALIGNED, SCF_ERR_INVALID_ARG, SCF_ERR_CUDA. */
 int scf_bound(scf_handle* h, const void* pos, const void* vel, double kin, double frac, double* E_out,
               uint8_t* bound_out, uint8_t* mask_out, double* stats_out);

@@ -1070,7 +1070,6 @@ int scf_init(const scf_config* cfg, int n_prog, const int64_t* offsets, const do
   const size_t o_adj = cfg->precision == SCF_FP64 ? take(sizeof(double) * SCF_ADJ_Q * nb3) : off;
   h->bound = scf_bound_plan(offsets, n_prog, cfg->precision == SCF_MIXED, h->n_sm);
   const size_t o_off = take(sizeof(int64_t) * (n_prog + 1));
-  const size_t o_bpart = take(sizeof(double) * (size_t)h->bound.slots * (size_t)h->n_total);
   const size_t o_key = take(sizeof(unsigned long long) * (size_t)h->n_total);
   const size_t o_tid = take(sizeof(double) * 16 * (size_t)n_prog);
   const size_t o_half = take(sizeof(double) * 4 * (size_t)n_prog);
@@ -1083,9 +1082,16 @@ int scf_init(const scf_config* cfg, int n_prog, const int64_t* offsets, const do
   const size_t o_cs = take(sizeof(float4) * (size_t)(cfg->lmax + 1) * (cfg->nmax + 1));
   const size_t o_tidf = take(sizeof(float) * SCF_HOST_CAP * SCF_TIDAL_W * (size_t)n_prog);
   const size_t o_tidn = take(sizeof(float) * SCF_HOST_CAP * SCF_TIDAL_W * (size_t)n_prog);
-  if (cudaMalloc(&h->d_base, off) != cudaSuccess) {
+  const size_t slot = sizeof(double) * (size_t)h->n_total, o_bpart = off;  // the pair sums come last
+  if (cudaMalloc(&h->d_base, o_bpart + round_up(slot * h->bound.slots)) != cudaSuccess) {
+    // without the memory for their slots the pair sums run over ordered pairs in one
     cudaGetLastError();
-    return fail(SCF_ERR_OUT_OF_MEMORY);
+    h->bound.ordered = true;
+    h->bound.slots = 1;
+    if (cudaMalloc(&h->d_base, o_bpart + round_up(slot)) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(SCF_ERR_OUT_OF_MEMORY);
+    }
   }
   char* base = static_cast<char*>(h->d_base);
   h->d_partials = reinterpret_cast<double*>(base + o_part);

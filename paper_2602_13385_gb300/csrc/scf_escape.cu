@@ -771,13 +771,6 @@ __global__ void k_tidal(TidalArgs a) {
 
 static int64_t scf_bound_chunk(int f32) { return f32 ? kPairChunk<float4> : kPairChunk<ScfD4>; }
 
-// Slots of the pair sums: 64, fewer where they would take more than 2 GiB (at
-// least 4: two groups of one round).
-static int scf_bound_slots(int64_t n_total) {
-  const int64_t fit = n_total > 0 ? ((int64_t)1 << 31) / (8 * n_total) : kBoundMaxSlots;
-  return (int)(fit > kBoundMaxSlots ? kBoundMaxSlots : fit < 4 ? 4 : fit);
-}
-
 // Rounds of chunks or ordered pairs.  Both evaluate about 3e12 pairs a second in single
 // precision and 3.6e11 in float-float when the chip is full, of C^2 (P + P (P - 1) / 2) for the
 // P chunks of a progenitor and of C P n, and a call over rounds takes the time of kLag pairs more:
@@ -803,7 +796,18 @@ BoundPlan scf_bound_plan(const int64_t* offsets, int n_prog, int f32, int n_sm) 
     const int64_t s = pl.chunks > 0 ? (4 * (int64_t)n_sm + pl.chunks - 1) / pl.chunks : 1;
     pl.slots = (int)std::min<int64_t>(s, kBoundMaxSegments);
   } else {
-    pl.slots = scf_bound_slots(offsets[n_prog]);
+    // Blocks of a launch: as many groups as leave about 32 blocks an SM, a few waves of short
+    // blocks (with eight, King N = 1e5 in double precision ran 1.5 waves a launch).  Rounds a
+    // block: so many that a launch takes about 2 ms, since its start and end cost some 10 us (one
+    // round a block took 144.5 ms at N = 1e6 in single precision where 20 took 140.1, and 14.68
+    // ms where 14.45 for ten progenitors of 1e5); each takes a slot, 8 N bytes that every call
+    // clears and reads.
+    const int64_t total = pl.max_chunks / 2, groups = (32 * (int64_t)n_sm + pl.chunks - 1) / pl.chunks;
+    pl.groups = (int)std::max<int64_t>(1, std::min({groups, total, (int64_t)kBoundMaxSlots / 2}));
+    const int64_t per = (int64_t)((f32 ? 6e9 : 7.2e8) / ((double)pl.chunks * pl.groups * C * C)) + 1;
+    const int64_t most = std::min<int64_t>(kBoundMaxSlots / pl.groups - 1, (total + pl.groups - 1) / pl.groups);
+    pl.rounds = (int)std::max<int64_t>(1, std::min(per, most));
+    pl.slots = pl.groups * (1 + pl.rounds);
   }
   return pl;
 }
@@ -834,18 +838,12 @@ cudaError_t scf_bound_launch(const BoundArgs& a, const BoundPlan& pl, cudaStream
     } else {
       cudaError_t e = cudaMemsetAsync(a.part, 0, sizeof(double) * (size_t)a.slots * (size_t)a.n_total, s);
       if (e != cudaSuccess) return e;
-      // groups x (1 + rounds) slots a launch: as many rounds a block (its
-      // i-particles are loaded once, its sums stored once) as still leave about 32
-      // blocks an SM, a few waves of short blocks (with eight, King N = 1e5 in
-      // double precision ran 1.5 waves a launch)
       const int64_t total = pl.max_chunks / 2;  // rounds of the largest progenitor
-      int groups = (int)((32 * (int64_t)a.n_sm + pl.chunks - 1) / pl.chunks);
-      groups = groups < 1 ? 1 : groups > a.slots / 2 ? a.slots / 2 : groups;
-      if (groups > total) groups = total < 1 ? 1 : (int)total;
       BoundArgs b = a;
-      b.rounds = a.slots / groups - 1;
-      for (b.round0 = 1; b.round0 == 1 || b.round0 <= total; b.round0 += groups * b.rounds) {
-        const dim3 grid((unsigned)pl.max_chunks, gy, (unsigned)groups);
+      b.rounds = pl.rounds;
+      for (int64_t r = 1; r == 1 || r <= total; r += (int64_t)pl.groups * pl.rounds) {
+        b.round0 = (int)r;
+        const dim3 grid((unsigned)pl.max_chunks, gy, (unsigned)pl.groups);
         if (a.f32) k_bound_pairs<<<grid, kPairThreads, 0, s>>>(b);
         else k_bound_pairs_ff<<<grid, kPairThreads, 0, s>>>(b);
       }

@@ -17,6 +17,7 @@ constexpr int kBoundMaxSegments = 16;
 struct BoundPlan {
   bool ordered = true;         // every ordered pair; else rounds of chunks
   int slots = 1;               // of BoundArgs::part
+  int groups = 1, rounds = 1;  // of a launch over rounds, of a block: groups (1 + rounds) slots
   int64_t chunks = 0, max_chunks = 0;  // of all progenitors, of the largest
 };
 
@@ -49,6 +50,7 @@ struct TidalArgs {
   double* out;                 // [n_prog][16]
 };
 
+// With one slot every sample can run ordered pairs (ordered = true, slots = 1).
 BoundPlan scf_bound_plan(const int64_t* offsets, int n_prog, int f32, int n_sm);
 cudaError_t scf_bound_launch(const BoundArgs& a, const BoundPlan& pl, cudaStream_t s);
 cudaError_t scf_tidal_launch(const TidalArgs& a, cudaStream_t s);

@@ -126,3 +126,29 @@ def test_small_samples_take_ordered_pairs(fake, precision, sizes, ordered):
         assert h.call("scf_bound", 0x1000, 0x2000, ctypes.c_double(0.5), ctypes.c_double(0.9), None, 0x3000, None, 0x4000) == 0
         assert bool(grid_of(fake, "k_bound_ordered")) == ordered
         assert bool(grid_of(fake, "k_bound_pairs")) != ordered
+
+
+@pytest.mark.parametrize("precision,sizes,megabytes", [("mixed", [10 ** 6], 120), ("fp64", [10 ** 6], 60),
+                                                       ("mixed", [100000] * 10, 120), ("fp64", [1000] * 1024, 50)])
+def test_workspace_of_the_pair_sums(fake, precision, sizes, megabytes):
+    """The handle's memory without bins (lmax 2): keys, block maps, and the pair sums' slots."""
+    off = [0]
+    for s in sizes:
+        off.append(off[-1] + s)
+    with Handle(fake, 0, nmax=4, lmax=2, precision=precision, offsets=off) as h:
+        assert h.rc == 0
+        assert fake.used() < (megabytes + 20) * 1e6
+
+
+def test_pair_sums_without_the_memory_for_their_slots(fake):
+    n = 10 ** 6
+    with Handle(fake, n, nmax=4, lmax=2) as h:
+        full = fake.used()
+    with Handle(fake, n, nmax=4, lmax=2, limit=full - 8 * n) as h:
+        assert h.rc == 0 and fake.used() <= full - 8 * n
+        fake.reset()
+        assert h.call("scf_bound", 0x1000, 0x2000, ctypes.c_double(0.5), ctypes.c_double(0.9), None, 0x3000, None, 0x4000) == 0
+        assert [g[2] for g in grid_of(fake, "k_bound_ordered")] == [1]  # one slot
+        assert not [x for x in fake.log() if x.startswith("memset")]
+    with Handle(fake, n, nmax=4, lmax=2, limit=full - 48 * n) as h:
+        assert h.rc == -6  # out of memory
