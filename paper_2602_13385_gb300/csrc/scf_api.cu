@@ -67,7 +67,7 @@ struct scf_handle {
   bool graphs = true;
   cudaGraphExec_t step_exec = nullptr;
   const void* step_key[4] = {nullptr, nullptr, nullptr, nullptr};
-  bool step_split = false;      // the graph is of a split-state step (scf_step_host, below)
+  int step_route = 0;                    // and which passes it runs over (step_route())
   // scf_step_host on mapped host memory (mixed precision, register-tiled
   // kernel 1): device copies of the drifted positions and the half-kicked
   // velocities, so that kernel 3 reads them from device memory; allocated by
@@ -220,7 +220,7 @@ void drop_graph(scf_handle* h) {
   if (h->step_exec) cudaGraphExecDestroy(h->step_exec);
   h->step_exec = nullptr;
   for (auto& k : h->step_key) k = nullptr;
-  h->step_split = false;
+  h->step_route = 0;
 }
 
 size_t round_up(size_t x) { return (x + 255) & ~size_t(255); }
@@ -1252,6 +1252,13 @@ int launch_step(scf_handle* h, void* pos, void* vel, void* acc, double* com, boo
   return rc;
 }
 
+// What a step runs over, as far as calls may differ in it: scf_step_host switches the
+// bins off for itself, so a graph that scf_step captured on the same (page-locked)
+// arrays is not its graph, and the reverse.
+int step_route(const scf_handle* h, bool split) {
+  return 1 | (split ? 2 : 0) | (bins_k1(h) ? 4 : 0) | (bins_k3(h) ? 8 : 0);
+}
+
 // Captures one step on the handle's stream into an executable graph.  Returns
 // false (and leaves the handle without a graph) when the stream cannot be
 // captured, e.g. the legacy default stream.
@@ -1277,7 +1284,7 @@ bool capture_step(scf_handle* h, void* pos, void* vel, void* acc, double* com, b
   h->step_key[1] = vel;
   h->step_key[2] = acc;
   h->step_key[3] = com;
-  h->step_split = split;
+  h->step_route = step_route(h, split);
   return true;
 }
 
@@ -1286,7 +1293,7 @@ int step_impl(scf_handle* h, void* pos, void* vel, void* acc, double* com, int n
   // and their arguments are the same every step); plain launches otherwise
   if (h->graphs && !h->prof_on) {
     const bool same = h->step_exec && h->step_key[0] == pos && h->step_key[1] == vel && h->step_key[2] == acc &&
-                      h->step_key[3] == com && h->step_split == split;
+                      h->step_key[3] == com && h->step_route == step_route(h, split);
     if (same || capture_step(h, pos, vel, acc, com, split)) {
       for (int st = 0; st < nsteps; ++st)
         if (cudaGraphLaunch(h->step_exec, h->stream) != cudaSuccess) return SCF_ERR_CUDA;

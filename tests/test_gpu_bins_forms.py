@@ -1,0 +1,145 @@
+"""Radial bins against the direct kernels of the same handle options (SCF_OPT_RADIAL_BINS 2
+and 0), where a mistake cannot be in both: steps with their kicks and drifts, masks and
+progenitors, every exponent, an adjoint level, and a handle moved between exponents.
+
+Tolerances (derived as in test_gpu_bins.py): a double-precision sum of N terms with
+recurrences of tens of steps, 1e-11; single-precision terms with some tens of roundings of
+6e-8, 5e-6 of the largest value and 2e-5 of a particle's own acceleration (a few of the
+terms of a particle cancel); a state kept in single precision adds its own rounding of
+6e-8 a step to increments.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+from test_gpu_bins import TOL, bi_orthonormal, sample  # noqa: E402
+
+OWN = {"fp64": 1e-11, "mixed": 2e-5}
+
+
+@pytest.fixture(scope="module")
+def scf():
+    import paper_2602_13385_gb300 as m
+    return m
+
+
+def both(scf, cfg, **kw):
+    """(binned, direct) handles."""
+    from paper_2602_13385_gb300 import _lib
+    sims = [scf.SCF(cfg, **kw) for _ in range(2)]
+    for sim, mode in zip(sims, (2, 0)):
+        _lib.scf_set_option(sim._h, _lib.SCF_OPT_RADIAL_BINS, mode)
+    assert [s.launches_per_call("step") > 4 for s in sims] == [True, False]
+    return sims
+
+
+def same_field(got, ref, prec):
+    """Each particle's acceleration on its own scale (a thousandth of the median's at least)."""
+    a, b = got[:, :3].double(), ref[:, :3].double()
+    own = b.norm(dim=1)
+    assert ((a - b).norm(dim=1) / (own + 1e-3 * own.median())).max().item() <= OWN[prec]
+    assert ((got - ref)[:, 3].abs() / ref[:, 3].abs()).max().item() <= OWN[prec]
+
+
+@pytest.mark.parametrize("prec,nmax,lmax,n", [("fp64", 20, 8, 12001), ("fp64", 20, 10, 60013), ("mixed", 20, 10, 70001),
+                                              ("mixed", 20, 10, 420007)])
+@pytest.mark.parametrize("alpha", [0.1, 0.5, 1.0, 2.0, 4.0])
+def test_every_exponent(scf, prec, nmax, lmax, n, alpha):
+    cfg = scf.Config(nmax=nmax, lmax=lmax, b=0.7, precision=prec, alpha=alpha)
+    pos = sample(n, 3, cfg.dtype)
+    pos[n // 2] = pos[n // 2 + 3]            # (the field of alpha > 1 diverges at the centre)
+    pos[n // 2, 1] = 0.01
+    sims = both(scf, cfg, n=n)
+    A = [s.coeffs(pos) for s in sims]
+    a, ref = (bi_orthonormal(x, nmax, lmax, alpha) for x in A)
+    assert ((a - ref).abs().max() / ref.abs().max()).item() <= TOL[prec]
+    acc = [s.forces(pos, A[1]) for s in sims]
+    same_field(*acc, prec)
+    for s in sims:
+        assert s.status() == (0, 0)
+        s.close()
+
+
+@pytest.mark.parametrize("prec,nmax,lmax,offsets", [("fp64", 20, 8, [0, 30001]), ("fp64", 10, 5, [0, 20000, 20000, 20031, 60007]),
+                                                    ("mixed", 20, 10, [0, 70001]), ("mixed", 10, 5, [0, 300001]),
+                                                    ("mixed", 20, 8, [0, 100000, 100000, 100031, 205000])])
+@pytest.mark.parametrize("with_mask", [False, True])
+def test_steps(scf, prec, nmax, lmax, offsets, with_mask):
+    """Displacements, velocity changes and the last field of three steps from a moving state."""
+    n, P, dt = offsets[-1], len(offsets) - 1, 0.05
+    cfg = scf.Config(nmax=nmax, lmax=lmax, b=0.7, dt=dt, precision=prec, host=[(2, 6.6e6, 5000.0, 0.0), (3, 6.8e5, 750.0, 70.0)])
+    pos = sample(n, 7, cfg.dtype)
+    far = pos[:, :3].norm(dim=1) > 20.0
+    pos[far, :3] *= 20.0 / pos[far, :3].norm(dim=1, keepdim=True)
+    vel = (0.5 * torch.randn(n, 4, device="cuda", dtype=torch.float64,
+                             generator=torch.Generator("cuda").manual_seed(2))).to(cfg.dtype)
+    com = torch.tensor([[2000.0 + 50 * p, 100.0, -30.0, 0.0, 40.0, 0.0] for p in range(P)], device="cuda", dtype=torch.float64)
+    mask = (torch.arange(n, device="cuda") % 3 != 0).to(torch.uint8) if with_mask else None
+    out = []
+    for sim in both(scf, cfg, offsets=offsets, b_per_prog=[0.7 + 0.1 * p for p in range(P)]):
+        sim.set_mask(mask)
+        p, v, c = pos.clone(), vel.clone(), com.clone()
+        a = sim.forces(p, sim.coeffs(p, mask=mask), com=c)
+        sim.step(p, v, a, c, nsteps=3)
+        assert sim.status() == (0, 0)
+        out.append(((p - pos)[:, :3].double(), (v - vel)[:, :3].double(), a, c, p, v))
+        sim.close()
+    (dx, dv, a, c, _, _), (dx0, dv0, a0, c0, p0, v0) = out
+    assert torch.equal(c, c0)
+    eps = 0.0 if prec == "fp64" else 3 * 6e-8
+    assert (dx - dx0).abs().max().item() <= TOL[prec] * dx0.abs().max().item() + eps * p0[:, :3].abs().max().item()
+    assert (dv - dv0).abs().max().item() <= TOL[prec] * dv0.abs().max().item() + eps * v0[:, :3].abs().max().item()
+    assert (a - a0)[:, :3].abs().max().item() <= 2 * TOL[prec] * a0[:, :3].abs().max().item()
+
+
+@pytest.mark.parametrize("nmax,lmax,offsets", [(20, 10, [0, 9001]), (10, 5, [0, 16385]), (20, 8, [0, 60013]),
+                                               (20, 10, [0, 20001, 20001, 20050, 43210])])
+def test_adjoint_level(scf, nmax, lmax, offsets):
+    from paper_2602_13385_gb300 import _lib
+    n, P = offsets[-1], len(offsets) - 1
+    g = np.random.default_rng(n + lmax)
+    x = g.normal(size=(n, 3))
+    x *= (np.exp(g.normal(-0.3, 0.9, n)) / np.linalg.norm(x, axis=1))[:, None]
+
+    def dev(a):
+        return torch.tensor(a, dtype=torch.float64, device="cuda")
+    pos = dev(np.concatenate([x, g.uniform(0.5, 1.5, (n, 1)) / n], 1))
+    com = dev(np.concatenate([g.normal(size=(P, 3)) * 3000.0, g.normal(size=(P, 3))], 1))
+    start = [dev(g.normal(size=(n, 4))), dev(g.normal(size=(n, 4))), dev(g.normal(size=(P, 6))), dev(np.zeros((P, 4)))]
+    cfg = scf.Config(nmax=nmax, lmax=lmax, b=0.7, host=[(2, 6.6e6, 5000.0, 0.0), (3, 6.8e5, 750.0, 70.0)])
+    out = []
+    for sim in both(scf, cfg, offsets=offsets):
+        t = [s.clone() for s in start]
+        _lib.scf_adjoint_level(sim._h, pos, com, 0.01, True, *t)
+        assert sim.status() == (0, 0)
+        out.append([a - b for a, b in zip(t, start)])
+        sim.close()
+    for got, ref in zip(*out):
+        assert (got - ref).abs().max().item() <= 1e-11 * ref.abs().max().item() + 1e-15
+
+
+@pytest.mark.parametrize("prec,n", [("fp64", 12001), ("fp64", 60013), ("mixed", 70001)])
+def test_a_handle_moved_between_exponents(scf, prec, n):
+    """scf_retune_alpha over narrow ranges: other bins, past the allocation (direct), and back.
+    Each time the handle is one that was made for the exponent."""
+    nmax, lmax = 20, 8
+    cfg = scf.Config(nmax=nmax, lmax=lmax, b=0.7, precision=prec)
+    pos = sample(n, 9, cfg.dtype)
+    pos[n // 2] = pos[n // 2 + 3]
+    pos[n // 2, 1] = 0.01
+    sim = scf.SCF(cfg, n=n)
+    for lo, hi, binned in ((0.5, 0.51, True), (1.9, 1.95, True), (3.4, 3.5, False), (0.3, 0.31, True), (3.9, 3.95, False),
+                           (1.2, 1.21, True)):
+        al = sim.retune_alpha(pos, alpha_lo=lo, alpha_hi=hi)
+        assert lo * (1 - 1e-12) <= al <= hi * (1 + 1e-12)
+        assert (sim.launches_per_call("step") > 4) == binned, al
+        fresh = scf.SCF(scf.Config(nmax=nmax, lmax=lmax, b=0.7, precision=prec, alpha=al), n=n, b_per_prog=sim.scales().tolist())
+        A, ref = sim.coeffs(pos), fresh.coeffs(pos)
+        a, r = bi_orthonormal(A, nmax, lmax, al), bi_orthonormal(ref, nmax, lmax, al)
+        assert ((a - r).abs().max() / r.abs().max()).item() <= TOL[prec]
+        same_field(sim.forces(pos, ref), fresh.forces(pos, ref), prec)
+        assert sim.status() == (0, 0)
+        fresh.close()
+    sim.close()

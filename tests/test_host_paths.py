@@ -152,3 +152,25 @@ def test_pair_sums_without_the_memory_for_their_slots(fake):
         assert not [x for x in fake.log() if x.startswith("memset")]
     with Handle(fake, n, nmax=4, lmax=2, limit=full - 48 * n) as h:
         assert h.rc == -6  # out of memory
+
+
+@pytest.mark.parametrize("first", ["scf_step", "scf_step_host"])
+def test_a_captured_step_is_replayed_on_its_own_route_only(fake, first):
+    """A mixed host step runs the direct kernels, a step over the same page-locked arrays
+    the bins (here the field alone: one thread per output is chosen for kernel 1)."""
+    arrays = (0x1000, 0x2000, 0x3000)
+    with Handle(fake, 100000, precision="mixed") as h:
+        assert h.call("scf_set_option", 2, 128) == 0
+        fake.host_mapped()
+        calls = {"scf_step": lambda: h.call("scf_step", *arrays, None, 1),
+                 "scf_step_host": lambda: h.call("scf_step_host", None, None, None, None, *arrays, None, 8)}
+        for name in sorted(calls, key=lambda c: c != first) * 2:
+            fake.reset()
+            fake.host_mapped()
+            assert calls[name]() == 0
+            bins = [k for k in fake.launches() if "k_bin" in k or "k_field" in k]
+            assert fake.log().count("capture") == 1
+            assert bool(bins) == (name == "scf_step"), (name, fake.launches())
+        fake.reset()
+        fake.host_mapped()
+        assert calls[name]() == 0 and fake.log().count("capture") == 0  # the same route again: no new capture
