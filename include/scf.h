@@ -203,7 +203,8 @@ int scf_step(scf_handle* h, void* pos, void* vel, void* acc, double* com, int ns
  * owned by the handle (2 records per particle, allocated by the first such
  * call, freed by scf_free), so the host link carries the state in once and out
  * once; over radial bins kernel 3 leaves its results there and they go back by
- * copies.  (In SCF_MIXED the host link bounds such a step and it runs the
+ * copies (a double-precision handle without the memory for it runs the direct
+ * kernels in place).  (In SCF_MIXED the host link bounds such a step and it runs the
  * direct kernels unless SCF_OPT_RADIAL_BINS is 2.)  Otherwise the state is staged through the
  * device arrays: copied in on a second stream of the handle, kernels 1 and 2,
  * then the positions and the centres copied back while kernel 3 runs, which

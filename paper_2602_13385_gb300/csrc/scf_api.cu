@@ -1365,7 +1365,7 @@ int scf_step_host(scf_handle* h, void* pos, void* vel, void* acc, double* com, v
     // mixed precision with the register-tiled kernel 1 and the native kernel
     // 3: the intermediate state stays on the device (launch_step, split)
     // (both precisions over radial bins, whose passes read and write in radial order)
-    const bool split = ((h->cfg.precision == SCF_MIXED && h->k1.variant == 1 && h->k3.variant != 2) ||
+    bool split = ((h->cfg.precision == SCF_MIXED && h->k1.variant == 1 && h->k3.variant != 2) ||
                         (bins_k1(h) && bins_k3(h))) &&
                        h->n_total > 0;
     if (split && !h->d_split) {
@@ -1373,7 +1373,9 @@ int scf_step_host(scf_handle* h, void* pos, void* vel, void* acc, double* com, v
       if (cudaMalloc(&h->d_split, 2 * rec * (size_t)h->n_total) != cudaSuccess) {
         cudaGetLastError();
         h->d_split = nullptr;
-        return SCF_ERR_OUT_OF_MEMORY;
+        if (h->cfg.precision == SCF_MIXED) return SCF_ERR_OUT_OF_MEMORY;
+        split = false;  // in place, as the direct double-precision kernels run it
+        h->bins_off = true;
       }
     }
     if (h->host.n > 0 && !mp[3]) return SCF_ERR_NULL_POINTER;

@@ -18,7 +18,7 @@ std::vector<float> g_elapsed;
 size_t g_used, g_limit, g_elapsed_at;
 std::string g_log;
 struct { dim3 grid, block; size_t smem; cudaStream_t s; } g_call;
-int g_host_mapped, g_capturing;
+int g_host_mapped, g_capturing, g_recording;  // the last: between begin and end of a capture
 
 template <typename... A>
 void note(const char* fmt, A... a) {
@@ -89,7 +89,7 @@ cudaError_t cudaFree(void* p) {
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { note("copy %zu", n); memcpy(d, s, n); return cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t st) {
   note("copy_async %zu %p", n, (void*)st);
-  memcpy(d, s, n);
+  if (!g_recording) memcpy(d, s, n);
   return cudaSuccess;
 }
 cudaError_t cudaMemset(void*, int, size_t n) { note("memset %zu", n); return cudaSuccess; }
@@ -139,8 +139,8 @@ cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* c) {
   *c = g_capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
   return cudaSuccess;
 }
-cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { note("%s", "capture"); return cudaSuccess; }
-cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) { *g = (cudaGraph_t)0x71; return cudaSuccess; }
+cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { note("%s", "capture"); g_recording = 1; return cudaSuccess; }
+cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) { *g = (cudaGraph_t)0x71; g_recording = 0; return cudaSuccess; }
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t, unsigned long long) {
   note("%s", "instantiate");
   *e = (cudaGraphExec_t)0x72;

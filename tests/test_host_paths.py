@@ -174,3 +174,15 @@ def test_a_captured_step_is_replayed_on_its_own_route_only(fake, first):
         fake.reset()
         fake.host_mapped()
         assert calls[name]() == 0 and fake.log().count("capture") == 0  # the same route again: no new capture
+
+
+def test_host_step_without_the_memory_for_its_device_copy(fake):
+    n, arrays = 60000, (0x1000, 0x2000, 0x3000)
+    with Handle(fake, n) as h:
+        assert h.binned()
+        for limit, binned in ((fake.used() + 1000, False), (0, True)):
+            fake.reset(limit)
+            fake.host_mapped()
+            assert h.call("scf_step_host", None, None, None, None, *arrays, None, 8) == 0
+            assert bool([k for k in fake.launches() if "k_bin" in k]) == binned
+            assert h.binned()
