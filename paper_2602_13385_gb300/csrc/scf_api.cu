@@ -1040,7 +1040,8 @@ int scf_init(const scf_config* cfg, int n_prog, const int64_t* offsets, const do
   h->cap_blk3 = make_map3(h->offsets, n_prog, 32).prog.size();  // smallest kernel 3 tile (64 threads, split)
   if (h->cap_blk1 == 0 && h->n_total > 0) return fail(SCF_ERR_UNSUPPORTED);
 
-  // the radial bins' own allocation, then one for the rest of the workspace
+  // the radial bins' own allocation, then one for the rest of the workspace: what is not
+  // needed for a handle to run gives way where memory is short
   rc = bin_init(h);
   if (rc != SCF_OK) return fail(rc);
   const size_t nb1 = std::max<size_t>(1, h->cap_blk1), nb3 = std::max<size_t>(1, h->cap_blk3);
@@ -1083,16 +1084,24 @@ int scf_init(const scf_config* cfg, int n_prog, const int64_t* offsets, const do
   const size_t o_tidf = take(sizeof(float) * SCF_HOST_CAP * SCF_TIDAL_W * (size_t)n_prog);
   const size_t o_tidn = take(sizeof(float) * SCF_HOST_CAP * SCF_TIDAL_W * (size_t)n_prog);
   const size_t slot = sizeof(double) * (size_t)h->n_total, o_bpart = off;  // the pair sums come last
-  if (cudaMalloc(&h->d_base, o_bpart + round_up(slot * h->bound.slots)) != cudaSuccess) {
-    // without the memory for their slots the pair sums run over ordered pairs in one
+  auto reserve = [&] {
+    if (cudaMalloc(&h->d_base, o_bpart + round_up(slot * h->bound.slots)) == cudaSuccess) return true;
     cudaGetLastError();
+    h->d_base = nullptr;
+    return false;
+  };
+  bool got = reserve();
+  if (!got) {  // without the memory for their slots the pair sums run over ordered pairs in one
     h->bound.ordered = true;
     h->bound.slots = 1;
-    if (cudaMalloc(&h->d_base, o_bpart + round_up(slot)) != cudaSuccess) {
-      cudaGetLastError();
-      return fail(SCF_ERR_OUT_OF_MEMORY);
-    }
+    got = reserve();
   }
+  if (!got && h->d_bin_base) {  // and without the bins' the direct kernels run
+    cudaFree(h->d_bin_base);
+    h->d_bin_base = nullptr;
+    got = reserve();
+  }
+  if (!got) return fail(SCF_ERR_OUT_OF_MEMORY);
   char* base = static_cast<char*>(h->d_base);
   h->d_partials = reinterpret_cast<double*>(base + o_part);
   h->d_A = reinterpret_cast<double*>(base + o_A);

@@ -186,3 +186,24 @@ def test_host_step_without_the_memory_for_its_device_copy(fake):
             assert h.call("scf_step_host", None, None, None, None, *arrays, None, 8) == 0
             assert bool([k for k in fake.launches() if "k_bin" in k]) == binned
             assert h.binned()
+
+
+@pytest.mark.parametrize("precision,n", [("fp64", 100000), ("mixed", 200000)])
+def test_bins_give_way_to_the_workspace_that_a_handle_needs(fake, precision, n):
+    with Handle(fake, n, precision=precision) as h:
+        mallocs = [int(x.split()[1]) for x in fake.log() if x.startswith("malloc")]
+        assert h.binned() and len(mallocs) == 2
+    least = mallocs[1] - 8 * n * (mallocs[1] // (8 * n))  # at least this much without the pair sums
+    ran = []
+    for limit in range(sum(mallocs), least, -max(1, sum(mallocs) // 60)):
+        with Handle(fake, n, precision=precision, limit=limit) as h:
+            ran.append((h.rc, h.rc == 0 and h.binned()))
+            if h.rc == 0:
+                fake.reset()
+                assert h.call("scf_step", 0x1000, 0x2000, 0x3000, None, 1) == 0
+                assert bool([k for k in fake.launches() if "k_bin" in k]) == h.binned()
+        assert fake.used() == 0
+    kinds = [r for i, r in enumerate(ran) if i == 0 or r != ran[i - 1]]
+    # with bins, then without, and only a handle that has no room for one slot is refused
+    assert kinds in ([(0, True), (0, False), (-6, False)], [(0, True), (0, False)]), kinds
+    assert ran.count((0, False)) * (sum(mallocs) // 60) > mallocs[0] * 0.8
