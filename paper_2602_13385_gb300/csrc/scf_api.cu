@@ -828,7 +828,7 @@ bool bin_tables(scf_handle* h) {
   if (!h->d_bin_base || !choose_bins(h, &large)) return false;
   const scf_config& c = h->cfg;
   ScfBinShape s = bin_shape(c, c.alpha, large);
-  if (s.K > h->bin_kcap) return false;
+  if (s.K > h->bin_kcap || s.K > kBinMaxK) return false;
   s.chunk = h->bin.chunk;
   s.groups = h->bin.groups;
   s.task = h->bin.task;
@@ -946,6 +946,9 @@ int bin_init(scf_handle* h) {
   h->d_field_rows = base + o_P;
   at(h->d_bin_t, o_t), at(h->d_bin_tf, o_tf), at(h->d_bin_t2, o_t2), at(h->d_bin_aux, o_aux);
   h->bin = s;
+  if (scf_bin_sort_prepare(f32, s) != cudaSuccess || scf_moments_prepare(f32, s) != cudaSuccess ||
+      (!f32 && scf_moments_dual_prepare(s) != cudaSuccess))
+    return SCF_ERR_CUDA;
   h->bin_blocks = (int)nsb;
   h->bin_mblocks = (int)mb_prog.size();
   h->bin_fblocks = (int)nfb;

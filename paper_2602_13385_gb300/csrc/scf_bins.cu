@@ -637,17 +637,26 @@ cudaError_t scf_bin_table_launch(const BinTableArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// What every handle may launch with, set once a handle to the same value: the limit
+// belongs to the kernel, and a launch must not find it lowered for another handle.
+template <typename T, int J>
+static cudaError_t sort_prepare() {
+  return cudaFuncSetAttribute(k_bin_count<T, J>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)(sizeof(unsigned short) * kBinWarps * kBinMaxK));
+}
+
 template <typename T, int J>
 static cudaError_t sort_t(const BinArgs& a, cudaStream_t s) {
-  const size_t sm = sizeof(unsigned short) * (size_t)kBinWarps * a.K;
-  if (sm > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(k_bin_count<T, J>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-  }
-  k_bin_count<T, J><<<a.n_blocks, kBinSortThreads, sm, s>>>(a);
+  k_bin_count<T, J><<<a.n_blocks, kBinSortThreads, sizeof(unsigned short) * kBinWarps * a.K, s>>>(a);
   k_bin_scan<<<dim3((a.K + kScanX - 1) / kScanX, a.n_prog), kScanX * kScanY, 0, s>>>(a);
   k_bin_scatter<T, J><<<a.n_blocks, kBinSortThreads, sizeof(unsigned) * a.K, s>>>(a);
   return cudaGetLastError();
+}
+
+cudaError_t scf_bin_sort_prepare(int f32, const ScfBinShape& sh) {
+  const int J = sh.chunk / kBinSortThreads;
+  if (f32) return J == 1 ? sort_prepare<float, 1>() : J == 2 ? sort_prepare<float, 2>() : sort_prepare<float, 4>();
+  return J == 1 ? sort_prepare<double, 1>() : J == 2 ? sort_prepare<double, 2>() : sort_prepare<double, 4>();
 }
 
 cudaError_t scf_bin_sort_launch(const BinArgs& a, cudaStream_t s) {

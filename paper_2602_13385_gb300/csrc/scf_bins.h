@@ -24,6 +24,7 @@
 
 constexpr int kBinSortThreads = 512;
 constexpr int kBinWarps = kBinSortThreads / 32;
+constexpr int kBinMaxK = 7168;         // bins that the sort's per-warp counts have room for (224 KB)
 constexpr int kBinFieldThreads = 128;  // field block, single precision
 constexpr int kBinFieldTask = 256;     // and its particles, all of one bin, at most
 
@@ -104,6 +105,10 @@ struct BinArgs {
   int2* skey;              // [N] (particle, bin) (masked mass in w)
   int count_status;        // flag non-finite particles (the coefficient pass)
 };
+// The shared memory that a handle's sort and moment kernels may take (once, before the first launch).
+cudaError_t scf_bin_sort_prepare(int f32, const ScfBinShape& sh);
+cudaError_t scf_moments_prepare(int f32, const ScfBinShape& sh);
+cudaError_t scf_moments_dual_prepare(const ScfBinShape& sh);
 cudaError_t scf_bin_sort_launch(const BinArgs& a, cudaStream_t s);
 
 struct MomentArgs {

@@ -344,22 +344,21 @@ __global__ void __launch_bounds__(32) k_moments_dual(MomentDualArgs a) {
 }
 
 template <int L, int NT>
-cudaError_t moments(const MomentDualArgs& a, int blocks, cudaStream_t s) {
+cudaError_t moments(const MomentDualArgs* a, int blocks, cudaStream_t s) {
   constexpr size_t sm = dual_smem<L, NT>();
-  const cudaError_t e = cudaFuncSetAttribute(k_moments_dual<L, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e != cudaSuccess) return e;
-  k_moments_dual<L, NT><<<blocks, 32, sm, s>>>(a);
+  if (!a) return cudaFuncSetAttribute(k_moments_dual<L, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  k_moments_dual<L, NT><<<blocks, 32, sm, s>>>(*a);
   return cudaGetLastError();
 }
 
 template <int L, int NT>
-cudaError_t field(const BinFieldArgs& a, int blocks, cudaStream_t s) {
-  k_field_dual<L, NT><<<blocks, kBinField64Threads, 0, s>>>(a);
+cudaError_t field(const BinFieldArgs* a, int blocks, cudaStream_t s) {
+  k_field_dual<L, NT><<<blocks, kBinField64Threads, 0, s>>>(*a);
   return cudaGetLastError();
 }
 
 template <int NT, typename A>
-cudaError_t by_degree(int L, const A& a, int blocks, cudaStream_t s) {
+cudaError_t by_degree(int L, const A* a, int blocks, cudaStream_t s) {
   auto run = [&](auto deg) -> cudaError_t {
     constexpr int D = decltype(deg)::value;
     if constexpr (std::is_same<A, BinFieldArgs>::value) return field<D, NT>(a, blocks, s);
@@ -378,10 +377,15 @@ cudaError_t by_degree(int L, const A& a, int blocks, cudaStream_t s) {
 
 }  // namespace
 
+cudaError_t scf_moments_dual_prepare(const ScfBinShape& sh) {
+  const MomentDualArgs* none = nullptr;
+  return sh.T == 8 ? by_degree<8>(sh.L, none, 0, nullptr) : by_degree<10>(sh.L, none, 0, nullptr);
+}
+
 cudaError_t scf_moments_dual_launch(const ScfBinShape& sh, const MomentDualArgs& a, int blocks, cudaStream_t s) {
-  return sh.T == 8 ? by_degree<8>(sh.L, a, blocks, s) : by_degree<10>(sh.L, a, blocks, s);
+  return sh.T == 8 ? by_degree<8>(sh.L, &a, blocks, s) : by_degree<10>(sh.L, &a, blocks, s);
 }
 
 cudaError_t scf_bin_field_dual_launch(const ScfBinShape& sh, const BinFieldArgs& a, int blocks, cudaStream_t s) {
-  return sh.T == 8 ? by_degree<8>(sh.L, a, blocks, s) : by_degree<10>(sh.L, a, blocks, s);
+  return sh.T == 8 ? by_degree<8>(sh.L, &a, blocks, s) : by_degree<10>(sh.L, &a, blocks, s);
 }

@@ -261,17 +261,16 @@ __global__ void __launch_bounds__(32 * warps_of(sizeof(T) == 4), 3) k_moments(Mo
 }
 
 template <typename T, int L, int NT>
-cudaError_t launch(const MomentArgs& a, int blocks, cudaStream_t s) {
+cudaError_t launch(const MomentArgs* a, int blocks, cudaStream_t s) {
   constexpr int W = warps_of(sizeof(T) == 4);
-  const size_t sm = sizeof(T) * W * warp_elems<T, L, NT>();
-  const cudaError_t e = cudaFuncSetAttribute(k_moments<T, L, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e != cudaSuccess) return e;
-  k_moments<T, L, NT><<<blocks, 32 * W, sm, s>>>(a);
+  constexpr size_t sm = sizeof(T) * W * warp_elems<T, L, NT>();
+  if (!a) return cudaFuncSetAttribute(k_moments<T, L, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  k_moments<T, L, NT><<<blocks, 32 * W, sm, s>>>(*a);
   return cudaGetLastError();
 }
 
 template <typename T, int NT>
-cudaError_t by_degree(int L, const MomentArgs& a, int blocks, cudaStream_t s) {
+cudaError_t by_degree(int L, const MomentArgs* a, int blocks, cudaStream_t s) {
   switch (L) {
     case 4: return launch<T, 4, NT>(a, blocks, s);
     case 5: return launch<T, 5, NT>(a, blocks, s);
@@ -283,9 +282,16 @@ cudaError_t by_degree(int L, const MomentArgs& a, int blocks, cudaStream_t s) {
   }
 }
 
-}  // namespace
-
-cudaError_t scf_moments_launch(int f32, const ScfBinShape& sh, const MomentArgs& a, int blocks, cudaStream_t s) {
+// The shape's kernel: launched, or (no arguments) given its shared memory.
+cudaError_t by_shape(int f32, const ScfBinShape& sh, const MomentArgs* a, int blocks, cudaStream_t s) {
   if (f32) return sh.T == 6 ? by_degree<float, 6>(sh.L, a, blocks, s) : by_degree<float, 8>(sh.L, a, blocks, s);
   return sh.T == 8 ? by_degree<double, 8>(sh.L, a, blocks, s) : by_degree<double, 10>(sh.L, a, blocks, s);
+}
+
+}  // namespace
+
+cudaError_t scf_moments_prepare(int f32, const ScfBinShape& sh) { return by_shape(f32, sh, nullptr, 0, nullptr); }
+
+cudaError_t scf_moments_launch(int f32, const ScfBinShape& sh, const MomentArgs& a, int blocks, cudaStream_t s) {
+  return by_shape(f32, sh, &a, blocks, s);
 }

@@ -207,3 +207,20 @@ def test_bins_give_way_to_the_workspace_that_a_handle_needs(fake, precision, n):
     # with bins, then without, and only a handle that has no room for one slot is refused
     assert kinds in ([(0, True), (0, False), (-6, False)], [(0, True), (0, False)]), kinds
     assert ran.count((0, False)) * (sum(mallocs) // 60) > mallocs[0] * 0.8
+
+
+def test_shared_memory_limits_are_set_once_to_the_same_value(fake):
+    """A kernel's limit is not the handle's: set at the first need to what any handle may
+    take, so no handle lowers it between another's set and launch, nor under its graph."""
+    with Handle(fake, 60000, nmax=20, lmax=10) as a:
+        first = [x for x in fake.log() if x.startswith("attribute") and "k_bin_count" in x]
+        with Handle(fake, 60000, nmax=40, lmax=12, alpha=4.0) as b:  # many more bins
+            limits = first + [x for x in fake.log() if x.startswith("attribute") and "k_bin_count" in x]
+            assert len(set(limits)) == 1 and len(limits) == 2
+            for h in (a, b):
+                fake.reset()
+                assert h.binned() and h.call("scf_step", 0x1000, 0x2000, 0x3000, None, 1) == 0
+                assert h.call("scf_adjoint_level", 0x1000, None, ctypes.c_double(0.01), 1, 0x2000, 0x3000, None, None) in (0, -4)
+                assert not [x for x in fake.log() if x.startswith("attribute") and ("k_bin" in x or "k_moments" in x)]
+                smem = [int(x.split()[6]) for x in fake.log() if x.startswith("launch") and "k_bin_count" in x]
+                assert smem and max(smem) <= int(limits[0].split()[-1])
