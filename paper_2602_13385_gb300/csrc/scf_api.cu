@@ -1564,6 +1564,16 @@ int scf_autotune(scf_handle* h, const void* pos, const double* com, void* acc, i
       tp_best = k1_candidates[i];
     }
   }
+  // a tile of the one-thread-per-output kernel keeps a mixed handle's coefficients off the
+  // bins (bins_k1): only where it beats them too
+  if (rc == SCF_OK && tp_best != 0 && h->cfg.precision == SCF_MIXED && h->binned && h->bins_mode != 0 &&
+      use_k1(h, 0) == SCF_OK) {
+    double ms = 0.0;
+    h->bins_off = false;
+    rc = time_it([&] { return run_coeffs(h, p, nullptr, nullptr, nullptr, h->d_A, nullptr, SCF_MODE_COEFFS); }, &ms);
+    h->bins_off = true;
+    if (rc == SCF_OK && ms < best1) tp_best = 0;
+  }
   if (rc == SCF_OK) rc = use_k1(h, tp_best);
   if (rc == SCF_OK) rc = run_coeffs(h, p, nullptr, nullptr, nullptr, h->d_A, nullptr, SCF_MODE_COEFFS);
   if (rc == SCF_OK) rc = run_prep(h, h->d_A, com);

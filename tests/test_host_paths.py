@@ -224,3 +224,22 @@ def test_shared_memory_limits_are_set_once_to_the_same_value(fake):
                 assert not [x for x in fake.log() if x.startswith("attribute") and ("k_bin" in x or "k_moments" in x)]
                 smem = [int(x.split()[6]) for x in fake.log() if x.startswith("launch") and "k_bin_count" in x]
                 assert smem and max(smem) <= int(limits[0].split()[-1])
+
+
+@pytest.mark.parametrize("precision,n,ms,tile", [
+    ("mixed", 300000, [0.2, 0.5, 0.5, 0.4, 0.1], 0),     # one thread per output beats the direct kernels, the bins beat it
+    ("mixed", 300000, [0.2, 0.5, 0.5, 0.4, 0.3], 64),
+    ("mixed", 300000, [0.5, 0.5, 0.5, 0.4], 0),
+    ("mixed", 3000, [0.5, 0.2, 0.5, 0.4], 128),          # no bins
+    ("fp64", 30000, [0.5, 0.5, 0.2], 256)])              # any tile leaves them on
+def test_autotuning_does_not_drop_the_bins(fake, precision, n, ms, tile):
+    with Handle(fake, n, precision=precision) as h:
+        was = h.binned()
+        fake.reset()
+        fake.elapsed(ms)
+        assert h.call("scf_autotune", 0x1000, None, 0x2000, 1, None) == 0
+        got = ctypes.c_int()
+        assert h.call("scf_get_option", 2, ctypes.byref(got)) == 0 and got.value == tile
+        fake.reset()
+        assert h.call("scf_step", 0x1000, 0x2000, 0x3000, None, 1) == 0
+        assert bool([k for k in fake.launches() if "k_moments" in k]) == (was and tile != 64)
