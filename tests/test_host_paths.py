@@ -243,3 +243,17 @@ def test_autotuning_does_not_drop_the_bins(fake, precision, n, ms, tile):
         fake.reset()
         assert h.call("scf_step", 0x1000, 0x2000, 0x3000, None, 1) == 0
         assert bool([k for k in fake.launches() if "k_moments" in k]) == (was and tile != 64)
+
+
+@pytest.mark.parametrize("precision,n", [("mixed", 300000), ("fp64", 20000), ("mixed", 2000)])
+def test_a_step_on_new_arrays_updates_the_graph(fake, precision, n):
+    with Handle(fake, n, precision=precision) as h:
+        fake.reset()
+        for k in (1, 2, 3):
+            assert h.call("scf_step", 0x1000 * k, 0x10000 * k, 0x100000 * k, None, 1) == 0
+        log = fake.log()
+        assert [log.count(x) for x in ("capture", "instantiate", "update", f"graph_launch {hex(STREAM)}")] == [3, 1, 2, 3]
+        assert h.call("scf_set_option", 3, 64) == 0  # another shape: another graph
+        fake.reset()
+        assert h.call("scf_step", 0x1000, 0x2000, 0x3000, None, 1) == 0
+        assert fake.log().count("instantiate") == 1 and fake.log().count("update") == 0
