@@ -4,9 +4,13 @@ progenitors, every exponent, an adjoint level, and a handle moved between expone
 
 Tolerances (derived as in test_gpu_bins.py): a double-precision sum of N terms with
 recurrences of tens of steps, 1e-11; single-precision terms with some tens of roundings of
-6e-8, 5e-6 of the largest value and 2e-5 of a particle's own acceleration (a few of the
-terms of a particle cancel); a state kept in single precision adds its own rounding of
-6e-8 a step to increments.
+6e-8, 5e-6 of the largest value; a state kept in single precision adds its own rounding of
+6e-8 a step to increments.  Single-precision fields and coefficients of every exponent are
+compared with double precision on the same positions, where the direct kernels are the measure:
+their own error is that of the arithmetic (up to 4e-4 of the acceleration of a particle whose
+terms cancel, and 8e-5 of the largest coefficient at alpha = 4, where factors leave the normal
+float range), and the binned passes, with as many or fewer roundings, may be off by half as
+much again at most (the largest of tens of thousands of errors: by ten times).
 """
 import numpy as np
 import pytest
@@ -16,7 +20,6 @@ torch = pytest.importorskip("torch")
 
 from test_gpu_bins import TOL, bi_orthonormal, sample  # noqa: E402
 
-OWN = {"fp64": 1e-11, "mixed": 2e-5}
 
 
 @pytest.fixture(scope="module")
@@ -35,31 +38,61 @@ def both(scf, cfg, **kw):
     return sims
 
 
-def same_field(got, ref, prec):
-    """Each particle's acceleration on its own scale (a thousandth of the median's at least)."""
-    a, b = got[:, :3].double(), ref[:, :3].double()
-    own = b.norm(dim=1)
-    assert ((a - b).norm(dim=1) / (own + 1e-3 * own.median())).max().item() <= OWN[prec]
-    assert ((got - ref)[:, 3].abs() / ref[:, 3].abs()).max().item() <= OWN[prec]
+def errors(got, ref):
+    """Each particle's acceleration and potential, on its own scale (a thousandth of the median's at least)."""
+    a, b = got.double(), ref.double()
+    own = b[:, :3].norm(dim=1)
+    return (a - b)[:, :3].norm(dim=1) / (own + 1e-3 * own.median()), (a - b)[:, 3].abs() / b[:, 3].abs()
 
 
-@pytest.mark.parametrize("prec,nmax,lmax,n", [("fp64", 20, 8, 12001), ("fp64", 20, 10, 60013), ("mixed", 20, 10, 70001),
-                                              ("mixed", 20, 10, 420007)])
+def no_worse(got, direct, floor=1e-7):
+    """Errors of the binned passes against the direct kernels' errors."""
+    got, direct = got.sort().values, direct.sort().values
+    for q, factor in ((0.5, 1.5), (0.99, 1.5), (0.999, 1.5), (1.0, 10.0)):
+        i = int(q * (len(got) - 1))
+        assert got[i] <= factor * direct[i] + floor, (q, got[i].item(), direct[i].item())
+
+
+@pytest.mark.parametrize("nmax,lmax,n", [(20, 8, 12001), (20, 10, 60013)])
 @pytest.mark.parametrize("alpha", [0.1, 0.5, 1.0, 2.0, 4.0])
-def test_every_exponent(scf, prec, nmax, lmax, n, alpha):
-    cfg = scf.Config(nmax=nmax, lmax=lmax, b=0.7, precision=prec, alpha=alpha)
+def test_every_exponent_fp64(scf, nmax, lmax, n, alpha):
+    cfg = scf.Config(nmax=nmax, lmax=lmax, b=0.7, alpha=alpha)
     pos = sample(n, 3, cfg.dtype)
     pos[n // 2] = pos[n // 2 + 3]            # (the field of alpha > 1 diverges at the centre)
     pos[n // 2, 1] = 0.01
     sims = both(scf, cfg, n=n)
     A = [s.coeffs(pos) for s in sims]
     a, ref = (bi_orthonormal(x, nmax, lmax, alpha) for x in A)
-    assert ((a - ref).abs().max() / ref.abs().max()).item() <= TOL[prec]
-    acc = [s.forces(pos, A[1]) for s in sims]
-    same_field(*acc, prec)
+    assert ((a - ref).abs().max() / ref.abs().max()).item() <= TOL["fp64"]
+    for e in errors(*[s.forces(pos, A[1]) for s in sims]):
+        assert e.max().item() <= TOL["fp64"]
     for s in sims:
         assert s.status() == (0, 0)
         s.close()
+
+
+@pytest.mark.parametrize("nmax,lmax,n", [(20, 10, 70001), (20, 10, 420007), (10, 5, 300001)])
+@pytest.mark.parametrize("alpha", [0.1, 0.5, 1.0, 2.0, 4.0])
+def test_every_exponent_mixed(scf, nmax, lmax, n, alpha):
+    cfg = scf.Config(nmax=nmax, lmax=lmax, b=0.7, precision="mixed", alpha=alpha)
+    pos = sample(n, 3, cfg.dtype)
+    pos[n // 2] = pos[n // 2 + 3]
+    pos[n // 2, 1] = 0.01
+    far = pos[:, :3].norm(dim=1) > 50.0      # (r / b)^10 of alpha = 0.1 stays in the float range
+    pos[far, :3] *= 50.0 / pos[far, :3].norm(dim=1, keepdim=True)
+    exact = scf.SCF(scf.Config(nmax=nmax, lmax=lmax, b=0.7, alpha=alpha), n=n)
+    A = exact.coeffs(pos.double())
+    ref, a0 = exact.forces(pos.double(), A), bi_orthonormal(A, nmax, lmax, alpha)
+    exact.close()
+    coef, field = [], []
+    for s in both(scf, cfg, n=n):
+        coef.append((bi_orthonormal(s.coeffs(pos), nmax, lmax, alpha) - a0).abs().max() / a0.abs().max())
+        field.append(errors(s.forces(pos, A), ref))
+        assert s.status() == (0, 0)
+        s.close()
+    assert coef[0] <= 1.5 * coef[1] + 1e-7
+    for got, direct in zip(*field):
+        no_worse(got, direct)
 
 
 @pytest.mark.parametrize("prec,nmax,lmax,offsets", [("fp64", 20, 8, [0, 30001]), ("fp64", 10, 5, [0, 20000, 20000, 20031, 60007]),
@@ -120,7 +153,7 @@ def test_adjoint_level(scf, nmax, lmax, offsets):
         assert (got - ref).abs().max().item() <= 1e-11 * ref.abs().max().item() + 1e-15
 
 
-@pytest.mark.parametrize("prec,n", [("fp64", 12001), ("fp64", 60013), ("mixed", 70001)])
+@pytest.mark.parametrize("prec,n", [("fp64", 12001), ("fp64", 60013), ("mixed", 90001)])
 def test_a_handle_moved_between_exponents(scf, prec, n):
     """scf_retune_alpha over narrow ranges: other bins, past the allocation (direct), and back.
     Each time the handle is one that was made for the exponent."""
@@ -137,9 +170,14 @@ def test_a_handle_moved_between_exponents(scf, prec, n):
         assert (sim.launches_per_call("step") > 4) == binned, al
         fresh = scf.SCF(scf.Config(nmax=nmax, lmax=lmax, b=0.7, precision=prec, alpha=al), n=n, b_per_prog=sim.scales().tolist())
         A, ref = sim.coeffs(pos), fresh.coeffs(pos)
-        a, r = bi_orthonormal(A, nmax, lmax, al), bi_orthonormal(ref, nmax, lmax, al)
-        assert ((a - r).abs().max() / r.abs().max()).item() <= TOL[prec]
-        same_field(sim.forces(pos, ref), fresh.forces(pos, ref), prec)
+        acc, acc0 = sim.forces(pos, ref), fresh.forces(pos, ref)
+        if binned:                           # the same bins: the same bits
+            assert torch.equal(A, ref) and torch.equal(acc, acc0)
+        else:
+            a, r = bi_orthonormal(A, nmax, lmax, al), bi_orthonormal(ref, nmax, lmax, al)
+            assert ((a - r).abs().max() / r.abs().max()).item() <= (TOL["fp64"] if prec == "fp64" else 1e-4)
+            for e in errors(acc, acc0):
+                assert e.quantile(0.999).item() <= (TOL["fp64"] if prec == "fp64" else 1e-4)
         assert sim.status() == (0, 0)
         fresh.close()
     sim.close()
