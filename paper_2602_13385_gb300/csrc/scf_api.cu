@@ -113,6 +113,7 @@ struct scf_handle {
   int bins_mode = 1;                     // SCF_OPT_RADIAL_BINS
   ScfBinShape bin{};
   int bin_kcap = 0;                      // bins the allocation holds
+  double bin_occupied = 0.0;             // bins of all progenitors, at most one a particle
   int bin_blocks = 0, bin_mblocks = 0, bin_fblocks = 0;  // sorting, moment and field blocks
   void* d_bin_base = nullptr;
   int *d_sb_prog = nullptr, *d_sb_off = nullptr, *d_mb_prog = nullptr, *d_mb_task = nullptr, *d_fb_prog = nullptr,
@@ -348,33 +349,68 @@ K3Args k3_args(scf_handle* h, const void* pos, void* vel, void* acc, const doubl
   return a;
 }
 
-// The radial-bin passes replace the default kernels: register-tiled kernel 1 in
-// mixed precision, the native kernels in double precision.
-bool bins_k1(const scf_handle* h) {
-  return h->binned && !h->bins_off && h->bins_mode != 0 && (h->cfg.precision == SCF_MIXED ? h->k1.variant == 1 : h->k1.variant != 2);
-}
-bool bins_k3(const scf_handle* h) {
-  return h->binned && !h->bins_off && h->bins_mode != 0 && h->k3.variant != 2;
+// The calls that choose between the radial bins and the direct kernels, each by its own
+// rule: a step (coefficients and field of one sort; also a refresh's pair of passes), the
+// coefficients or the field alone, an adjoint level, a step staged through device arrays.
+enum BinCall { kStep, kCoeffs, kField, kAdjoint, kStaged };
+
+// Double precision: what the bins save against what they add, in us.
+//   saved  N (w W - t T (L + 1)^2 + c), W = (nmax + 1)(lmax + 1)^2: the direct sums less the
+//          binned ones (ps a particle; c, and gen for alpha != 1, the powers and the sort)
+//   added  tab K T (L + 1)^2 (nmax + 1 + n0) per progenitor (of its occupied bins): transform,
+//          field rows, partly filled tiles; `fixed` for the chain of launches, less `wait` W
+//          for the latency that the direct kernels of few particles do not hide either
+// Coefficients by least regret over 382 handles of (6..40, 3..12), 1 to 300 progenitors,
+// alpha 1/2 and 1, timed on a GB300 both ways: the slower side is taken at most 1.13 times the
+// faster one for a step (0.2% in the mean), 1.10 for the field, 1.04 for an adjoint level, 1.25
+// for the coefficients.  Direct / bins, us, on both sides of the lines:
+//   step     (20,8) 4738 258/200;  (10,5) ten progenitors 76k 377/442, 149k 764/665;
+//            (9,12) ten 67k 1105/1581, 329k 5085/4731;  (6,3) 84k 228/271, ten 105k 242/388
+//   field    (10,5) 14k 76/80, 27k 110/102;  (20,8) 9291 121/130, 23k 308/156;  (16,7) 7293 94/123
+//   adjoint  (6,3) ten 105k 1133/1282, 43k 644/578;  (9,12) ten 67k 4702/5117, 132k 8717/8077
+//   coeffs   (8,7) thirty 503k 1012/1605;  (9,12) ten 226k 1102/1703;  (20,10) 19k 207/163, ten 325k 2145/1538
+struct BinRule {
+  double w, t, c, gen, tab, n0, fixed, wait;
+};
+bool bins_pay(const scf_handle* h, const BinRule& r) {
+  const double W = (h->cfg.nmax + 1.0) * (h->cfg.lmax + 1.0) * (h->cfg.lmax + 1.0);
+  const double TL = h->bin.T * (h->bin.L + 1.0) * (h->bin.L + 1.0);
+  const double saved = 1e-6 * h->n_total * (r.w * W - r.t * TL + r.c + (h->gen ? r.gen : 0.0));
+  return saved >= 1e-6 * r.tab * TL * (h->cfg.nmax + 1.0 + r.n0) * h->bin_occupied + r.fixed - 1e-3 * r.wait * W;
 }
 
-// The coefficients or the field alone: a step shares one sort and one set of
-// per-progenitor passes between the two, so alone each pays from a larger size.
-// Measured on a GB300, bins against direct (us; P progenitors):
-//   coefficients, mixed   (10,5) 600k 73/73, P = 8 79/72;  (20,10) 200k 70/70, 600k 105/152, P = 8 132/153
-//   coefficients, double  (10,5) 60k 143/131, 200k 274/361;  (20,8) 16k 153/149, 60k 271/360, P = 8 413/355, 140k 610/686
-//   field, mixed          (10,5) 600k 75/58, P = 8 77/58;  (20,10) 200k 69/81, 600k 110/193, P = 8 136/193
-//   field, double         (10,5) 60k 171/240;  (20,8) 12k 134/208, 60k 314/686, P = 8 407/688
-// (what the bins save grows with W above a floor that the sort costs; the field in double precision
-// pays wherever the step does).
-bool bins_alone(const scf_handle* h, bool field) {
-  if (h->bins_mode == 2 || (field && h->cfg.precision == SCF_FP64)) return true;
+// Mixed precision: a step pays wherever choose_bins admits the handle; the coefficients or the field alone
+// from a larger size, since they share nothing.  Bins / direct, us (P progenitors):
+//   coefficients  (10,5) 600k 73/73, P = 8 79/72;  (20,10) 200k 70/70, 600k 105/152, P = 8 132/153
+//   field         (10,5) 600k 75/58, P = 8 77/58;  (20,10) 200k 69/81, 600k 110/193, P = 8 136/193;
+//                 (9,12) 164k 69/61, 411k 104/118
+bool bins_chosen(const scf_handle* h, BinCall call) {
+  if (h->bins_mode == 2 || call == kStaged) return true;
   const double n = (double)h->n_total, P = h->n_prog, W = (h->cfg.nmax + 1.0) * (h->cfg.lmax + 1.0) * (h->cfg.lmax + 1.0);
-  if (W <= 350.0) return false;
-  if (h->cfg.precision == SCF_FP64) return n >= 2000.0 + 14000.0 * (P - 1.0) + 2.0e7 / (W - 280.0);
-  return field ? n >= 30000.0 * P + 1.8e8 / (W - 350.0) : n >= 35000.0 * P + 4.0e8 / W;
+  const double TL = h->bin.T * (h->bin.L + 1.0) * (h->bin.L + 1.0);
+  if (h->cfg.precision == SCF_MIXED) {
+    if (call == kCoeffs) return W > 350.0 && n >= 35000.0 * P + 4.0e8 / W;
+    const double gain = W - std::max(350.0, 0.7 * TL);
+    return call != kField || (gain > 0.0 && n >= 30000.0 * P + 1.8e8 / gain);
+  }
+  if (call == kCoeffs)
+    return W > 350.0 && n >= 2000.0 + 14000.0 * (P - 1.0) + 2.0e7 / (W - 280.0) &&
+           bins_pay(h, {1.81, 1.94, -154.0, -242.0, 2.36, 6.4, 4.9, 15.4});
+  const bool wave = n <= 64.0 * h->n_sm;  // one of the direct kernels' blocks: their time does not depend on n
+  if (call == kField) return wave ? 0.161 * W - 0.223 * TL >= 106.0 : bins_pay(h, {6.43, 2.84, 17.0, 1480.0, 2.21, 16.2, 26.7, 19.9});
+  if (call == kAdjoint) return wave || bins_pay(h, {44.9, 2.97, -793.0, 0.0, 3.27, 215.0, 115.0, 185.0});
+  return bins_pay(h, {8.59, 5.54, -259.0, 591.0, 2.95, 28.9, 0.0, 28.9});
 }
-bool bins_coeffs(const scf_handle* h) { return bins_k1(h) && bins_alone(h, false); }
-bool bins_forces(const scf_handle* h) { return bins_k3(h) && bins_alone(h, true); }
+
+// The radial-bin passes replace the default kernels: register-tiled kernel 1 in
+// mixed precision, the native kernels in double precision.
+bool bins_k1(const scf_handle* h, BinCall call = kStep) {
+  return h->binned && !h->bins_off && h->bins_mode != 0 &&
+         (h->cfg.precision == SCF_MIXED ? h->k1.variant == 1 : h->k1.variant != 2) && bins_chosen(h, call);
+}
+bool bins_k3(const scf_handle* h, BinCall call = kStep) {
+  return h->binned && !h->bins_off && h->bins_mode != 0 && h->k3.variant != 2 && bins_chosen(h, call);
+}
 
 // The state of a step in host memory crosses the link inside the direct
 // kernels; over radial bins the sorted passes wait for all of it.  In single
@@ -479,8 +515,8 @@ int run_binned_k1(scf_handle* h, void* pos, void* vel, const void* acc, const ui
 }
 
 int run_coeffs(scf_handle* h, void* pos, void* vel, const void* acc, const uint8_t* mask, double* A_out, double* com,
-               int mode, void* pos_copy = nullptr, void* vel_out = nullptr, bool alone = false) {
-  const bool binned = alone ? bins_coeffs(h) : bins_k1(h);
+               int mode, void* pos_copy = nullptr, void* vel_out = nullptr, BinCall call = kStep) {
+  const bool binned = bins_k1(h, call);
   if (binned) {
     if (timed(h, 0, [&] {
           return run_binned_k1(h, pos, vel, acc, mask, mode, pos_copy, vel_out) == SCF_OK ? cudaSuccess
@@ -579,11 +615,11 @@ int run_binned_k3(scf_handle* h, void* vel, void* acc, const double* com, int mo
 // Kernel 3 on the handle's F / a_host(R) (from kernel 2 or run_prep).  sorted:
 // run_coeffs has just run on the same positions (its sort serves this pass too).
 int run_forces(scf_handle* h, const void* pos, void* vel, void* acc, const double* com, int mode,
-               const void* vel_in = nullptr, bool sorted = false, bool alone = false) {
+               const void* vel_in = nullptr, bool sorted = false, BinCall call = kStep) {
   if (h->k3_blocks == 0) return SCF_OK;
-  if (alone ? bins_forces(h) : bins_k3(h)) {
+  if (bins_k3(h, call)) {
     return cuda_fail(timed(h, 2, [&] {
-      int rc = sorted && bins_k1(h) ? SCF_OK
+      int rc = sorted && bins_k1(h, call) ? SCF_OK
                                     : run_sort(h, const_cast<void*>(pos), nullptr, nullptr, nullptr, SCF_MODE_COEFFS,
                                                nullptr, nullptr, false);
       if (rc == SCF_OK) rc = run_binned_k3(h, vel, acc, com, mode, vel_in);
@@ -797,7 +833,7 @@ ScfBinShape bin_shape(const scf_config& c, double alpha, bool large) {
   return s;
 }
 
-// Whether a handle's passes run over radial bins, and with which (K, T).  The
+// Whether a handle has radial bins (bins_chosen says which of its calls run over them), and with which (K, T).  The
 // direct kernels cost N W, W = (nmax + 1)(lmax + 1)^2; the bins replace the
 // nmax + 1 terms by T, for a fixed sequence of passes and, per progenitor, the
 // K-sized tables.  Steps measured on a GB300, bins against direct (us):
@@ -821,7 +857,8 @@ bool choose_bins(const scf_handle* h, bool* large) {
 }
 
 // Tables of the handle's exponent; false (direct kernels) when they do not fit
-// the allocation or a value is not finite.
+// the allocation.  (Their values are finite where the direct kernels' tables are, tables_finite:
+// |C_n| is largest at xi = 1, below gscale, its leading coefficient.)
 bool bin_tables(scf_handle* h) {
   bool large = false;
   h->binned = false;
@@ -833,6 +870,8 @@ bool bin_tables(scf_handle* h) {
   s.groups = h->bin.groups;
   s.task = h->bin.task;
   h->bin = s;
+  h->bin_occupied = 0.0;
+  for (int p = 0; p < h->n_prog; ++p) h->bin_occupied += (double)std::min<int64_t>(h->offsets[p + 1] - h->offsets[p], s.K);
   std::unique_ptr<ScfConst> t(new (std::nothrow) ScfConst);
   if (!t) return false;
   scf_make_const(t.get(), c.alpha);
@@ -1181,7 +1220,7 @@ int scf_coeffs(scf_handle* h, const void* pos, const uint8_t* mask, double* A_ou
   if (!h || !A_out || (!pos && h->n_total > 0)) return SCF_ERR_NULL_POINTER;
   if (!aligned16(pos)) return SCF_ERR_MISALIGNED;
   return run_coeffs(h, const_cast<void*>(pos), nullptr, nullptr, mask, A_out, nullptr, SCF_MODE_COEFFS, nullptr,
-                    nullptr, true);
+                    nullptr, kCoeffs);
 }
 
 int scf_forces(scf_handle* h, const void* pos, const double* A, const double* com, void* acc) {
@@ -1190,7 +1229,7 @@ int scf_forces(scf_handle* h, const void* pos, const double* A, const double* co
   if (!aligned16(pos) || !aligned16(acc)) return SCF_ERR_MISALIGNED;
   int rc = run_prep(h, A, com);
   if (rc != SCF_OK) return rc;
-  return run_forces(h, pos, nullptr, acc, com, SCF_MODE_COEFFS, nullptr, false, true);
+  return run_forces(h, pos, nullptr, acc, com, SCF_MODE_COEFFS, nullptr, false, kField);
 }
 
 namespace {
@@ -1426,14 +1465,15 @@ int scf_step_host(scf_handle* h, void* pos, void* vel, void* acc, double* com, v
     if (bytes && !ok(cudaMemcpyAsync(dp[i], hh[i], bytes, cudaMemcpyHostToDevice, cs))) return SCF_ERR_CUDA;
   if (with_com && !ok(cudaMemcpyAsync(com, host_com, com_bytes, cudaMemcpyHostToDevice, cs))) return SCF_ERR_CUDA;
   if (!ok(cudaEventRecord(ev_in, cs)) || !ok(cudaStreamWaitEvent(h->stream, ev_in, 0))) return SCF_ERR_CUDA;
-  int rc = run_coeffs(h, pos, vel, acc, h->step_mask, h->d_A, com, SCF_MODE_STEP);
+  int rc = run_coeffs(h, pos, vel, acc, h->step_mask, h->d_A, com, SCF_MODE_STEP, nullptr, nullptr, kStaged);
   if (rc != SCF_OK) return rc;
   // kernel 2 (already queued) does not touch the positions; kernel 3 only reads them
   if (!ok(cudaEventRecord(ev_out[0], h->stream)) || !ok(cudaStreamWaitEvent(cs, ev_out[0], 0))) return SCF_ERR_CUDA;
   if (bytes && !ok(cudaMemcpyAsync(hh[0], dp[0], bytes, cudaMemcpyDeviceToHost, cs))) return SCF_ERR_CUDA;
   if (with_com && !ok(cudaMemcpyAsync(host_com, com, com_bytes, cudaMemcpyDeviceToHost, cs))) return SCF_ERR_CUDA;
-  // (over radial bins in one piece: a chunk of sorted particles is no range of the arrays)
-  const bool binned = bins_k3(h);
+  // (over radial bins in one piece: a chunk of sorted particles is no range of the arrays; us, pageable arrays,
+  // in one piece over the bins / in eight over the direct kernels: (10,5) 14k 252/648, 300k 1345/2165; (20,8) 200k 1567/3889)
+  const bool binned = bins_k3(h, kStaged);
   const int c3 = binned ? 1 : std::max(1, std::min(chunks, h->k3_blocks));
   for (int c = 0; c < c3 && h->k3_blocks > 0; ++c) {
     int b0, b1;
@@ -1444,7 +1484,7 @@ int scf_step_host(scf_handle* h, void* pos, void* vel, void* acc, double* com, v
     a.blk_begin += b0;
     a.blk_end += b0;
     if (binned) {
-      rc = run_forces(h, pos, vel, acc, com, SCF_MODE_STEP, nullptr, true);
+      rc = run_forces(h, pos, vel, acc, com, SCF_MODE_STEP, nullptr, true, kStaged);
       if (rc != SCF_OK) return rc;
     } else if (timed(h, 2, [&] {
                  return h->k3.variant == 2 ? scf_k3_ff_launch(a, b1 - b0, h->k3, h->stream)
@@ -1621,8 +1661,8 @@ int scf_adjoint_level(scf_handle* h, const void* pos, const double* com, double 
   if (!aligned16(pos) || !aligned16(xbar) || !aligned16(vbar)) return SCF_ERR_MISALIGNED;
   if (!std::isfinite(weight)) return SCF_ERR_INVALID_ARG;
   if (h->n_total == 0) return SCF_OK;
-  // over radial bins as the passes themselves: one sort serves the whole level
-  const bool binned = bins_k1(h) && bins_k3(h);
+  // over radial bins one sort serves the whole level
+  const bool binned = bins_k1(h, kAdjoint) && bins_k3(h, kAdjoint);
   if (!h->adj_ready) {
     int bps = 0;
     if (scf_k1_dual_prepare(h->cfg.lmax, h->cfg.nmax, &h->k1d, &bps) != cudaSuccess || bps < 1 ||
@@ -1642,7 +1682,7 @@ int scf_adjoint_level(scf_handle* h, const void* pos, const double* com, double 
   adj.drift = drift ? 1 : 0;
   adj.part = binned ? h->d_bin_adj_part : h->d_adj_part;
   // 1. coefficients and force coefficients at x_t
-  int rc = run_coeffs(h, p, nullptr, nullptr, nullptr, h->d_A, nullptr, SCF_MODE_COEFFS);
+  int rc = run_coeffs(h, p, nullptr, nullptr, nullptr, h->d_A, nullptr, SCF_MODE_COEFFS, nullptr, nullptr, kAdjoint);
   if (rc != SCF_OK) return rc;
   // 2. own-position term and tidal partials (dual numbers)
   if (binned) {
@@ -2165,8 +2205,8 @@ int scf_launches_per_call(const scf_handle* h, int which) {
   // over radial bins: three sorting passes, moments, transform; field rows, field
   const int k1 = bins_k1(h) ? 5 : h->k1_blocks > 0 ? 1 : 0, k3 = bins_k3(h) ? 2 : h->k3_blocks > 0 ? 1 : 0;
   const int sort = bins_k3(h) ? 3 : 0;
-  if (which == 0) return (bins_coeffs(h) ? 5 : h->k1_blocks > 0 ? 1 : 0) + 1;
-  if (which == 1) return 1 + (bins_forces(h) ? 5 : h->k3_blocks > 0 ? 1 : 0);
+  if (which == 0) return (bins_k1(h, kCoeffs) ? 5 : h->k1_blocks > 0 ? 1 : 0) + 1;
+  if (which == 1) return 1 + (bins_k3(h, kField) ? 5 : h->k3_blocks > 0 ? 1 : 0);
   if (which == 2) return k1 + 1 + (bins_k1(h) ? 0 : sort) + k3;
   return SCF_ERR_INVALID_ARG;
 }

@@ -257,3 +257,31 @@ def test_a_step_on_new_arrays_updates_the_graph(fake, precision, n):
         fake.reset()
         assert h.call("scf_step", 0x1000, 0x2000, 0x3000, None, 1) == 0
         assert fake.log().count("instantiate") == 1 and fake.log().count("update") == 0
+
+
+@pytest.mark.parametrize("nmax,lmax,sizes,calls", [   # calls over the bins: coefficients, field, step, adjoint level
+    (20, 8, [4738], "s a"), (20, 8, [23000], "cfsa"), (20, 10, [1000000], "cfsa"), (10, 5, [26000], "fsa"),
+    (10, 5, [7600] * 10, "fa"), (10, 5, [14900] * 10, "fsa"), (6, 3, [84000], "a"), (6, 3, [10500] * 10, ""),
+    (9, 12, [6700] * 10, "f"), (9, 12, [33000] * 10, "fsa"), (9, 12, [6900] * 64, "f"), (8, 7, [16700] * 30, "fa"),
+    (20, 10, [66000, 0, 5], "cfsa")])
+def test_double_precision_calls_over_the_bins(fake, nmax, lmax, sizes, calls):
+    """Each call where it is the faster one over the bins (rules in scf_api.cu)."""
+    off = [0]
+    for s in sizes:
+        off.append(off[-1] + s)
+    with Handle(fake, 0, nmax=nmax, lmax=lmax, offsets=off) as h:
+        assert h.rc == 0
+        got = ""
+        for name, args in (("scf_coeffs", (0x1000, None, 0x2000)), ("scf_forces", (0x1000, 0x2000, None, 0x3000)),
+                           ("scf_step", (0x1000, 0x2000, 0x3000, None, 1)),
+                           ("scf_adjoint_level", (0x1000, None, ctypes.c_double(0.01), 1, 0x2000, 0x3000, None, None))):
+            fake.reset()
+            assert h.call(name, *args) == 0
+            over = {any(k in x for x in fake.launches()) for k in ("k_bin_count", "k_bin_scatter")}
+            assert len(over) == 1
+            got += name[4] if over.pop() else ""
+        assert got == calls.replace(" ", "")
+        assert h.call("scf_set_option", 7, 2) == 0  # every pass of a handle that has bins
+        fake.reset()
+        assert h.call("scf_step", 0x1000, 0x2000, 0x3000, None, 1) == 0
+        assert any("k_moments" in x for x in fake.launches())
