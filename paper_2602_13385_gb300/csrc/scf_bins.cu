@@ -1,7 +1,6 @@
 // Radial bins (scf_bins.h): the stable counting sort of the particles by bin,
 // the interpolation tables, and the two small contractions between bins and
 // radial orders.
-#include <algorithm>
 #include <cmath>
 #include <type_traits>
 #include <vector>
@@ -315,22 +314,21 @@ __device__ __forceinline__ void pair_fma(float2& acc, float2 a, float2 b) {
 
 // Partial coefficient rows from the moments: block (g, p, z) takes the bins g,
 // g + groups, ... of progenitor p in order.  A bin's moment rows (one per task)
-// are added in a fixed order, four values and several rows in flight a thread,
-// then thread (column, n mod slices) adds t M to its outputs.  Double precision:
-// T (nmax + 1) FP64 FMAs a column and occupied bin, bound by that pipe.  Single
-// precision: the rows by an error-free two-sum and the products and their sums as
-// (high, low) float pairs (an FP64 FMA takes 64 single-precision slots here, a
-// pair term 12), folded into double at the end; two blocks (z) a bin group.
+// are added in order, four values and four rows in flight a thread, then the
+// block's two threads of a column add t M to every other of its radial orders (z
+// splits them further).  Double precision: T (nmax + 1) FP64 FMAs a column and
+// occupied bin, bound by that pipe.  Single precision: the rows by an error-free
+// two-sum and the products and their sums as (high, low) float pairs (an FP64 FMA
+// takes 64 single-precision slots here, a pair term 12), folded into double at the end.
 template <typename T, int NT, int NH>
 __global__ void __maxnreg__(64) k_transform(TransformArgs a) {
-  extern __shared__ double s_m[];  // [slices of rows][NT][colpad], pairs of floats in single precision
+  extern __shared__ double s_m[];  // [NT][colpad], pairs of floats in single precision
   using V = typename std::conditional<sizeof(T) == 8, ScfD4, float4>::type;
   using M = typename std::conditional<sizeof(T) == 8, double, float2>::type;
   M* sm = reinterpret_cast<M*>(s_m);
-  const int p = blockIdx.y, colpad = a.colpad, E = NT * colpad, EV = E / 4;
+  const int p = blockIdx.y, colpad = a.colpad, EV = NT * colpad / 4;
   const int nq = gridDim.z * (blockDim.x / colpad);
   const int col = threadIdx.x % colpad, q = blockIdx.z * (blockDim.x / colpad) + threadIdx.x / colpad;
-  const int slices = max(1, (int)blockDim.x / EV);
   const int lmax = a.lmax, NN = a.nmax + 1;
   int l = 0;
   while ((l + 1) * (l + 1) <= col) ++l;
@@ -344,14 +342,13 @@ __global__ void __maxnreg__(64) k_transform(TransformArgs a) {
     const int r0 = (int)ts[bin], r1 = (int)ts[bin + 1];
     if (r0 == r1) continue;  // the same for the whole block
     __syncthreads();
-    for (int e = threadIdx.x; e < slices * EV; e += blockDim.x) {
-      const int sl = e / EV, ev = e - sl * EV;
+    for (int ev = threadIdx.x; ev < EV; ev += blockDim.x) {
       T hi[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};
-      for (int k = r0 + sl; k < r1; k += 4 * slices) {
+      for (int k = r0; k < r1; k += 4) {
         V v[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          if (k + j * slices < r1) v[j] = rows[(size_t)(k + j * slices) * EV + ev];
+          if (k + j < r1) v[j] = rows[(size_t)(k + j) * EV + ev];
           else v[j].x = v[j].y = v[j].z = v[j].w = 0;
         }
 #pragma unroll
@@ -366,8 +363,8 @@ __global__ void __maxnreg__(64) k_transform(TransformArgs a) {
       }
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        if constexpr (sizeof(T) == 8) sm[(size_t)sl * E + 4 * ev + c] = hi[c];
-        else sm[(size_t)sl * E + 4 * ev + c] = make_float2(hi[c], lo[c]);
+        if constexpr (sizeof(T) == 8) sm[4 * ev + c] = hi[c];
+        else sm[4 * ev + c] = make_float2(hi[c], lo[c]);
       }
     }
     __syncthreads();
@@ -376,15 +373,6 @@ __global__ void __maxnreg__(64) k_transform(TransformArgs a) {
 #pragma unroll
       for (int d = 0; d < NT; ++d) {
         m[d] = sm[d * colpad + col];
-        for (int sl = 1; sl < slices; ++sl) {
-          const M o = sm[(size_t)sl * E + d * colpad + col];
-          if constexpr (sizeof(T) == 8) {
-            m[d] += o;
-          } else {
-            two_sum_add(m[d].x, m[d].y, o.x);
-            m[d].y += o.y;
-          }
-        }
         if constexpr (sizeof(T) == 4) {  // renormalised, as the products need
           const float t = __fadd_rn(m[d].x, m[d].y);
           m[d].y = __fsub_rn(m[d].y, __fsub_rn(t, m[d].x));
@@ -671,12 +659,13 @@ static cudaError_t transform_t(const TransformArgs& a, cudaStream_t s) {
   // so that all blocks are resident at once
   const int z = sizeof(T) == 8 ? 2 : 4;
   const dim3 grid(a.groups, a.n_prog, z);
-  const int threads = 2 * a.colpad, EV = NT * a.colpad / 4, per = (a.nmax + 2 * z) / (2 * z);
-  const size_t sm = sizeof(double) * NT * a.colpad * std::max(1, threads / EV);
+  const int threads = 2 * a.colpad, per = (a.nmax + 2 * z) / (2 * z);
+  constexpr int kMost = sizeof(T) == 8 ? (SCF_NMAX_CAP + 4) / 4 : (SCF_NMAX_CAP + 8) / 8;
+  const size_t sm = sizeof(double) * NT * a.colpad;
   if (per <= 3) k_transform<T, NT, 3><<<grid, threads, sm, s>>>(a);
   else if (per <= 6) k_transform<T, NT, 6><<<grid, threads, sm, s>>>(a);
-  else if (per <= 11) k_transform<T, NT, 11><<<grid, threads, sm, s>>>(a);
-  else k_transform<T, NT, 21><<<grid, threads, sm, s>>>(a);
+  else if constexpr (kMost > 6) k_transform<T, NT, kMost><<<grid, threads, sm, s>>>(a);
+  else return cudaErrorInvalidValue;
   return cudaGetLastError();
 }
 
