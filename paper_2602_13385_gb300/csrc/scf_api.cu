@@ -127,7 +127,7 @@ struct scf_handle {
   double* d_bin_adj_part = nullptr;   // double precision: [bin_fblocks][SCF_ADJ_Q]
   void *d_spos = nullptr, *d_mrows = nullptr, *d_bin_frame = nullptr, *d_field_rows = nullptr;
   int2* d_skey = nullptr;
-  double *d_bin_t = nullptr, *d_bin_aux = nullptr;  // tables; nodes, node-to-monomial matrix and gscale
+  double *d_bin_t = nullptr, *d_bin_aux = nullptr;  // tables; what bin_tables uploads for them
   float* d_bin_tf = nullptr;
   float2* d_bin_t2 = nullptr;
 };
@@ -876,11 +876,12 @@ bool bin_tables(scf_handle* h) {
   if (!t) return false;
   scf_make_const(t.get(), c.alpha);
   const int nd = s.T - 1, nn = c.nmax + 1;
-  std::vector<double> aux(2 * (size_t)nd + 2 * (size_t)nd * nd + (size_t)(c.lmax + 1) * nn);
-  scf_bin_nodes(s.T, aux.data(), aux.data() + 2 * nd);
-  double* gs = aux.data() + 2 * nd + 2 * nd * nd;
+  const size_t o_nodes = 2 * (size_t)s.T * nn, o_vinv = o_nodes + 2 * nd, o_gs = o_vinv + 2 * (size_t)nd * nd;
+  std::vector<double> aux(o_gs + (size_t)(c.lmax + 1) * nn);
+  scf_bin_scale(s.T, c.nmax, aux.data());
+  scf_bin_nodes(s.T, &aux[o_nodes], &aux[o_vinv]);
   for (int l = 0; l <= c.lmax; ++l)
-    for (int n = 0; n < nn; ++n) gs[l * nn + n] = t->gscale[l][n];
+    for (int n = 0; n < nn; ++n) aux[o_gs + l * nn + n] = 1.0 / t->gscale[l][n];
   if (!put(h, h->d_bin_aux, aux.data(), sizeof(double) * aux.size())) return false;
   BinTableArgs a{};
   a.K = s.K;
@@ -889,9 +890,10 @@ bool bin_tables(scf_handle* h) {
   a.lmax = c.lmax;
   a.f32 = c.precision == SCF_MIXED;
   a.alpha = c.alpha;
-  a.nodes = h->d_bin_aux;
-  a.vinv = h->d_bin_aux + 2 * nd;
-  a.gscale = h->d_bin_aux + 2 * nd + 2 * nd * nd;
+  a.scale = h->d_bin_aux;
+  a.nodes = h->d_bin_aux + o_nodes;
+  a.vinv = h->d_bin_aux + o_vinv;
+  a.inv_gscale = h->d_bin_aux + o_gs;
   a.frame = h->d_bin_frame;
   a.t = h->d_bin_t;
   a.tf = h->d_bin_tf;
@@ -964,7 +966,7 @@ int bin_init(scf_handle* h) {
   const size_t o_fr = take(2 * es * K), o_P = take(es * np * K * scf_bin_row(s.L, s.T));
   const size_t o_t = f32 ? off : take(8 * K * nl * nn * s.T), o_tf = f32 ? take(4 * K * nl * nn * s.T) : off,
                o_t2 = f32 ? take(8 * K * nl * nn * s.T) : off;
-  const size_t o_aux = take(8 * (2 * (size_t)s.T * (s.T + 1) + nl * nn));
+  const size_t o_aux = take(8 * (2 * (size_t)s.T * (nn + s.T) + nl * nn));
   if (cudaMalloc(&h->d_bin_base, off) != cudaSuccess) {
     cudaGetLastError();
     h->d_bin_base = nullptr;

@@ -506,6 +506,15 @@ __device__ __forceinline__ DD dd_divd(DD a, double b) {
   const double r = __fma_rn(-q, b, a.h);
   return dd_fast(q, (r + a.l) / b);
 }
+// s += a b, the low parts collected unnormalised.
+__device__ __forceinline__ void dd_acc(DD& s, DD a, DD b) {
+  const double p = __dmul_rn(a.h, b.h);
+  const double e = __fma_rn(a.l, b.h, __fma_rn(a.h, b.l, __fma_rn(a.h, b.h, -p)));
+  const double t = __dadd_rn(s.h, p), bb = __dsub_rn(t, s.h);
+  const double r = __dadd_rn(__dsub_rn(s.h, __dsub_rn(t, bb)), __dsub_rn(p, bb));
+  s.l = __dadd_rn(s.l, __dadd_rn(r, e));
+  s.h = t;
+}
 
 // Bin frames: q_c and inv = 2 / (q range), rounded to the element type so that
 // the tables are exact for the tau that the kernels form.
@@ -520,14 +529,20 @@ __global__ void k_bin_frame(BinTableArgs a) {
 }
 
 // Interpolation polynomials of degree l in a bin: one group of GW lanes per
-// (bin, l).  Lane j < T - 1 runs the Gegenbauer recurrence of dC_n/dxi
-// (2 lambda C_{n-1}^(lambda+1)) at node j, lane T - 1 that of C_n at tau = 0;
+// (bin, l).  Lane j < T - 1 runs the Gegenbauer recurrence of dC_n/dtau
+// (2 lambda dxi/dtau C_{n-1}^(lambda+1)) at node j, lane T - 1 that of C_n at tau = 0;
 // the derivative's node values become monomial coefficients and are integrated.
-template <int GW>
+// Bound by the FP64 pipe: the recurrences carry n! C_n, without a division a step
+// (1 / n! is folded into the last product), and the nodes are symmetric, so even
+// coefficients take the sums of node pairs and odd ones the differences ((20,10),
+// K = 1664: 1251 us with a division a step and full products, 631 with these).
+template <int GW, int T>
 __global__ void __launch_bounds__(32) k_bin_table(BinTableArgs a) {
   extern __shared__ DD s_f[];  // [32 / GW][nmax + 1][GW]
+  constexpr int ND = T - 1, H = ND / 2;
+  static_assert(ND % 2 == 1 && T <= GW, "");
   const int lane = threadIdx.x, g = lane / GW, j = lane % GW;
-  const int NN = a.nmax + 1, T = a.T, ND = T - 1;
+  const int NN = a.nmax + 1;
   const int item = blockIdx.x * (32 / GW) + g;
   const bool on = item < a.K * (a.lmax + 1);
   const int bin = on ? item / (a.lmax + 1) : 0, l = on ? item % (a.lmax + 1) : 0;
@@ -550,14 +565,13 @@ __global__ void __launch_bounds__(32) k_bin_table(BinTableArgs a) {
     if (!value) xi = dd_add(xi, dd_mul(hw, {a.nodes[j], a.nodes[ND + j]}));
     const double al = value ? lam : lam + 1.0;
     DD c1 = {0.0, 0.0}, c0 = value ? DD{1.0, 0.0} : dd_mul({2.0 * lam, 0.0}, hw);
-    // value lane: f[n] = C_n; derivative lanes: f[n] = dC_n/dtau = 2 lambda hw C_{n-1}^(lambda+1)
+    // value lane: f[n] = n! C_n; derivative lanes: f[n] = (n - 1)! dC_n/dtau
     const int shift = value ? 0 : 1;
     if (!value) f[j] = {0.0, 0.0};
     if (shift < NN) f[shift * GW + j] = c0;
     for (int n = 1; n + shift < NN; ++n) {
-      const DD u = dd_muld(dd_mul(xi, c0), 2.0 * (n + al - 1.0));
-      const DD v = dd_muld(c1, -(n + 2.0 * al - 2.0));
-      const DD c = dd_divd(dd_add(u, v), (double)n);
+      const double v = n + 2.0 * al - 2.0, w = -(n - 1.0) * v;
+      const DD c = dd_add(dd_muld(dd_mul(xi, c0), 2.0 * (n + al - 1.0)), dd_mul(c1, {w, __fma_rn(-(n - 1.0), v, -w)}));
       c1 = c0;
       c0 = c;
       f[(n + shift) * GW + j] = c;
@@ -567,22 +581,36 @@ __global__ void __launch_bounds__(32) k_bin_table(BinTableArgs a) {
   if (!on) return;
   for (int n = j; n < NN; n += GW) {
     const size_t at = ((size_t)item * NN + n) * T;
-    const double gs = a.gscale[l * NN + n];
-    auto put = [&](int d, double v) {
+    const double igs = a.inv_gscale[l * NN + n];
+    const double2* scale = reinterpret_cast<const double2*>(a.scale) + n * T;
+    auto put = [&](int d, DD e) {
+      const double2 w = __ldg(scale + d);
+      const double v = dd_mul(e, {w.x, w.y}).h;
       if (a.f32) {
         const float hi = (float)v;
-        a.tf[at + d] = (float)(v / gs);
+        a.tf[at + d] = (float)(v * igs);
         a.t2[at + d] = make_float2(hi, (float)(v - (double)hi));
       } else {
         a.t[at + d] = v;
       }
     };
-    put(0, f[n * GW + ND].h);
+    const DD* fn = f + n * GW;
+    DD sum[H + 1], dif[H];
+#pragma unroll
+    for (int k = 0; k < H; ++k) {
+      const DD u = fn[k], w = fn[ND - 1 - k];
+      sum[k] = dd_add(u, w);
+      dif[k] = dd_add(u, {-w.h, -w.l});
+    }
+    sum[H] = fn[H];
+    put(0, fn[ND]);
+#pragma unroll
     for (int d = 0; d < ND; ++d) {
       DD e = {0.0, 0.0};
-      for (int k = 0; k < ND; ++k)
-        e = dd_add(e, dd_mul({a.vinv[d * ND + k], a.vinv[ND * ND + d * ND + k]}, f[n * GW + k]));
-      put(d + 1, dd_divd(e, (double)(d + 1)).h);
+#pragma unroll
+      for (int k = 0; k < (d % 2 == 0 ? H + 1 : H); ++k)
+        dd_acc(e, {__ldg(a.vinv + d * ND + k), __ldg(a.vinv + ND * ND + d * ND + k)}, d % 2 == 0 ? sum[k] : dif[k]);
+      put(d + 1, e);
     }
   }
 }
@@ -594,8 +622,8 @@ void scf_bin_nodes(int T, double* nodes, double* vinv) {
   const int N = T - 1;
   const LD pi = 3.14159265358979323846264338327950288L;
   std::vector<LD> x(N);
-  for (int j = 0; j < N; ++j) {
-    x[j] = std::cos((2 * j + 1) * pi / (2 * N));
+  for (int j = 0; j < N; ++j) {  // symmetric to the last bit
+    x[j] = 2 * j + 1 == N ? 0.0L : 2 * j + 1 < N ? std::cos((2 * j + 1) * pi / (2 * N)) : -x[N - 1 - j];
     nodes[j] = (double)x[j];
     nodes[N + j] = (double)(x[j] - (LD)nodes[j]);
   }
@@ -616,12 +644,29 @@ void scf_bin_nodes(int T, double* nodes, double* vinv) {
   }
 }
 
+void scf_bin_scale(int T, int nmax, double* scale) {
+  using LD = long double;
+  LD fact = 1.0L, last = 1.0L;  // n!, (n - 1)!
+  for (int n = 0; n <= nmax; ++n) {
+    if (n > 0) {
+      last = fact;
+      fact *= n;
+    }
+    for (int d = 0; d < T; ++d) {
+      const LD v = 1.0L / (d == 0 ? fact : last * d);
+      scale[2 * (n * T + d)] = (double)v;
+      scale[2 * (n * T + d) + 1] = (double)(v - (LD)(double)v);
+    }
+  }
+}
+
 cudaError_t scf_bin_table_launch(const BinTableArgs& a, cudaStream_t s) {
   k_bin_frame<<<(a.K + 127) / 128, 128, 0, s>>>(a);
   const int items = a.K * (a.lmax + 1);
   const size_t sm = 32 * sizeof(DD) * (size_t)(a.nmax + 1);
-  if (a.T <= 8) k_bin_table<8><<<(items + 3) / 4, 32, sm, s>>>(a);
-  else k_bin_table<16><<<(items + 1) / 2, 32, sm, s>>>(a);
+  if (a.T == 6) k_bin_table<8, 6><<<(items + 3) / 4, 32, sm, s>>>(a);
+  else if (a.T == 8) k_bin_table<8, 8><<<(items + 3) / 4, 32, sm, s>>>(a);
+  else k_bin_table<16, 10><<<(items + 1) / 2, 32, sm, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -196,15 +196,17 @@ struct BinTableArgs {
   double alpha;
   const double* vinv;      // device [2][(T-1)][(T-1)]: hi and lo parts of the node-to-monomial matrix
   const double* nodes;     // device [2][T-1]: hi and lo parts of the Chebyshev nodes
-  const double* gscale;    // device [lmax + 1][nmax + 1]
+  const double* scale;     // device [nmax + 1][T] (hi, lo): 1 / n! at d = 0, 1 / ((n - 1)! d) (16-byte aligned)
+  const double* inv_gscale;  // device [lmax + 1][nmax + 1]
   void* frame;             // [K] pairs of the element type
   double* t;               // [K][lmax + 1][nmax + 1][T]
   float* tf;               // single precision: t / gscale
   float2* t2;              // single precision: t as (high, low) floats
 };
 cudaError_t scf_bin_table_launch(const BinTableArgs& a, cudaStream_t s);
-// Host side of it: nodes and node-to-monomial matrix, hi and lo parts.
+// Host side of it: nodes and node-to-monomial matrix, hi and lo parts; scale.
 void scf_bin_nodes(int T, double* nodes, double* vinv);
+void scf_bin_scale(int T, int nmax, double* scale);
 
 cudaError_t scf_upload_const_bins(const ScfBinConst* t);
 cudaError_t scf_upload_const_bin_moments(const ScfBinConst* t);
