@@ -181,3 +181,31 @@ def test_a_handle_moved_between_exponents(scf, prec, n):
         assert sim.status() == (0, 0)
         fresh.close()
     sim.close()
+
+
+def test_evolution_with_retuned_exponents(scf):
+    """scf_evolve with complete refreshes of alpha and b: the step's graph, the tables and the bins of every
+    new exponent.  Fields agree to 1e-11 and thirty short steps amplify little; the exponent is the root of a
+    sum over the particles, found to 1e-8."""
+    nmax, lmax, n = 10, 6, 20011
+    pos0 = sample(n, 5, torch.float64)
+    far = pos0[:, :3].norm(dim=1) > 20.0
+    pos0[far, :3] *= 20.0 / pos0[far, :3].norm(dim=1, keepdim=True)
+    com = torch.tensor([[2000.0, 100.0, -30.0, 0.0, 40.0, 0.0]], device="cuda", dtype=torch.float64)
+    cfg = dict(nmax=nmax, lmax=lmax, b=0.7, dt=0.01, host=[(2, 6.6e6, 5000.0, 0.0), (3, 6.8e5, 750.0, 70.0)])
+    out = []
+    for sim in both(scf, scf.Config(**cfg), n=n):
+        sim.config = scf.Config(**cfg)       # (evolve writes the exponent into it)
+        p, v, c = pos0.clone(), torch.zeros_like(pos0), com.clone()
+        a = sim.forces(p, sim.coeffs(p), com=c)
+        alphas = []
+        for _ in range(3):
+            sim.evolve(p, v, a, c, nsteps=10, max_steps=5, retune_every=1, retune_rule="alpha_a000", alpha_range=(0.5, 1.8))
+            alphas.append(sim.config.alpha)
+        assert sim.status() == (0, 0)
+        out.append((alphas, sim.scales(), (p - pos0)[:, :3], v[:, :3], a[:, :3], c))
+        sim.close()
+    (al, *got), (al0, *ref) = out
+    assert al[0] != 1.0 and np.allclose(al, al0, rtol=1e-8, atol=0)
+    for x, y in zip(got, ref):
+        assert (x - y).abs().max().item() <= 1e-8 * y.abs().max().item()
