@@ -95,7 +95,7 @@ def per_particle_flops_binned(nmax, lmax, precision, n_per_prog):
     """The same over radial bins: T polynomial terms in place of the nmax + 1
     radial orders (coefficients: T FMAs per angular column; field: value and
     derivative of two polynomials per (l, m >= 1) and one per degree, four pairs
-    of sums)."""
+    of sums).  T as choose_bins (scf_api.cu) takes it."""
     T = (6 if n_per_prog >= 400000 else 8) if precision == "mixed" else (8 if n_per_prog >= 50000 else 10)
     nl = lmax + 1
     nlm = nl * (nl + 1) // 2
@@ -110,10 +110,11 @@ def per_particle_bytes(elem):
     return 5 * rec, 4 * rec      # kernel 1: r pos,vel,acc w pos,vel; kernel 3: r pos,vel w acc,vel
 
 
-# sources that decide the code and launch shapes of the three step kernels
-# the sources of the step kernels' code (kernels 1-3, their device helpers and
-# tables); the launch shapes are fixed by --tiles in the capture command
-STEP_SOURCES = ["scf_coeffs.cu", "scf_device.cuh", "scf_forces.cu", "scf_tables.cu"]
+# the sources of the step kernels' code (kernels 1-3, the passes over radial bins,
+# their device helpers and tables); the launch shapes are fixed by --tiles in the
+# capture command and by the size rules
+STEP_SOURCES = ["scf_bins.cu", "scf_bins.h", "scf_bins_field.cu", "scf_bins_moments.cu", "scf_coeffs.cu",
+                "scf_device.cuh", "scf_forces.cu", "scf_tables.cu"]
 
 
 def src_hash():

@@ -49,12 +49,14 @@
  * word), allocated once in scf_init.  No call allocates after scf_init
  * (scf_step_host's first call excepted, see there).
  *
- * Radial bins.  A handle with enough particles for its (nmax, lmax) runs its
- * coefficient and field passes (alone, from a larger size) over particles sorted by
- * radius, with the radial polynomials of each radius bin replaced by
- * interpolants exact to the precision's rounding (workspace of about 40 to 50 bytes
- * a particle and the bins' tables; without the memory for it the handle keeps
- * the direct kernels).  The block shapes below are those of the direct
+ * Radial bins.  A handle with enough particles for its (nmax, lmax) runs the
+ * calls that are faster so (a rule each: steps, coefficients or field alone,
+ * adjoint levels) over particles sorted by radius, with the radial polynomials
+ * of each radius bin replaced by interpolants exact to the precision's rounding.
+ * The workspace for it grows by about 41 (SCF_MIXED) or 85 bytes a particle on
+ * top of a part by (nmax, lmax) and progenitor, 5 to 35 MB for one ((20,10): in
+ * all 62 MB at N = 1e6 in SCF_MIXED, 165 MB in SCF_FP64; (20,8) SCF_FP64 22 MB at
+ * N = 2e4); without the memory for it the handle keeps the direct kernels.  The block shapes below are those of the direct
  * kernels; selecting a float-float variant, or the one-thread-per-output
  * kernel 1 in SCF_MIXED, selects the direct kernel.
  *
@@ -204,12 +206,15 @@ int scf_step(scf_handle* h, void* pos, void* vel, void* acc, double* com, int ns
  * call, freed by scf_free), so the host link carries the state in once and out
  * once; over radial bins kernel 3 leaves its results there and they go back by
  * copies (a double-precision handle without the memory for it runs the direct
- * kernels in place).  (In SCF_MIXED the host link bounds such a step and it runs the
- * direct kernels unless SCF_OPT_RADIAL_BINS is 2.)  Otherwise the state is staged through the
+ * kernels in place).  (In SCF_MIXED the direct kernels, whose arithmetic runs
+ * while the state crosses the link, are the faster ones and run unless
+ * SCF_OPT_RADIAL_BINS is 2.)  Otherwise the state is staged through the
  * device arrays: copied in on a second stream of the handle, kernels 1 and 2,
  * then the positions and the centres copied back while kernel 3 runs, which
  * is launched in `chunks` pieces of its block map so that each piece's
- * velocities and accelerations go back while the next piece runs.  The copy
+ * velocities and accelerations go back while the next piece runs; over radial
+ * bins (SCF_FP64) it runs in one piece, since sorted particles are no range of
+ * the arrays, and `chunks` has no effect.  The copy
  * stream and its events are created by the first staged call and freed by
  * scf_free; the handle's stream waits for the copies, so a synchronisation of
  * the handle's stream covers the whole call.
@@ -367,7 +372,8 @@ int scf_energy(scf_handle* h, const void* pos, const void* vel, const void* acc,
  * are added in double.  In mixed precision each pair term and blocks of 64
  * of them (128, in sums of four, for the second particle of a pair) are float
  * (1/r the hardware approximation), added in double.  Each unordered pair is
- * evaluated once for both of its particles.  In
+ * evaluated once for both of its particles, or, in samples too small to fill
+ * the GPU so, once for each.  In
  * both, pairs whose r^2 lies outside the normal float range
  * [1.18e-38, 3.40e38] add nothing.
  *   pos, vel   device [N][4] in the handle's element type (16-byte aligned)

@@ -363,7 +363,7 @@ enum BinCall { kStep, kCoeffs, kField, kAdjoint, kStaged };
 // Coefficients by least regret over 382 handles of (6..40, 3..12), 1 to 300 progenitors,
 // alpha 1/2 and 1, timed on a GB300 both ways: the slower side is taken at most 1.13 times the
 // faster one for a step (0.2% in the mean), 1.10 for the field, 1.04 for an adjoint level, 1.25
-// for the coefficients.  Direct / bins, us, on both sides of the lines:
+// for the coefficients (60 further handles near the lines: 1.13, 1.10, 1.00, 1.06).  Direct / bins, us, on both sides of the lines:
 //   step     (20,8) 4738 258/200;  (10,5) ten progenitors 76k 377/442, 149k 764/665;
 //            (9,12) ten 67k 1105/1581, 329k 5085/4731;  (6,3) 84k 228/271, ten 105k 242/388
 //   field    (10,5) 14k 76/80, 27k 110/102;  (20,8) 9291 121/130, 23k 308/156;  (16,7) 7293 94/123
@@ -413,8 +413,9 @@ bool bins_k3(const scf_handle* h, BinCall call = kStep) {
 }
 
 // The state of a step in host memory crosses the link inside the direct
-// kernels; over radial bins the sorted passes wait for all of it.  In single
-// precision the link bounds the step and the direct kernels are faster (us, bins
+// kernels; over radial bins the sorted passes wait for all of it.  48 MB (N = 1e6 in single
+// precision) cross in 230 us, return in 250 and do both at once in 290, so what the
+// link adds to the bins' 234 us in single precision the direct kernels (534 us) hide (us, bins
 // against direct, mapped memory: (10,5) 400k 256/193, 700k 411/316; (20,10) 200k 214/151, 700k 454/428,
 // 1e6 607/599, eight progenitors 700k 554/430); in double precision the bins stay ((20,8) 60k 615/1085).
 bool host_step_direct(const scf_handle* h) { return h->cfg.precision == SCF_MIXED && h->bins_mode != 2; }

@@ -7,9 +7,12 @@
 // degree T - 1 in the bin's coordinate tau = (q_c - q) inv (xi = 1 - 2 q),
 //   C_n^(lambda_l)(xi) = sum_{d < T} t[bin][l][n][d] tau^d,
 // interpolated so that value and derivative agree to rounding (the bin's width
-// in theta is chosen from the fastest oscillation, nmax + lambda_lmax, and T;
-// worst relative derivative error over all bins and n: 6e-9 for the
-// single-precision pairs of (K, T), 3e-17 for the double-precision ones).  So
+// in theta is chosen from the fastest oscillation, nmax + lambda_lmax, and T).
+// Largest error of dC_n/dxi over all bins, l and n, relative to its amplitude there
+// (the envelope of its oscillation), coarser / finer bins: (20,10), alpha = 1, 2.5e-9
+// / 8e-9 for the single-precision pairs of (K, T) and 3.3e-17 / 1.9e-16 for the
+// double-precision ones; over (6..40, 3..12) and alpha from 0.1 to 4 at most 3.3e-8
+// and 5e-16, at nmax = 40 and alpha = 0.1.  So
 //   coefficients  Sh_nlm = sum_bins sum_d t[bin][l][n][d] M[bin][d][lm],
 //                 M = the moments sum_k tau_k^d (m_k s^l q^(2l+1) Pb_lm W_m),
 //   field         sum_n F_nlm C_n = sum_d P[bin][lm][d] tau^d,
