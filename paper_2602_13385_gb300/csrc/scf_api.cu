@@ -21,6 +21,7 @@ struct scf_handle {
   int device = 0;
   cudaStream_t stream = nullptr;
   cudaStream_t setup = nullptr;          // where put, clear and the tables go: stream (see scf_init)
+  std::vector<std::vector<char>> uploads;  // sources of uploads that no call has waited for yet (put)
   int nlm = 0, nc = 0;
   int64_t n_total = 0;
   int n_sm = 0;
@@ -222,6 +223,13 @@ void drop_graph(scf_handle* h) {
   h->step_exec = nullptr;
   for (auto& k : h->step_key) k = nullptr;
   h->step_route = 0;
+}
+
+// Waits for the handle's stream.
+bool settle(scf_handle* h) {
+  if (cudaStreamSynchronize(h->stream) != cudaSuccess) return false;
+  h->uploads.clear();
+  return true;
 }
 
 size_t round_up(size_t x) { return (x + 255) & ~size_t(255); }
@@ -702,10 +710,14 @@ Map3 make_map3(const std::vector<int64_t>& off, int n_prog, int64_t tb) {
 
 // Uploads and clears in the order of the kernels that read them (h->setup): a copy
 // from pageable memory or a memset on the legacy stream may still be under way when
-// the call returns, and a non-blocking stream does not wait for it.  (src is staged
-// before the call returns.)
-bool put(const scf_handle* h, void* dst, const void* src, size_t bytes) {
-  return bytes == 0 || cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, h->setup) == cudaSuccess;
+// the call returns, and a non-blocking stream does not wait for it.  The copy may read
+// its source after the call too, so that stays with the handle until the stream has
+// been waited for (settle), which no upload does by itself.
+bool put(scf_handle* h, void* dst, const void* src, size_t bytes) {
+  if (bytes == 0) return true;
+  const char* p = static_cast<const char*>(src);
+  h->uploads.emplace_back(p, p + bytes);
+  return cudaMemcpyAsync(dst, h->uploads.back().data(), bytes, cudaMemcpyHostToDevice, h->setup) == cudaSuccess;
 }
 bool clear(const scf_handle* h, void* dst, int value, size_t bytes) {
   return bytes == 0 || cudaMemsetAsync(dst, value, bytes, h->setup) == cudaSuccess;
@@ -1213,7 +1225,10 @@ int scf_init(const scf_config* cfg, int n_prog, const int64_t* offsets, const do
   rc = use_k3(h, 128);
   if (rc != SCF_OK) return fail(rc);
   bin_tables(h);
-  if (h->setup != h->stream && cudaStreamSynchronize(h->setup) != cudaSuccess) return fail(SCF_ERR_CUDA);
+  if (h->setup != h->stream) {
+    if (cudaStreamSynchronize(h->setup) != cudaSuccess) return fail(SCF_ERR_CUDA);
+    h->uploads.clear();
+  }
   h->setup = h->stream;
   *out = h;
   return SCF_OK;
@@ -1516,14 +1531,14 @@ int scf_set_option(scf_handle* h, int option, int value) {
   }
   if (option == SCF_OPT_CENTRE_AHEAD) {
     if (value != 0 && value != 1) return SCF_ERR_INVALID_ARG;
-    if (cudaStreamSynchronize(h->stream) != cudaSuccess) return SCF_ERR_CUDA;
+    if (!settle(h)) return SCF_ERR_CUDA;
     h->centre_ahead = value == 1;
     drop_graph(h);
     return SCF_OK;
   }
   if (option == SCF_OPT_RADIAL_BINS) {
     if (value < 0 || value > 2) return SCF_ERR_INVALID_ARG;
-    if (cudaStreamSynchronize(h->stream) != cudaSuccess) return SCF_ERR_CUDA;
+    if (!settle(h)) return SCF_ERR_CUDA;
     h->bins_mode = value;
     drop_graph(h);
     return SCF_OK;
@@ -1531,13 +1546,13 @@ int scf_set_option(scf_handle* h, int option, int value) {
   if (option == SCF_OPT_K1_TILE || option == SCF_OPT_K3_BLOCK) {
     if (value != 64 && value != 128 && value != 256 && !(option == SCF_OPT_K3_BLOCK && value == 320))
       return SCF_ERR_INVALID_ARG;
-    if (cudaStreamSynchronize(h->stream) != cudaSuccess) return SCF_ERR_CUDA;
+    if (!settle(h)) return SCF_ERR_CUDA;
     return option == SCF_OPT_K1_TILE ? use_k1(h, value) : use_k3(h, value);
   }
   if (option == SCF_OPT_K3_VARIANT) {
     if (value != 0 && value != 1) return SCF_ERR_INVALID_ARG;
     if (value == 1 && h->cfg.precision != SCF_FP64) return SCF_ERR_UNSUPPORTED;
-    if (cudaStreamSynchronize(h->stream) != cudaSuccess) return SCF_ERR_CUDA;
+    if (!settle(h)) return SCF_ERR_CUDA;
     const bool old = h->k3_ff;
     h->k3_ff = value == 1;
     const int rc = use_k3(h, h->k3.threads);
@@ -1547,7 +1562,7 @@ int scf_set_option(scf_handle* h, int option, int value) {
   if (option == SCF_OPT_K1_VARIANT) {
     if (value < 0 || value > 2) return SCF_ERR_INVALID_ARG;
     if (value == 2 && h->cfg.precision != SCF_FP64) return SCF_ERR_UNSUPPORTED;
-    if (cudaStreamSynchronize(h->stream) != cudaSuccess) return SCF_ERR_CUDA;
+    if (!settle(h)) return SCF_ERR_CUDA;
     const bool old = h->k1_ff;
     h->k1_ff = value == 2;
     const int rc = use_k1(h, value == 1 ? 0 : 128);
@@ -1595,6 +1610,7 @@ int scf_autotune(scf_handle* h, const void* pos, const double* com, void* acc, i
       if ((rc = work()) != SCF_OK) return rc;
     cudaEventRecord(e1, h->stream);
     if (cudaEventSynchronize(e1) != cudaSuccess) return SCF_ERR_CUDA;
+    h->uploads.clear();
     float t = 0.f;
     cudaEventElapsedTime(&t, e0, e1);
     *ms = t / reps;
@@ -1818,7 +1834,7 @@ int scf_set_mask(scf_handle* h, const uint8_t* mask) {
   if (!h) return SCF_ERR_NULL_POINTER;
   if (mask != h->step_mask) {
     // the captured step holds the old pointer
-    if (cudaStreamSynchronize(h->stream) != cudaSuccess) return SCF_ERR_CUDA;
+    if (!settle(h)) return SCF_ERR_CUDA;
     drop_graph(h);
     h->step_mask = mask;
   }
@@ -1893,7 +1909,7 @@ int scf_evolve(scf_handle* h, void* pos, void* vel, void* acc, double* com, int 
       if (rc != SCF_OK) return rc;
       if (cudaMemcpyAsync(tid.data(), h->d_tid, sizeof(double) * tid.size(), cudaMemcpyDeviceToHost, h->stream) !=
               cudaSuccess ||
-          cudaStreamSynchronize(h->stream) != cudaSuccess)
+          !settle(h))
         return SCF_ERR_CUDA;
       double dmin = HUGE_VAL;
       for (int p = 0; p < h->n_prog; ++p) dmin = std::min(dmin, tid[16 * (size_t)p + 15]);
@@ -1951,7 +1967,7 @@ int scf_recentre(scf_handle* h, void* pos, void* vel, void* acc, double* com, co
   std::vector<double> st(16 * (size_t)h->n_prog);
   if (cudaMemcpyAsync(st.data(), h->d_rc, sizeof(double) * st.size(), cudaMemcpyDeviceToHost, h->stream) !=
           cudaSuccess ||
-      cudaStreamSynchronize(h->stream) != cudaSuccess)
+      !settle(h))
     return SCF_ERR_CUDA;
   for (int p = 0; p < h->n_prog; ++p) {
     const double* s = st.data() + 16 * (size_t)p;
@@ -2023,7 +2039,7 @@ double dln_i00(double al) {
 // normalisation and field-kernel scales rebuilt and uploaded, the general
 // kernels selected for alpha != 1 (default shapes; no float-float variants).
 int set_alpha(scf_handle* h, double alpha) {
-  if (cudaStreamSynchronize(h->stream) != cudaSuccess) return SCF_ERR_CUDA;
+  if (!settle(h)) return SCF_ERR_CUDA;
   const bool gen = alpha != 1.0;
   {
     std::unique_ptr<ScfConst> t(new (std::nothrow) ScfConst);
@@ -2067,7 +2083,7 @@ int scf_retune_alpha(scf_handle* h, const void* pos, const uint8_t* mask, double
   const int P = h->n_prog;
   std::vector<double> b0(P), st(4 * (size_t)P);
   if (cudaMemcpyAsync(b0.data(), h->d_b, sizeof(double) * P, cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
-      cudaStreamSynchronize(h->stream) != cudaSuccess)
+      !settle(h))
     return SCF_ERR_CUDA;
   ScaleArgs a{};
   a.pos = pos;
@@ -2097,7 +2113,7 @@ int scf_retune_alpha(scf_handle* h, const void* pos, const uint8_t* mask, double
     std::vector<double> bt(P), sm(3 * (size_t)P);
     if (cudaMemcpyAsync(bt.data(), d_bt, sizeof(double) * P, cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
         cudaMemcpyAsync(sm.data(), d_sums, sizeof(double) * 3 * P, cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
-        cudaStreamSynchronize(h->stream) != cudaSuccess)
+        !settle(h))
       return SCF_ERR_CUDA;
     double hs = 0.0, ds = 0.0;
     live = 0;
@@ -2197,7 +2213,7 @@ int scf_status(scf_handle* h, int* status) {
   unsigned word = 0;
   if (cudaMemcpyAsync(&word, h->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess)
     return SCF_ERR_CUDA;
-  if (cudaStreamSynchronize(h->stream) != cudaSuccess) return SCF_ERR_CUDA;
+  if (!settle(h)) return SCF_ERR_CUDA;
   if (cudaMemsetAsync(h->d_status, 0, sizeof(unsigned), h->stream) != cudaSuccess) return SCF_ERR_CUDA;
   if (status) *status = (int)word;
   return word ? SCF_ERR_DEVICE_STATUS : SCF_OK;
@@ -2217,7 +2233,7 @@ int scf_launches_per_call(const scf_handle* h, int which) {
 int scf_profile(scf_handle* h, int enable) {
   if (!h) return SCF_ERR_NULL_POINTER;
   if (!enable) {
-    if (cudaStreamSynchronize(h->stream) != cudaSuccess) return SCF_ERR_CUDA;
+    if (!settle(h)) return SCF_ERR_CUDA;
     prof_release(h);
     return SCF_OK;
   }
@@ -2239,7 +2255,7 @@ int scf_profile_read(scf_handle* h, double* ms, int64_t* launches) {
   if (!h) return SCF_ERR_NULL_POINTER;
   double t[3] = {0, 0, 0};
   int64_t n[3] = {0, 0, 0};
-  if (cudaStreamSynchronize(h->stream) != cudaSuccess) return SCF_ERR_CUDA;
+  if (!settle(h)) return SCF_ERR_CUDA;
   for (int i = 0; i < h->prof_used; ++i) {
     float e = 0.f;
     if (cudaEventElapsedTime(&e, h->prof_ev[2 * i], h->prof_ev[2 * i + 1]) != cudaSuccess) return SCF_ERR_CUDA;

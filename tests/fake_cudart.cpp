@@ -15,6 +15,8 @@ namespace {
 std::map<const void*, std::string> g_name;  // kernels by host stub
 std::map<void*, size_t> g_mem;
 std::vector<float> g_elapsed;
+struct Pending { const char* src; std::vector<char> was; cudaStream_t s; };
+std::vector<Pending> g_pending;  // uploads that nothing has waited for
 size_t g_used, g_limit, g_elapsed_at;
 std::string g_log;
 struct { dim3 grid, block; size_t smem; cudaStream_t s; } g_call;
@@ -42,6 +44,14 @@ void fake_reset(size_t limit) {  // bytes that cudaMalloc may hand out at once (
   g_host_mapped = 0;
 }
 const char* fake_log() { return g_log.c_str(); }
+// Uploads under way whose source is no longer what it was at the call (the copy may read it until the stream is waited for).
+int fake_lost_uploads() {
+  int n = 0;
+  for (const Pending& p : g_pending) n += memcmp(p.src, p.was.data(), p.was.size()) != 0;
+  return n;
+}
+void fake_forget_uploads() { g_pending.clear(); }
+int fake_uploads() { return (int)g_pending.size(); }
 size_t fake_used() { return g_used; }
 void fake_elapsed(const float* ms, int n) { g_elapsed.assign(ms, ms + n); g_elapsed_at = 0; }
 void fake_capturing(int on) { g_capturing = on; }
@@ -87,8 +97,9 @@ cudaError_t cudaFree(void* p) {
   return cudaSuccess;
 }
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { note("copy %zu", n); memcpy(d, s, n); return cudaSuccess; }
-cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t st) {
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind k, cudaStream_t st) {
   note("copy_async %zu %p", n, (void*)st);
+  if (k == cudaMemcpyHostToDevice && !g_recording) g_pending.push_back({(const char*)s, {(const char*)s, (const char*)s + n}, st});
   if (!g_recording) memcpy(d, s, n);
   return cudaSuccess;
 }
@@ -120,7 +131,12 @@ cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {
   return cudaSuccess;
 }
 
-cudaError_t cudaStreamSynchronize(cudaStream_t s) { note("synchronize %p", (void*)s); return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t s) {
+  note("synchronize %p", (void*)s);
+  for (size_t i = g_pending.size(); i-- > 0;)
+    if (g_pending[i].s == s) g_pending.erase(g_pending.begin() + i);
+  return cudaSuccess;
+}
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = (cudaStream_t)0x51; return cudaSuccess; }
 cudaError_t cudaStreamCreateWithPriority(cudaStream_t* s, unsigned, int) { *s = (cudaStream_t)0x52; return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
@@ -130,7 +146,7 @@ cudaError_t cudaEventCreate(cudaEvent_t* e) { *e = (cudaEvent_t)0x61; return cud
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { *e = (cudaEvent_t)0x61; return cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventSynchronize(cudaEvent_t) { g_pending.clear(); return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) {
   *ms = g_elapsed_at < g_elapsed.size() ? g_elapsed[g_elapsed_at++] : 1.f;
   return cudaSuccess;

@@ -78,6 +78,22 @@ def test_setup_is_ordered_before_the_kernels_that_read_it(fake, precision, n, al
         assert unordered_uploads(fake.log(), STREAM) == ([], 0)
 
 
+@pytest.mark.parametrize("precision,n,alpha", [("fp64", 5000, 1.0), ("fp64", 5000, 0.5), ("mixed", 2000, 1.0)])
+def test_sources_of_uploads_outlive_them(fake, precision, n, alpha):
+    """A copy from pageable memory may read its source until the stream is waited for."""
+    fake.lib.fake_forget_uploads()
+    with Handle(fake, n, precision=precision, alpha=alpha) as h:
+        assert h.rc == 0 and fake.lib.fake_uploads() > 10 and fake.lib.fake_lost_uploads() == 0
+        assert h.call("scf_set_option", 3, 64 if alpha == 1.0 else 128) == 0
+        assert h.call("scf_set_option", 2, 128) == 0
+        assert fake.lib.fake_lost_uploads() == 0
+        assert h.call("scf_autotune", 0x1000, None, 0x2000, 1, None) == 0
+        assert fake.lib.fake_lost_uploads() == 0
+        h.call("scf_retune_alpha", 0x1000, None, ctypes.c_double(0.5), ctypes.c_double(1.5), None)
+        assert fake.lib.fake_lost_uploads() == 0
+    fake.lib.fake_forget_uploads()
+
+
 def test_setup_stays_out_of_a_capture(fake):
     with Handle(fake, 20000, stream=STREAM):  # the constants are up
         pass
